@@ -339,7 +339,7 @@ template <class Rl> int nls_set(pss_grid *g, const void *a, int where)
 {
     int rc = g->cuda(cudaMemcpyAsync(g->buf[0], a, g->field_bytes(), kind_in(where), g->stream), "set_state copy");
     if (rc) return rc;
-    rc = g->cuda(fft_rows<Rl>(B<Rl>(g, 0), g->nx, g->batch * g->ny, -1, Rl(1), Tw<Rl>(g->twx), g->stream),
+    rc = g->cuda(fft_rows<Rl>(B<Rl>(g, 0), g->nx, g->ny, g->batch, -1, Rl(1), Tw<Rl>(g->twx), g->stream),
                  "set_state row fft");
     if (rc) return rc;
     if (where == PSS_HOST) return g->cuda(cudaStreamSynchronize(g->stream), "set_state sync");
@@ -362,7 +362,7 @@ template <class Rl> int nls_step(pss_grid *g, int64_t n)
     if ((rc = g->pass_end())) return rc;
     for (int64_t i = 0; i < n && e == cudaSuccess; ++i) {
         if ((rc = g->pass_begin(0))) return rc;
-        e = nls_row_pass<Rl>(B<Rl>(g, 0), g->nx, g->batch * g->ny, sdt, Tw<Rl>(g->twx), g->stream);
+        e = nls_row_pass<Rl>(B<Rl>(g, 0), g->nx, g->ny, g->batch, sdt, Tw<Rl>(g->twx), g->stream);
         if ((rc = g->pass_end())) return rc;
         if (e != cudaSuccess) break;
         const bool last = (i + 1 == n);
@@ -379,7 +379,7 @@ template <class Rl> int nls_physical(pss_grid *g)
     int rc = g->cuda(cudaMemcpyAsync(g->buf[1], g->buf[0], g->field_bytes(), cudaMemcpyDeviceToDevice, g->stream),
                      "copy");
     if (rc) return rc;
-    return g->cuda(fft_rows<Rl>(B<Rl>(g, 1), g->nx, g->batch * g->ny, +1, Rl(1.0 / double(g->nx)),
+    return g->cuda(fft_rows<Rl>(B<Rl>(g, 1), g->nx, g->ny, g->batch, +1, Rl(1.0 / double(g->nx)),
                                 Tw<Rl>(g->twx), g->stream),
                    "row inverse");
 }
@@ -432,7 +432,7 @@ namespace {
 // forward (-1) or inverse (+1, with 1/(nx ny)) 2D transform of buffer b
 template <class Rl> cudaError_t fft2(pss_grid *g, V2<Rl> *b, int dir)
 {
-    cudaError_t e = fft_rows<Rl>(b, g->nx, g->batch * g->ny, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
+    cudaError_t e = fft_rows<Rl>(b, g->nx, g->ny, g->batch, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
     if (e != cudaSuccess) return e;
     const Rl sc = dir > 0 ? Rl(1.0 / (double(g->nx) * double(g->ny))) : Rl(1);
     return fft_cols<Rl>(b, g->nx, g->ny, g->batch, dir, sc, Tw<Rl>(g->twy), g->stream);
@@ -550,7 +550,7 @@ template <class Rl> int sg_step(pss_grid *g, int64_t n)
                *h = static_cast<V2<Rl> *>(g->hbuf[2]);
         for (int64_t i = 0; i < n; ++i) {
             if ((rc = g->pass_begin(0))) return rc;
-            cudaError_t e = sg_row_pass_r2c<Rl>(h, g->nx, g->sx, g->batch * g->ny, Tw<Rl>(g->twm), Tw<Rl>(g->twx),
+            cudaError_t e = sg_row_pass_r2c<Rl>(h, g->nx, g->sx, g->ny, g->batch, Tw<Rl>(g->twm), Tw<Rl>(g->twx),
                                                 g->stream);
             if ((rc = g->pass_end()) || (rc = g->cuda(e, "sg row pass (half spectrum)"))) return rc;
             if ((rc = g->pass_begin(1))) return rc;
@@ -562,7 +562,7 @@ template <class Rl> int sg_step(pss_grid *g, int64_t n)
     }
     for (int64_t i = 0; i < n; ++i) {
         if ((rc = g->pass_begin(0))) return rc;
-        cudaError_t e = sg_row_pass<Rl>(B<Rl>(g, 2), g->nx, g->batch * g->ny, Tw<Rl>(g->twx), g->stream);
+        cudaError_t e = sg_row_pass<Rl>(B<Rl>(g, 2), g->nx, g->ny, g->batch, Tw<Rl>(g->twx), g->stream);
         if ((rc = g->pass_end()) || (rc = g->cuda(e, "sg row pass"))) return rc;
         if ((rc = g->pass_begin(1))) return rc;
         e = sg_col_pass<Rl>(B<Rl>(g, 2), B<Rl>(g, 0), B<Rl>(g, 1), g->nx, g->ny, g->batch, Rt<Rl>(g->kx2),
@@ -850,7 +850,7 @@ namespace {
 
 template <class Rl> cudaError_t fft2_one(pss_grid *g, V2<Rl> *b, int dir)
 {
-    cudaError_t e = fft_rows<Rl>(b, g->nx, g->ny, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
+    cudaError_t e = fft_rows<Rl>(b, g->nx, g->ny, 1, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
     if (e != cudaSuccess) return e;
     const Rl sc = dir > 0 ? Rl(1.0 / (double(g->nx) * double(g->ny))) : Rl(1);
     return fft_cols<Rl>(b, g->nx, g->ny, 1, dir, sc, Tw<Rl>(g->twy), g->stream);
@@ -880,7 +880,7 @@ template <class Rl> int field_set(pss_grid *g, int64_t f, const void *a, const v
     const size_t fb = size_t(g->npts) * g->esz;
     if (g->p.eq == PSS_EQ_NLS) {
         if ((rc = g->cuda(cudaMemcpyAsync(Bf<Rl>(g, 0, f), a, fb, kind_in(where), g->stream), "copy")) ||
-            (rc = g->cuda(fft_rows<Rl>(Bf<Rl>(g, 0, f), g->nx, g->ny, -1, Rl(1), Tw<Rl>(g->twx), g->stream), "row fft")))
+            (rc = g->cuda(fft_rows<Rl>(Bf<Rl>(g, 0, f), g->nx, g->ny, 1, -1, Rl(1), Tw<Rl>(g->twx), g->stream), "row fft")))
             return rc;
     } else if (g->p.eq == PSS_EQ_SG) {
         if ((rc = load_real_one<Rl>(g, f, a, where, 3, 0, false)) ||
@@ -923,7 +923,7 @@ template <class Rl> int field_get(pss_grid *g, int64_t f, void *a, void *b, int 
     if (g->p.eq == PSS_EQ_NLS) {
         if ((rc = g->cuda(cudaMemcpyAsync(Bf<Rl>(g, 1, f), Bf<Rl>(g, 0, f), fb, cudaMemcpyDeviceToDevice, g->stream),
                           "copy")) ||
-            (rc = g->cuda(fft_rows<Rl>(Bf<Rl>(g, 1, f), g->nx, g->ny, +1, Rl(1.0 / double(g->nx)), Tw<Rl>(g->twx),
+            (rc = g->cuda(fft_rows<Rl>(Bf<Rl>(g, 1, f), g->nx, g->ny, 1, +1, Rl(1.0 / double(g->nx)), Tw<Rl>(g->twx),
                                        g->stream), "row inverse")) ||
             (rc = g->cuda(cudaMemcpyAsync(a, Bf<Rl>(g, 1, f), fb, kind_out(where), g->stream), "copy")))
             return rc;
@@ -1324,11 +1324,11 @@ extern "C" int pss_fft2d(void *data, int64_t nx, int64_t ny, int64_t batch, int 
     cudaError_t e;
     const double inv = direction > 0 ? 1.0 / (double(nx) * double(ny)) : 1.0;
     if (precision == PSS_FP32) {
-        e = fft_rows<float>(static_cast<float2 *>(data), nx, batch * ny, direction, 1.0f, static_cast<float4 *>(twx), s);
+        e = fft_rows<float>(static_cast<float2 *>(data), nx, ny, batch, direction, 1.0f, static_cast<float4 *>(twx), s);
         if (e == cudaSuccess)
             e = fft_cols<float>(static_cast<float2 *>(data), nx, ny, batch, direction, float(inv), static_cast<float4 *>(twy), s);
     } else {
-        e = fft_rows<double>(static_cast<double2 *>(data), nx, batch * ny, direction, 1.0, static_cast<double2 *>(twx), s);
+        e = fft_rows<double>(static_cast<double2 *>(data), nx, ny, batch, direction, 1.0, static_cast<double2 *>(twx), s);
         if (e == cudaSuccess)
             e = fft_cols<double>(static_cast<double2 *>(data), nx, ny, batch, direction, inv, static_cast<double2 *>(twy), s);
     }

@@ -23,7 +23,7 @@ template <class Rl> using TW = typename twid<Rl>::type;
 // ---- plain transforms (k_fft.cu) -------------------------------------------
 // dir -1 forward, +1 inverse (unnormalised); the result is multiplied by scale.
 template <class Rl>
-cudaError_t fft_rows(V2<Rl> *data, int64_t nx, int64_t rows_total, int dir, Rl scale,
+cudaError_t fft_rows(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, int dir, Rl scale,
                      const TW<Rl> *twx, cudaStream_t s);
 template <class Rl>
 cudaError_t fft_cols(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, int dir, Rl scale,
@@ -32,7 +32,7 @@ cudaError_t fft_cols(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, int di
 // ---- NLS passes (k_nls.cu) ---------------------------------------------------
 // Row pass: row inverse FFT, psi <- psi exp(-i sigma dt |psi|^2), row forward FFT.
 template <class Rl>
-cudaError_t nls_row_pass(V2<Rl> *data, int64_t nx, int64_t rows_total, Rl sigma_dt,
+cudaError_t nls_row_pass(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, Rl sigma_dt,
                          const TW<Rl> *twx, cudaStream_t s);
 // Column pass: column forward FFT, multiply by scale * a[x] * b[y]
 // (a = exp(-i kx^2 tau), b = exp(-i ky^2 tau); the tables hold a - 1 and
@@ -46,7 +46,7 @@ cudaError_t nls_col_pass(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, Rl
 // Row pass on H (column inverse transform of uhat^n / (nx ny)): row inverse
 // FFT, s = sin(Re), row forward FFT, in place.
 template <class Rl>
-cudaError_t sg_row_pass(V2<Rl> *h, int64_t nx, int64_t rows_total, const TW<Rl> *twx, cudaStream_t s);
+cudaError_t sg_row_pass(V2<Rl> *h, int64_t nx, int64_t ny, int64_t batch, const TW<Rl> *twx, cudaStream_t s);
 // Column pass: column FFT of S = F sin u^n; d <- d - (a u + dt^2 S)/(1 + a/4),
 // u <- u + d (a = dt^2 |k|^2), in place; H <- column inverse FFT of u / (nreal ny).
 // nx is the row stride (columns processed), nreal the real row length (0: nx).
@@ -58,7 +58,7 @@ cudaError_t sg_col_pass(V2<Rl> *h, V2<Rl> *u, V2<Rl> *d, int64_t nx, int64_t ny,
 // Half-spectrum (real-to-complex) sine-Gordon row pass, k_sg_r2c.cu: rows of
 // stride sx holding kx = 0 .. nx/2; twm: twiddles of length nx/2, twn: of nx.
 template <class Rl>
-cudaError_t sg_row_pass_r2c(V2<Rl> *h, int64_t nx, int64_t sx, int64_t rows_total, const TW<Rl> *twm,
+cudaError_t sg_row_pass_r2c(V2<Rl> *h, int64_t nx, int64_t sx, int64_t ny, int64_t batch, const TW<Rl> *twm,
                             const TW<Rl> *twn, cudaStream_t s);
 // full [batch][ny][nx] spectrum of real fields <-> half spectrum [batch][ny][sx]
 template <class Rl>

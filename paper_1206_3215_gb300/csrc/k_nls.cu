@@ -305,10 +305,10 @@ template <class Rl> struct NlsCol {
 };
 
 template <class Rl>
-cudaError_t nls_row_pass(V2<Rl> *data, int64_t nx, int64_t rows_total, Rl sigma_dt,
+cudaError_t nls_row_pass(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, Rl sigma_dt,
                          const TW<Rl> *twx, cudaStream_t s)
 {
-    return launch_row<Rl>(nx, NlsRow<Rl>{data, sigma_dt}, twx, rows_total, s);
+    return launch_row<Rl>(nx, ny, NlsRow<Rl>{data, sigma_dt}, twx, batch, s);
 }
 
 template <class Rl>
@@ -319,7 +319,7 @@ cudaError_t nls_col_pass(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, Rl
 }
 
 #define PSS_INST(Rl)                                                                            \
-    template cudaError_t nls_row_pass<Rl>(V2<Rl> *, int64_t, int64_t, Rl, const TW<Rl> *,        \
+    template cudaError_t nls_row_pass<Rl>(V2<Rl> *, int64_t, int64_t, int64_t, Rl, const TW<Rl> *, \
                                           cudaStream_t);                                          \
     template cudaError_t nls_col_pass<Rl>(V2<Rl> *, int64_t, int64_t, int64_t, Rl,               \
                                           const TW<Rl> *, const TW<Rl> *, const TW<Rl> *, int *, \

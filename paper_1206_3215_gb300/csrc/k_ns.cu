@@ -76,8 +76,8 @@ cudaError_t ns_row_pass(V2<Rl> *c1, V2<Rl> *c2, const void *fs, int64_t nx, int6
 {
     int lgy = 0;
     while ((int64_t(1) << lgy) < ny) ++lgy;  // ny is a power of two
-    return launch_row<Rl>(nx, NsRow<Rl>{c1, c2, static_cast<const NsField *>(fs), lgy, dealias ? 1 : 0, half ? 1 : 0},
-                          twx, batch * ny, s);
+    return launch_row<Rl>(nx, ny, NsRow<Rl>{c1, c2, static_cast<const NsField *>(fs), lgy, dealias ? 1 : 0, half ? 1 : 0},
+                          twx, batch, s);
 }
 
 template <class Rl>

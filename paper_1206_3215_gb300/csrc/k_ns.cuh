@@ -478,6 +478,7 @@ cudaError_t ns_col_run(V2<Rl> *c1, V2<Rl> *c2, V2<Rl> *const w[3], V2<Rl> *jn, v
     switch (ny) {
 #define PSS_CASE(N)                                                                          \
     case N:                                                                                  \
+        static_assert(ColCfgOf<Rl, N, Op>::W == ColCfgOf<Rl, N, Op, 2>::W, "one tile width"); \
         op.W = ColCfgOf<Rl, N, Op>::W;                                                       \
         if (sx % op.W) return cudaErrorInvalidValue;                                         \
         ns_skip_groups(nxf, sx, op.W, HALF, dealias, &op.skip_lo, &op.skip_n);               \

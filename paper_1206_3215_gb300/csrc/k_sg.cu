@@ -154,9 +154,9 @@ template <class Rl> struct SgCol {
 };
 
 template <class Rl>
-cudaError_t sg_row_pass(V2<Rl> *h, int64_t nx, int64_t rows_total, const TW<Rl> *twx, cudaStream_t s)
+cudaError_t sg_row_pass(V2<Rl> *h, int64_t nx, int64_t ny, int64_t batch, const TW<Rl> *twx, cudaStream_t s)
 {
-    return launch_row<Rl>(nx, SgRow<Rl>{h}, twx, rows_total, s);
+    return launch_row<Rl>(nx, ny, SgRow<Rl>{h}, twx, batch, s);
 }
 
 // nx: row stride of the arrays (the columns processed); nreal: points per
@@ -171,7 +171,7 @@ cudaError_t sg_col_pass(V2<Rl> *h, V2<Rl> *u, V2<Rl> *d, int64_t nx, int64_t ny,
 }
 
 #define PSS_INST(Rl)                                                                              \
-    template cudaError_t sg_row_pass<Rl>(V2<Rl> *, int64_t, int64_t, const TW<Rl> *, cudaStream_t); \
+    template cudaError_t sg_row_pass<Rl>(V2<Rl> *, int64_t, int64_t, int64_t, const TW<Rl> *, cudaStream_t); \
     template cudaError_t sg_col_pass<Rl>(V2<Rl> *, V2<Rl> *, V2<Rl> *, int64_t, int64_t, int64_t,   \
                                          const Rl *, const Rl *, Rl, const TW<Rl> *, int *, cudaStream_t, \
                                          int64_t);

@@ -26,10 +26,12 @@ namespace pss {
 
 namespace {
 
-template <class Rl, int M> struct R2cCfg {
-    static constexpr int P = Shape<Rl>::rowP(M);
+template <class Rl, int M, bool SMALL> struct R2cCfg {
+    static constexpr int P = Shape<Rl>::rowP(M, SMALL);
     static constexpr int T = M / P;
-    static constexpr int ROWS = T >= 256 ? 1 : 256 / T;
+    // short rows: smaller CTAs, so that few rows still spread over the SMs
+    static constexpr int RT = M <= 256 ? 128 : 256;
+    static constexpr int ROWS = T >= RT ? 1 : RT / T;
     static constexpr int THREADS = ROWS * T;
     // barrier of one row's threads (fft_sync): a warp (T <= 32: the rows are
     // warp-local), the CTA, or the row's own named barrier
@@ -37,17 +39,17 @@ template <class Rl, int M> struct R2cCfg {
     static constexpr int PADLOG = pad_log(P);
     static constexpr int LINE = M + (M >> PADLOG) + 2;  // the padded line plus X_M
     static constexpr size_t SMEM = size_t(ROWS) * LINE * sizeof(V2<Rl>);
-    static constexpr int MIN_CTAS = (sizeof(Rl) == 4 && THREADS * 2 <= 512) ? 2 : 1;
+    static constexpr int MIN_CTAS = sizeof(Rl) == 4 ? imin(imax(512 / THREADS, 1), 16) : 1;
 };
 
 // rows_total = batch * ny rows of stride sx; twm: length-M transform
 // twiddles, twn: length-N twiddles (e^{-2 pi i e / N}, e < N)
-template <class Rl, int M>
-__global__ void __launch_bounds__(R2cCfg<Rl, M>::THREADS, R2cCfg<Rl, M>::MIN_CTAS)
+template <class Rl, int M, bool SMALL>
+__global__ void __launch_bounds__(R2cCfg<Rl, M, SMALL>::THREADS, R2cCfg<Rl, M, SMALL>::MIN_CTAS)
     k_sg_row_r2c(V2<Rl> *__restrict__ h, int64_t sx, int64_t rows_total, const TW<Rl> *__restrict__ twm,
                  const TW<Rl> *__restrict__ twn)
 {
-    using C = R2cCfg<Rl, M>;
+    using C = R2cCfg<Rl, M, SMALL>;
     using V = V2<Rl>;
     using Sm = SmemLine<V, C::PADLOG>;
     constexpr int P = C::P, T = C::T;
@@ -109,12 +111,12 @@ __global__ void __launch_bounds__(R2cCfg<Rl, M>::THREADS, R2cCfg<Rl, M>::MIN_CTA
     cp_async_wait<0>();
 }
 
-template <class Rl, int M>
+template <class Rl, int M, bool SMALL>
 cudaError_t launch_r2c(V2<Rl> *h, int64_t sx, int64_t rows_total, const TW<Rl> *twm, const TW<Rl> *twn,
                        cudaStream_t s)
 {
-    using C = R2cCfg<Rl, M>;
-    auto k = k_sg_row_r2c<Rl, M>;
+    using C = R2cCfg<Rl, M, SMALL>;
+    auto k = k_sg_row_r2c<Rl, M, SMALL>;
     static std::atomic<unsigned> done{0};
     static int ctas[32] = {};
     cudaError_t e = allow_smem(k, C::SMEM, done);
@@ -158,12 +160,17 @@ __global__ void k_unpack_half(const V2<Rl> *__restrict__ half, V2<Rl> *__restric
 }  // namespace
 
 template <class Rl>
-cudaError_t sg_row_pass_r2c(V2<Rl> *h, int64_t nx, int64_t sx, int64_t rows_total, const TW<Rl> *twm,
+cudaError_t sg_row_pass_r2c(V2<Rl> *h, int64_t nx, int64_t sx, int64_t ny, int64_t batch, const TW<Rl> *twm,
                             const TW<Rl> *twn, cudaStream_t s)
 {
+    const int64_t rows_total = batch * ny;
+    const bool small = nx * ny <= SMALL_FIELD;
     switch (nx / 2) {
 #define PSS_CASE(N) \
-    case N: return launch_r2c<Rl, N>(h, sx, rows_total, twm, twn, s);
+    case N:                                                                                        \
+        if constexpr (short_variant<Rl>(N))                                                        \
+            if (small) return launch_r2c<Rl, N, true>(h, sx, rows_total, twm, twn, s);             \
+        return launch_r2c<Rl, N, false>(h, sx, rows_total, twm, twn, s);
         PSS_CASE(8) PSS_CASE(16) PSS_CASE(32) PSS_CASE(64) PSS_CASE(128) PSS_CASE(256) PSS_CASE(512)
         PSS_CASE(1024) PSS_CASE(2048) PSS_CASE(4096)
 #undef PSS_CASE
@@ -192,7 +199,7 @@ cudaError_t unpack_half(const V2<Rl> *half, V2<Rl> *full, int64_t nx, int64_t ny
 }
 
 #define PSS_INST(Rl)                                                                                        \
-    template cudaError_t sg_row_pass_r2c<Rl>(V2<Rl> *, int64_t, int64_t, int64_t, const TW<Rl> *,          \
+    template cudaError_t sg_row_pass_r2c<Rl>(V2<Rl> *, int64_t, int64_t, int64_t, int64_t, const TW<Rl> *, \
                                              const TW<Rl> *, cudaStream_t);                                 \
     template cudaError_t pack_half<Rl>(const V2<Rl> *, V2<Rl> *, int64_t, int64_t, int64_t, int64_t,        \
                                        cudaStream_t);                                                       \

@@ -254,8 +254,11 @@ inline cudaError_t launch_col_split(Op op, const TW<Rl> *tw, int64_t nx, int64_t
 }
 
 template <class Rl, int N, class Op>
-inline cudaError_t launch_row_n(Op op, const TW<Rl> *tw, int64_t rows_total, cudaStream_t s)
+inline cudaError_t launch_row_n(Op op, const TW<Rl> *tw, int64_t ny, int64_t batch, cudaStream_t s)
 {
+    const int64_t rows_total = batch * ny;
+    if constexpr (short_variant<Rl>(N))
+        if (N * ny <= SMALL_FIELD) return launch_row_v<Rl, N, Op, 2>(op, tw, rows_total, s);
     if constexpr (tunable<Rl, N, Op>()) {
         static PlanSlot slot;
         // every tile width divides the row stride: a variant choice needs no caller change
@@ -267,6 +270,10 @@ inline cudaError_t launch_row_n(Op op, const TW<Rl> *tw, int64_t rows_total, cud
 template <class Rl, int N, class Op>
 inline cudaError_t launch_col_n(Op op, const TW<Rl> *tw, int64_t nx, int64_t batch, cudaStream_t s)
 {
+    if constexpr (short_variant<Rl>(N)) {
+        static_assert(!tma_col<Rl, N, Op>(), "variant 2 has no tensor-copy pass");
+        if (N * nx <= SMALL_FIELD) return launch_col_v<Rl, N, Op, 2>(op, tw, nx, batch, s);
+    }
     if constexpr (tunable<Rl, N, Op>()) {
         static PlanSlot slot;
         if (nx % ColCfgOf<Rl, N, Op, 1>::W == 0 && plan_pick(slot) == 1)
@@ -283,11 +290,11 @@ inline cudaError_t launch_col_n(Op op, const TW<Rl> *tw, int64_t nx, int64_t bat
 
 // Row pass over every row of a [batch][ny][nx] array: transform length nx.
 template <class Rl, class Op>
-inline cudaError_t launch_row(int64_t nx, Op op, const TW<Rl> *tw, int64_t rows_total, cudaStream_t s)
+inline cudaError_t launch_row(int64_t nx, int64_t ny, Op op, const TW<Rl> *tw, int64_t batch, cudaStream_t s)
 {
     switch (nx) {
 #define PSS_CASE(N) \
-    case N: return launch_row_n<Rl, N>(op, tw, rows_total, s);
+    case N: return launch_row_n<Rl, N>(op, tw, ny, batch, s);
         PSS_FOR_EACH_N(PSS_CASE)
 #undef PSS_CASE
     default: return cudaErrorInvalidValue;

@@ -116,8 +116,39 @@ template <class Rl> struct Shape {
     // rows of at least PSS_BIG_N points may use PSS_ROW_P_BIG / PSS_COL_P_BIG
     static constexpr int RPB = sizeof(Rl) == 4 ? PSS_ROW_P_BIG : RP;
     static constexpr int CPB = sizeof(Rl) == 4 ? PSS_COL_P_BIG : CP;
-    __host__ __device__ static constexpr int rowP(int n) { return n < RP ? n : n >= PSS_BIG_N ? RPB : RP; }
-    __host__ __device__ static constexpr int colP(int n) { return n < CP ? n : n >= PSS_BIG_N ? CPB : CP; }
+    // Short lines take fewer points per thread: their grids are mostly small,
+    // and a pass over them is bound by the length of one thread's instruction
+    // chain (a 32-point thread runs about 3000 instructions per pass) on SMs
+    // that hold a warp or two, in FP64 by the two FP64 lanes of each SM in
+    // use, so the same points spread over more threads and SMs finish sooner.
+    // `small` (variant 2): fields of at most SMALL_FIELD points, where that
+    // outweighs the extra stages; larger fields of short lines keep more
+    // points (FP32 128 x 4096 x 32 NLS, 16 / 8 points: 206 / 216 us per step;
+    // FP64 fft 64 x 4096 x 8, 4 / 2 points: 274 / 300 us).  The choice
+    // depends on the grid alone, not on the batch, so that a batch rounds as
+    // its fields do alone.  Per step, from 32 (FP32) and 16 (FP64) points to
+    // these: FP32 NLS 64^2 9.8 -> 5.0 us, 128^2 x 8 11.5 -> 6.3,
+    // 256^2 x 8 13.6 -> 10.1, SG 256^2 x 8 on half spectra 24.9 -> 12.4;
+    // FP64 NLS 64^2 57.5 -> 13.3 us, 256^2 72 -> 26, SG 256^2 x 2 152 -> 31,
+    // NS 256^2 243 -> 102.  At 256 FP32, 8 points gain little more alone
+    // (NLS 256^2 7.9 -> 6.6 us) and lose 24 % at a batch of 32.
+    __host__ __device__ static constexpr int shortP(int n, bool small)
+    {
+        if (sizeof(Rl) == 4) return n <= 16 ? 4 : n <= 64 || (n <= 128 && small) ? 8 : 16;
+        if (small) return n <= 16 ? 4 : n <= 64 ? 2 : n <= 256 ? 4 : 8;
+        return n <= 64 ? 4 : 8;
+    }
+    // lines that take shortP points: up to 256 (FP32) and 512 (FP64; radix 8
+    // three times instead of 16, 16, 2: one 512^2 field 144 -> 99 us, four the same)
+    static constexpr int SHORT = sizeof(Rl) == 4 ? 256 : 512;
+    __host__ __device__ static constexpr int rowP(int n, bool small = false)
+    {
+        return n <= SHORT ? shortP(n, small) : n >= PSS_BIG_N ? RPB : RP;
+    }
+    __host__ __device__ static constexpr int colP(int n, bool small = false)
+    {
+        return n <= SHORT ? shortP(n, small) : n >= PSS_BIG_N ? CPB : CP;
+    }
     // columns per tile: 64-byte row segments (FP32) when the thread budget
     // (PSS_COL_THREADS) and shared memory (nbuf buffers) allow.  With `wide`,
     // a tile whose row segments would drop below 32 bytes (one DRAM sector)
@@ -126,7 +157,9 @@ template <class Rl> struct Shape {
     // where 32-byte segments fit in 256 threads, the wider tile was slower)
     __host__ __device__ static constexpr int cols_capped(int n, int p, int nbuf, int cap)
     {
-        int w = sizeof(Rl) == 4 ? PSS_COL_WMAX : 4;
+        // FP64 up to 256: two columns (32-byte row segments) for more tiles, at
+        // 16 a whole warp
+        int w = sizeof(Rl) == 4 ? PSS_COL_WMAX : n > 256 ? 4 : n > 16 ? 2 : 8;
         while (w > 1 && ((long)nbuf * w * (n + n / 16) * ESZ > 200 * 1024L || w * (n / p) > cap)) w /= 2;
         return w;
     }
@@ -140,7 +173,8 @@ template <class Rl> struct Shape {
 // Launch-shape variants a lean FP32 pass is compiled in (the plan the
 // autotuner picks from, per kernel instance): 0 = the shapes above (32 points
 // per thread, two CTAs of <= 128 registers per SM); 1 = 16 points per thread,
-// four CTAs per SM (<= 64 registers).
+// four CTAs per SM (<= 64 registers).  Variant 2 is not tuned: the shapes of
+// short lines in small fields (short_variant).
 template <class Rl, int VAR> struct VarShape {
     static constexpr int PCAP = VAR == 1 ? 16 : 1 << 20;
     static constexpr int CTAS = VAR == 1 ? 4 : Shape<Rl>::MIN_CTAS;
@@ -148,6 +182,23 @@ template <class Rl, int VAR> struct VarShape {
 };
 __host__ __device__ constexpr int imin(int a, int b) { return a < b ? a : b; }
 __host__ __device__ constexpr int imax(int a, int b) { return a > b ? a : b; }
+// fields whose short lines run in variant 2 (points per field), and the lines
+// whose points per thread that changes
+constexpr int64_t SMALL_FIELD = 1 << 16;
+template <class Rl> __host__ __device__ constexpr bool short_variant(int n)
+{
+    return Shape<Rl>::rowP(n, true) != Shape<Rl>::rowP(n, false);
+}
+// resident CTAs per SM a pass budgets its registers for (LEAN ops; else 1):
+// VS::CTAS, fewer where those exceed VS::TPS threads (512: 128 registers each);
+// the small CTAs of short FP32 lines as many (up to 16) as fill VS::TPS threads
+template <class Rl, int VAR> __host__ __device__ constexpr int lean_ctas(bool lean, int threads, int n)
+{
+    using VS = VarShape<Rl, VAR>;
+    const int fit = imax(VS::TPS / threads, 1);
+    if (!lean) return 1;
+    return sizeof(Rl) == 4 && n <= 256 ? imin(imax(VS::CTAS, fit), 16) : imin(VS::CTAS, fit);
+}
 
 // dynamic shared memory a pass may use per CTA (the GB300 limit is 227 KB)
 constexpr size_t SMEM_LIMIT = 200 * 1024;
@@ -183,11 +234,11 @@ __host__ __device__ constexpr int col_stride(int base, int W, int ESZ)
 // whose transforms fit in 128 registers; otherwise a double buffer, one CTA.
 template <class Rl, int N, int NIN, bool LEAN = false, int PMAX = 32, int VAR = 0> struct RowCfg {
     using VS = VarShape<Rl, VAR>;
-    static constexpr int P = imin(imin(Shape<Rl>::rowP(N), PMAX), VS::PCAP);
+    static constexpr int P = imin(imin(Shape<Rl>::rowP(N, VAR == 2), PMAX), VS::PCAP);
     static constexpr int T = N / P;
-    // ~256 threads per CTA; small rows (N <= 256) take ~64 so that a batch of
-    // small grids still spreads over many SMs (a 128^2 field is 2 CTAs, not 1/2)
-    static constexpr int RT = N <= 256 ? PSS_ROW_THREADS_SMALL : PSS_ROW_THREADS;
+    // ~256 threads per CTA; small rows (N <= 256) take ~64 (FP64: one warp) so
+    // that a batch of small grids still spreads over many SMs
+    static constexpr int RT = N <= 256 ? (sizeof(Rl) == 4 ? PSS_ROW_THREADS_SMALL : 32) : PSS_ROW_THREADS;
     static constexpr int ROWS = T >= RT ? 1 : RT / T;
     static constexpr int PADLOG = pad_log(P);
     static constexpr int LINE = N + (N >> PADLOG);
@@ -200,15 +251,12 @@ template <class Rl, int N, int NIN, bool LEAN = false, int PMAX = 32, int VAR = 
     static constexpr int MAXB = LEAN ? Shape<Rl>::MAX_NBUF : 2;
     static constexpr int NBUF = (MAXB > 1 && size_t(2) * BUF * Shape<Rl>::ESZ <= SMEM_LIMIT) ? 2 : 1;
     static constexpr size_t SMEM = size_t(NBUF) * BUF * Shape<Rl>::ESZ;
-    // resident CTAs the registers are budgeted for: at most VS::TPS threads
-    // per SM (512: 128 registers each)
-    static constexpr int MIN_CTAS =
-        LEAN ? (THREADS * VS::CTAS <= VS::TPS ? VS::CTAS : (VS::TPS / THREADS > 1 ? VS::TPS / THREADS : 1)) : 1;
+    static constexpr int MIN_CTAS = lean_ctas<Rl, VAR>(LEAN, THREADS, N);
 };
 
 template <class Rl, int N, int NIN, bool LEAN = false, int PMAX = 32, int VAR = 0> struct ColCfg {
     using VS = VarShape<Rl, VAR>;
-    static constexpr int P = imin(imin(Shape<Rl>::colP(N), PMAX), VS::PCAP);
+    static constexpr int P = imin(imin(Shape<Rl>::colP(N, VAR == 2), PMAX), VS::PCAP);
     static constexpr int T = N / P;
     // lean ops (one buffer, <= 128 registers) may take the wide tiles
     static constexpr int W = LEAN ? Shape<Rl>::cols(N, P, NIN * Shape<Rl>::MAX_NBUF, true) : Shape<Rl>::cols(N, P);
@@ -220,10 +268,7 @@ template <class Rl, int N, int NIN, bool LEAN = false, int PMAX = 32, int VAR = 
     static constexpr int MAXB = LEAN ? Shape<Rl>::MAX_NBUF : 2;
     static constexpr int NBUF = (MAXB > 1 && size_t(2) * BUF * Shape<Rl>::ESZ <= SMEM_LIMIT) ? 2 : 1;
     static constexpr size_t SMEM = size_t(NBUF) * BUF * Shape<Rl>::ESZ;
-    // resident CTAs the registers are budgeted for: at most VS::TPS threads
-    // per SM (512: 128 registers each)
-    static constexpr int MIN_CTAS =
-        LEAN ? (THREADS * VS::CTAS <= VS::TPS ? VS::CTAS : (VS::TPS / THREADS > 1 ? VS::TPS / THREADS : 1)) : 1;
+    static constexpr int MIN_CTAS = lean_ctas<Rl, VAR>(LEAN, THREADS, N);
 };
 
 // points per thread an op allows at length N: Op::pmax(N) where the op
