@@ -41,6 +41,26 @@ __device__ __forceinline__ void phase_short(float a, float &sn, float &cm1)
     cm1 = t2 * __fmaf_rn(t2, 1.0f / 24, -0.5f);
 }
 
+// FP64 on |a| < 2^-9: sin a = a - a^3/6 + a^5/120, cos a - 1 = -a^2/2 + a^4/24 -
+// a^6/720; the first omitted terms (a^7/5040, a^8/40320) are below 2e-23 and
+// 6e-27.  The FP64 passes are bound by the two FP64 lanes of an SM, so the
+// terms count: with the phase formed once and compared through its high word
+// (integer pipe), 16 FP64 operations per point instead of 26.
+constexpr double phase_short_range64() { return 0x1p-9; }
+__device__ __forceinline__ void phase_short(double a, double &sn, double &cm1)
+{
+    const double t2 = a * a;
+    sn = fma(a * t2, fma(t2, 1.0 / 120, -1.0 / 6), a);
+    cm1 = t2 * fma(t2, fma(t2, -1.0 / 720, 1.0 / 24), -0.5);
+}
+// |a| as an integer that orders like it (its high word); NaN counts as 0: the
+// straight-line sums carry it through
+__device__ __forceinline__ int phase_mag(double a)
+{
+    const int h = __double2hiint(a) & 0x7fffffff;
+    return h > 0x7ff00000 ? 0 : h;
+}
+
 template <class Rl> __device__ __forceinline__ void phase_terms(Rl th, Rl &sn, Rl &cm1)
 {
     constexpr int KMAX = sizeof(Rl) == 4 ? 130 : 1026;
@@ -88,8 +108,34 @@ template <class Rl> struct NlsRow {
             // increment is formed without cancellation, so the modulus is
             // kept to the final rounding.  When every phase of this thread is
             // in the Taylor range (always, at the workload's dt |psi|^2), the
-            // straight-line Taylor code runs (FP32: the short sums below
-            // 1/64); the halving path is out of line.
+            // straight-line Taylor code runs (the short sums below 1/64 in
+            // FP32, 2^-9 in FP64); the halving path is out of line.
+            if constexpr (sizeof(Rl) == 8) {
+                Rl th[P];
+                int big = 0;
+#pragma unroll
+                for (int m = 0; m < P; ++m) {
+                    th[m] = sigma_dt * fma(v[m].x, v[m].x, v[m].y * v[m].y);
+                    big = max(big, phase_mag(th[m]));
+                }
+                auto apply = [&](auto terms) {
+#pragma unroll
+                    for (int m = 0; m < P; ++m) {
+                        const Rl x = v[m].x, y = v[m].y;
+                        Rl sn, cm1;
+                        terms(th[m], sn, cm1);
+                        v[m].x = x + fma(x, cm1, y * sn);
+                        v[m].y = y + fma(y, cm1, -(x * sn));
+                    }
+                };
+                if (big < __double2hiint(phase_short_range64()))
+                    apply([](Rl a, Rl &sn, Rl &cm1) { phase_short(a, sn, cm1); });
+                else if (big < __double2hiint(phase_taylor_range<double>()))
+                    apply([](Rl a, Rl &sn, Rl &cm1) { phase_taylor(a, sn, cm1); });
+                else
+                    apply([](Rl a, Rl &sn, Rl &cm1) { phase_terms(a, sn, cm1); });
+                return;
+            }
             Rl big = Rl(0);
 #pragma unroll
             for (int m = 0; m < P; ++m) big = fmax(big, fabs(sigma_dt * (v[m].x * v[m].x + v[m].y * v[m].y)));
@@ -103,16 +149,9 @@ template <class Rl> struct NlsRow {
                     v[m].y = y + (y * cm1 - x * sn);
                 }
             };
-            // one straight-line body (FP32: the short sums; FP64: the Taylor
-            // sums) and the general path, so the code stays small
-            bool fast;
-            if constexpr (sizeof(Rl) == 4) fast = big <= phase_short_range();
-            else fast = big <= phase_taylor_range<Rl>();
-            if (fast) {
-                apply([](Rl a, Rl &sn, Rl &cm1) {
-                    if constexpr (sizeof(Rl) == 4) phase_short(a, sn, cm1);
-                    else phase_taylor(a, sn, cm1);
-                });
+            // one straight-line body and the general path, so the code stays small
+            if (big <= phase_short_range()) {
+                apply([](Rl a, Rl &sn, Rl &cm1) { phase_short(a, sn, cm1); });
             } else {
 #pragma unroll
                 for (int m = 0; m < P; ++m) {
@@ -162,6 +201,10 @@ template <class V, class W> __device__ __forceinline__ V apply_km1(V z, W km1)
 // the increment is formed as in apply_km1 and s z (exact) is added inside
 // the last fused multiply-add, so the result is bitwise that of
 // apply_km1(s z, K - 1) with the scaling folded in (two instructions fewer)
+__device__ __forceinline__ double2 apply_skm1(double2 z, double s, double2 skm1)
+{
+    return {fma(z.x, s, fma(z.x, skm1.x, -(z.y * skm1.y))), fma(z.y, s, fma(z.x, skm1.y, z.y * skm1.x))};
+}
 __device__ __forceinline__ float2 apply_skm1(float2 z, float s, float4 skm1)
 {
     const float cr = __fmaf_rn(z.x, skm1.z, -z.y * skm1.w);
@@ -273,12 +316,9 @@ template <class Rl> struct NlsCol {
                     }
                 }
             } else {
+                const V2<Rl> sa{a.x * scale, a.y * scale};  // scale is a power of two: exact
 #pragma unroll
-                for (int m = 0; m < P; ++m) {
-                    // scale is a power of two: exact
-                    const V2<Rl> z = apply_km1(cscale(v[m], scale), a);
-                    v[m] = apply_km1(z, __ldg(byl + t + T * m));
-                }
+                for (int m = 0; m < P; ++m) v[m] = apply_km1(apply_skm1(v[m], scale, sa), __ldg(byl + t + T * m));
             }
         };
         if constexpr (PSS_SHARED_FFT && sizeof(Rl) == 4) {
