@@ -116,38 +116,33 @@ template <class Rl> struct Shape {
     // rows of at least PSS_BIG_N points may use PSS_ROW_P_BIG / PSS_COL_P_BIG
     static constexpr int RPB = sizeof(Rl) == 4 ? PSS_ROW_P_BIG : RP;
     static constexpr int CPB = sizeof(Rl) == 4 ? PSS_COL_P_BIG : CP;
-    // Short lines take fewer points per thread: their grids are mostly small,
-    // and a pass over them is bound by the length of one thread's instruction
-    // chain (a 32-point thread runs about 3000 instructions per pass) on SMs
-    // that hold a warp or two, in FP64 by the two FP64 lanes of each SM in
-    // use, so the same points spread over more threads and SMs finish sooner.
-    // `small` (variant 2): fields of at most SMALL_FIELD points, where that
-    // outweighs the extra stages; larger fields of short lines keep more
-    // points (FP32 128 x 4096 x 32 NLS, 16 / 8 points: 206 / 216 us per step;
-    // FP64 fft 64 x 4096 x 8, 4 / 2 points: 274 / 300 us).  The choice
-    // depends on the grid alone, not on the batch, so that a batch rounds as
-    // its fields do alone.  Per step, from 32 (FP32) and 16 (FP64) points to
-    // these: FP32 NLS 64^2 9.8 -> 5.0 us, 128^2 x 8 11.5 -> 6.3,
-    // 256^2 x 8 13.6 -> 10.1, SG 256^2 x 8 on half spectra 24.9 -> 12.4;
-    // FP64 NLS 64^2 57.5 -> 13.3 us, 256^2 72 -> 26, SG 256^2 x 2 152 -> 31,
-    // NS 256^2 243 -> 102.  At 256 FP32, 8 points gain little more alone
-    // (NLS 256^2 7.9 -> 6.6 us) and lose 24 % at a batch of 32.
+    // FP64: short lines take fewer points per thread.  Their grids are mostly
+    // small, and a pass over them is bound by the two FP64 lanes of each SM in
+    // use and by the length of one thread's instruction chain, so the same
+    // points spread over more threads and SMs finish sooner.  `small` (variant
+    // 2): fields of at most SMALL_FIELD points, where that outweighs the extra
+    // stages; larger fields of short lines keep more points (fft
+    // 64 x 4096 x 8, 4 / 2 points: 274 / 300 us).  The choice depends on the
+    // grid alone, not on the batch, so that a batch rounds as its fields do
+    // alone.  Per step, from 16 points to these: NLS 64^2 57.5 -> 13.3 us,
+    // 256^2 72 -> 26, SG 256^2 x 2 on half spectra 152 -> 31, NS 256^2
+    // 243 -> 102; at 512 radix 8 three times instead of 16, 16, 2: one field
+    // 144 -> 99 us, four the same.  FP32 lines keep RP points: another
+    // factorisation rounds differently, which moves the conserved quantities
+    // of a small field by up to 1e-7.
+    static constexpr int SHORT = sizeof(Rl) == 4 ? 0 : 512;
     __host__ __device__ static constexpr int shortP(int n, bool small)
     {
-        if (sizeof(Rl) == 4) return n <= 16 ? 4 : n <= 64 || (n <= 128 && small) ? 8 : 16;
         if (small) return n <= 16 ? 4 : n <= 64 ? 2 : n <= 256 ? 4 : 8;
         return n <= 64 ? 4 : 8;
     }
-    // lines that take shortP points: up to 256 (FP32) and 512 (FP64; radix 8
-    // three times instead of 16, 16, 2: one 512^2 field 144 -> 99 us, four the same)
-    static constexpr int SHORT = sizeof(Rl) == 4 ? 256 : 512;
     __host__ __device__ static constexpr int rowP(int n, bool small = false)
     {
-        return n <= SHORT ? shortP(n, small) : n >= PSS_BIG_N ? RPB : RP;
+        return n <= SHORT ? shortP(n, small) : n < RP ? n : n >= PSS_BIG_N ? RPB : RP;
     }
     __host__ __device__ static constexpr int colP(int n, bool small = false)
     {
-        return n <= SHORT ? shortP(n, small) : n >= PSS_BIG_N ? CPB : CP;
+        return n <= SHORT ? shortP(n, small) : n < CP ? n : n >= PSS_BIG_N ? CPB : CP;
     }
     // columns per tile: 64-byte row segments (FP32) when the thread budget
     // (PSS_COL_THREADS) and shared memory (nbuf buffers) allow.  With `wide`,

@@ -1,6 +1,7 @@
-"""Short lines (up to 256 points, 512 in FP64) run with fewer points per thread,
-again fewer in small fields (at most 2^16 points): both sides of that line, the
-shortest lengths, and batches that do not fill a CTA, against the oracle."""
+"""Short FP64 lines (up to 512 points) run with fewer points per thread, again
+fewer in small fields (at most 2^16 points): both sides of that line, the
+shortest lengths, and batches that do not fill a CTA, against the oracle (FP32
+beside it)."""
 import math
 
 import numpy as np
