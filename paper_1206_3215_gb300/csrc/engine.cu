@@ -30,6 +30,22 @@ template <class Rl> const TW<Rl> *Tw(const void *p) { return static_cast<const T
 cudaMemcpyKind kind_in(int where) { return where == PSS_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice; }
 cudaMemcpyKind kind_out(int where) { return where == PSS_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice; }
 
+// whether a kernel may read or write a caller's device array directly: memory
+// of the current device (or managed), aligned for the kernel's widest access; anything
+// else goes through a copy, which reports what it cannot do
+bool kernel_access(const void *p, size_t align)
+{
+    if (reinterpret_cast<uintptr_t>(p) % align) return false;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    int dev = -1;
+    return cudaGetDevice(&dev) == cudaSuccess && at.device == dev &&
+           (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
+}
+
 // Upload a per-axis table of n complex values given by f(m) -> (re, im) in FP64,
 // in the twiddle layout of the grid's precision (FP32: hi + lo quadruples).
 template <class F> int upload_cplx_table(pss_grid *g, int64_t n, F f, void **dst)
@@ -140,6 +156,21 @@ int pss_grid::init()
         for (int64_t m = 0; m <= nx / 2; ++m) kh[m] = kx2v[m];
         if ((rc = p.precision == PSS_FP32 ? upload_real<float>(this, kh, &kx2h) : upload_real<double>(this, kh, &kx2h)))
             return rc;
+    }
+    if (p.eq == PSS_EQ_SG) {
+        // (dt^2/2) k^2 per axis, {hi, lo} in the grid's precision (start-up)
+        auto halves = [&](const std::vector<double> &k2, void **dst) {
+            std::vector<double> t(2 * k2.size());
+            std::vector<float> tf(2 * k2.size());
+            for (size_t m = 0; m < k2.size(); ++m) {
+                const double c = 0.5 * p.dt * p.dt * k2[m];
+                t[2 * m] = c;
+                tf[2 * m] = float(c);
+                tf[2 * m + 1] = float(c - double(float(c)));
+            }
+            return p.precision == PSS_FP32 ? upload(dst, tf.data(), tf.size() * 4) : upload(dst, t.data(), t.size() * 8);
+        };
+        if ((rc = halves(kx2v, &sgcx)) || (rc = halves(ky2v, &sgcy))) return rc;
     }
     if (p.eq == PSS_EQ_NLS) {
         // exp(-i k^2 tau) - 1 = (-2 sin^2(k^2 tau / 2), -sin(k^2 tau)) per axis,
@@ -440,13 +471,13 @@ template <class Rl> cudaError_t fft2(pss_grid *g, V2<Rl> *b, int dir)
 
 // real caller array (host or device) -> complex buffer dst (imaginary part 0),
 // through the raw scratch buffer `tmp`
-template <class Rl> int load_real(pss_grid *g, const void *src, int where, int tmp, int dst, bool apply_sin)
+template <class Rl> int load_real(pss_grid *g, const void *src, int where, int tmp, int dst)
 {
     const size_t bytes = size_t(g->ntot) * sizeof(Rl);
     int rc = g->cuda(cudaMemcpyAsync(g->buf[tmp], src, bytes, kind_in(where), g->stream), "state copy");
     if (rc) return rc;
-    return g->cuda(real_to_complex<Rl>(static_cast<const Rl *>(g->buf[tmp]), B<Rl>(g, dst), g->ntot, apply_sin,
-                                       g->stream), "real to complex");
+    return g->cuda(real_to_complex<Rl>(static_cast<const Rl *>(g->buf[tmp]), B<Rl>(g, dst), g->ntot, g->stream),
+                   "real to complex");
 }
 
 // Re(a - c b) of complex buffers into the caller array (through `tmp` for HOST)
@@ -477,24 +508,90 @@ int finish_sums(pss_grid *g)
 
 namespace {
 
-// H from uhat: the same scaling-then-transform as the fused column pass
-template <class Rl> int sg_make_h(pss_grid *g)
+// The state arrays of fields f .. f + nb - 1: the half spectra where the grid
+// steps those, else the full ones; w columns per row.
+template <class Rl> struct SgState {
+    V2<Rl> *u, *d, *h;
+    int64_t w, f, nb;
+};
+template <class Rl> SgState<Rl> sg_state(pss_grid *g, int64_t f, int64_t nb)
 {
-    const Rl s = Rl(1.0 / (double(g->nx) * double(g->ny)));  // power of two: exact before or after
-    int rc = g->cuda(cudaMemcpyAsync(g->buf[2], g->buf[0], g->field_bytes(), cudaMemcpyDeviceToDevice, g->stream),
-                     "copy");
-    if (rc) return rc;
-    return g->cuda(fft_cols<Rl>(B<Rl>(g, 2), g->nx, g->ny, g->batch, +1, s, Tw<Rl>(g->twy), g->stream), "H");
+    const int64_t w = g->half ? g->sx : g->nx, o = f * w * g->ny;
+    void *const *b = g->half ? g->hbuf : g->buf;
+    return {static_cast<V2<Rl> *>(b[0]) + o, static_cast<V2<Rl> *>(b[1]) + o, static_cast<V2<Rl> *>(b[2]) + o, w, f,
+            nb};
+}
+// scratch array i (3 or 4) of the fields, nb * npts complex points
+template <class Rl> V2<Rl> *sg_scratch(pss_grid *g, const SgState<Rl> &st, int i) { return B<Rl>(g, i) + st.f * g->npts; }
+
+template <class Rl> Rl sg_scale(pss_grid *g) { return Rl(1.0 / (double(g->nx) * double(g->ny))); }
+
+// H from uhat: the same scaling and transform as the step's column pass
+template <class Rl> int sg_make_h(pss_grid *g, const SgState<Rl> &st)
+{
+    return g->cuda(sg_level_cols<Rl>(st.u, nullptr, st.h, sg_scale<Rl>(g), st.w, g->ny, st.nb, Tw<Rl>(g->twy),
+                                     g->stream), "H");
+}
+
+// A caller's real array as the row kernels read it (pairs): the array itself
+// where it is device memory aligned for that, else a copy in `tmp`.
+template <class Rl> int sg_real_in(pss_grid *g, const void *src, int where, Rl *tmp, int64_t n, const Rl **out)
+{
+    if (where == PSS_DEVICE && kernel_access(src, 2 * sizeof(Rl))) {
+        *out = static_cast<const Rl *>(src);
+        return PSS_OK;
+    }
+    *out = tmp;
+    return g->cuda(cudaMemcpyAsync(tmp, src, size_t(n) * sizeof(Rl), kind_in(where), g->stream), "state copy");
+}
+
+// row transform of the real fields `a` into dst (rows of st.w)
+template <class Rl> cudaError_t sg_split(pss_grid *g, const SgState<Rl> &st, const Rl *a, V2<Rl> *dst)
+{
+    if (g->half && sizeof(Rl) == 8)  // FP32: see k_sg_io.cu
+        return sg_half_split<Rl>(a, dst, g->nx, g->sx, g->ny, st.nb, Tw<Rl>(g->twm), Tw<Rl>(g->twx), g->stream);
+    return rows_from_real<Rl>(a, dst, g->nx, g->half ? g->sx : 0, g->ny, st.nb, Tw<Rl>(g->twx), g->stream);
+}
+
+template <class Rl> int sg_set_fields(pss_grid *g, int64_t f, int64_t nb, const void *u0, const void *v0, int where)
+{
+    const SgState<Rl> st = sg_state<Rl>(g, f, nb);
+    const Rl *u = nullptr, *v = nullptr;
+    int rc;
+    if ((rc = sg_real_in<Rl>(g, u0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), nb * g->npts, &u)) ||
+        (v0 && (rc = sg_real_in<Rl>(g, v0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), nb * g->npts, &v))))
+        return rc;
+    cudaError_t e;
+    if (g->half) {
+        e = sg_half_start<Rl>(u, v, st.d, g->p.dt, g->nx, g->sx, g->ny, nb, Tw<Rl>(g->twm), Tw<Rl>(g->twx), g->stream);
+    } else {
+        e = sg_start_field<Rl>(u, v, st.d, g->p.dt, nb * g->npts, g->stream);
+        if (e == cudaSuccess)
+            e = fft_rows<Rl>(st.d, g->nx, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twx), g->stream);
+    }
+    if ((rc = g->cuda(e, "start-up rows")) || (rc = g->cuda(sg_split<Rl>(g, st, u, st.u), "forward rows")) ||
+        (rc = g->cuda(fft_cols<Rl>(st.u, st.w, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
+        (rc = g->cuda(sg_start_cols<Rl>(st.d, st.u, C<Rl>(g->sgcx), C<Rl>(g->sgcy), st.w, g->ny, nb, Tw<Rl>(g->twy),
+                                        g->stream), "start-up columns")) ||
+        (rc = sg_make_h<Rl>(g, st)))
+        return rc;
+    return where == PSS_HOST ? g->cuda(cudaStreamSynchronize(g->stream), "set_state sync") : PSS_OK;
 }
 
 // both levels from u^n, u^{n-1}: uhat^n = F u^n, d = uhat^n - F u^{n-1}
 template <class Rl> int sg_set_levels(pss_grid *g, const void *un, const void *unm1, int where)
 {
+    const SgState<Rl> st = sg_state<Rl>(g, 0, g->batch);
+    const Rl *a = nullptr, *b = nullptr;
     int rc;
-    if ((rc = load_real<Rl>(g, un, where, 3, 0, false)) || (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 0), -1), "forward")) ||
-        (rc = load_real<Rl>(g, unm1, where, 3, 1, false)) || (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 1), -1), "forward")) ||
-        (rc = g->cuda(cplx_axpy<Rl>(B<Rl>(g, 0), B<Rl>(g, 1), Rl(1), B<Rl>(g, 1), g->ntot, g->stream), "d")) ||
-        (rc = sg_make_h<Rl>(g)))
+    if ((rc = sg_real_in<Rl>(g, un, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), g->ntot, &a)) ||
+        (rc = sg_real_in<Rl>(g, unm1, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), g->ntot, &b)) ||
+        (rc = g->cuda(sg_split<Rl>(g, st, a, st.u), "forward rows")) ||
+        (rc = g->cuda(sg_split<Rl>(g, st, b, st.d), "forward rows")) ||
+        (rc = g->cuda(fft_cols<Rl>(st.u, st.w, g->ny, st.nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
+        (rc = g->cuda(fft_cols<Rl>(st.d, st.w, g->ny, st.nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
+        (rc = g->cuda(cplx_axpy<Rl>(st.u, st.d, Rl(1), st.d, st.w * g->ny * st.nb, g->stream), "d")) ||
+        (rc = sg_make_h<Rl>(g, st)))
         return rc;
     return where == PSS_HOST ? g->cuda(cudaStreamSynchronize(g->stream), "sync") : PSS_OK;
 }
@@ -503,43 +600,17 @@ template <class Rl> int sg_set_levels(pss_grid *g, const void *un, const void *u
 template <class Rl> int sg_half_sync(pss_grid *g, bool to_half)
 {
     int rc;
-    V2<Rl> *hu = static_cast<V2<Rl> *>(g->hbuf[0]), *hd = static_cast<V2<Rl> *>(g->hbuf[1]),
-           *hh = static_cast<V2<Rl> *>(g->hbuf[2]);
+    const SgState<Rl> st = sg_state<Rl>(g, 0, g->batch);
     if (to_half) {
-        const size_t hb = size_t(g->sx) * size_t(g->ny) * size_t(g->batch) * g->esz;
-        const Rl s = Rl(1.0 / (double(g->nx) * double(g->ny)));
-        if ((rc = g->cuda(pack_half<Rl>(B<Rl>(g, 0), hu, g->nx, g->ny, g->sx, g->batch, g->stream), "pack")) ||
-            (rc = g->cuda(pack_half<Rl>(B<Rl>(g, 1), hd, g->nx, g->ny, g->sx, g->batch, g->stream), "pack")) ||
-            (rc = g->cuda(cudaMemcpyAsync(hh, hu, hb, cudaMemcpyDeviceToDevice, g->stream), "copy")) ||
-            (rc = g->cuda(fft_cols<Rl>(hh, g->sx, g->ny, g->batch, +1, s, Tw<Rl>(g->twy), g->stream), "H")))
+        if ((rc = g->cuda(pack_half<Rl>(B<Rl>(g, 0), st.u, g->nx, g->ny, g->sx, g->batch, g->stream), "pack")) ||
+            (rc = g->cuda(pack_half<Rl>(B<Rl>(g, 1), st.d, g->nx, g->ny, g->sx, g->batch, g->stream), "pack")))
             return rc;
-        return PSS_OK;
+        return sg_make_h<Rl>(g, st);
     }
-    if ((rc = g->cuda(unpack_half<Rl>(hu, B<Rl>(g, 0), g->nx, g->ny, g->sx, g->batch, g->stream), "unpack")) ||
-        (rc = g->cuda(unpack_half<Rl>(hd, B<Rl>(g, 1), g->nx, g->ny, g->sx, g->batch, g->stream), "unpack")))
+    if ((rc = g->cuda(unpack_half<Rl>(st.u, B<Rl>(g, 0), g->nx, g->ny, g->sx, g->batch, g->stream), "unpack")) ||
+        (rc = g->cuda(unpack_half<Rl>(st.d, B<Rl>(g, 1), g->nx, g->ny, g->sx, g->batch, g->stream), "unpack")))
         return rc;
     return PSS_OK;
-}
-
-template <class Rl> int sg_set(pss_grid *g, const void *u0, const void *v0, int where)
-{
-    int rc;
-    if ((rc = load_real<Rl>(g, u0, where, 3, 0, false))) return rc;
-    if ((rc = g->cuda(real_to_complex<Rl>(static_cast<const Rl *>(g->buf[3]), B<Rl>(g, 2), g->ntot, true, g->stream),
-                      "sin u0")))
-        return rc;
-    if (v0) {
-        if ((rc = load_real<Rl>(g, v0, where, 3, 1, false))) return rc;
-    } else if ((rc = g->cuda(cudaMemsetAsync(g->buf[1], 0, g->field_bytes(), g->stream), "memset"))) {
-        return rc;
-    }
-    for (int b : {0, 1, 2})
-        if ((rc = g->cuda(fft2<Rl>(g, B<Rl>(g, b), -1), "forward transform"))) return rc;
-    if ((rc = g->cuda(sg_init<Rl>(B<Rl>(g, 0), B<Rl>(g, 1), B<Rl>(g, 2), g->kx2d, g->ky2d, g->p.dt, g->nx, g->ny,
-                                  g->batch, g->stream), "sg init")))
-        return rc;
-    if ((rc = sg_make_h<Rl>(g))) return rc;
-    return where == PSS_HOST ? g->cuda(cudaStreamSynchronize(g->stream), "sync") : PSS_OK;
 }
 
 template <class Rl> int sg_step(pss_grid *g, int64_t n)
@@ -572,35 +643,57 @@ template <class Rl> int sg_step(pss_grid *g, int64_t n)
     return PSS_OK;
 }
 
-// u^n -> a, u^{n-1} = Re F^-1 (uhat - d) -> b
-template <class Rl> int sg_get(pss_grid *g, void *a, void *b, int where)
+// real fields of the spectra a - b (b may be null) into dst: column pass into
+// scratch array 4, row pass into the real array
+template <class Rl>
+int sg_real_of(pss_grid *g, const SgState<Rl> &st, const V2<Rl> *a, const V2<Rl> *b, Rl *dst)
 {
-    int rc;
-    if ((rc = g->cuda(cudaMemcpyAsync(g->buf[3], g->buf[0], g->field_bytes(), cudaMemcpyDeviceToDevice, g->stream),
-                      "copy")) ||
-        (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 3), +1), "inverse")) ||
-        (rc = store_real<Rl>(g, B<Rl>(g, 3), nullptr, Rl(0), a, where, 4)))
-        return rc;
-    if (b) {
-        if ((rc = g->cuda(cplx_axpy<Rl>(B<Rl>(g, 0), B<Rl>(g, 1), Rl(1), B<Rl>(g, 3), g->ntot, g->stream), "axpy")) ||
-            (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 3), +1), "inverse")) ||
-            (rc = store_real<Rl>(g, B<Rl>(g, 3), nullptr, Rl(0), b, where, 4)))
-            return rc;
+    V2<Rl> *t = sg_scratch<Rl>(g, st, 4);
+    int rc = g->cuda(sg_level_cols<Rl>(a, b, t, sg_scale<Rl>(g), st.w, g->ny, st.nb, Tw<Rl>(g->twy), g->stream),
+                     "inverse columns");
+    if (rc) return rc;
+    return g->cuda(g->half ? sg_half_join<Rl>(t, dst, g->nx, g->sx, g->ny, st.nb, Tw<Rl>(g->twm), Tw<Rl>(g->twx),
+                                              g->stream)
+                           : rows_to_real<Rl>(t, dst, g->nx, g->ny, st.nb, Tw<Rl>(g->twx), g->stream),
+                   "inverse rows");
+}
+
+// u^n -> a, u^{n-1} = F^-1 (uhat - d) -> b (may be null) of fields f .. f + nb - 1
+template <class Rl> int sg_get_fields(pss_grid *g, int64_t f, int64_t nb, void *a, void *b, int where)
+{
+    const SgState<Rl> st = sg_state<Rl>(g, f, nb);
+    void *const dst[2] = {a, b};
+    for (int k = 0; k < 2; ++k) {
+        if (!dst[k]) continue;
+        const bool direct = where == PSS_DEVICE && kernel_access(dst[k], 2 * sizeof(Rl));
+        Rl *r = direct ? static_cast<Rl *>(dst[k]) : reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3));
+        int rc = sg_real_of<Rl>(g, st, st.u, k ? st.d : nullptr, r);
+        if (!rc && !direct)
+            rc = g->cuda(cudaMemcpyAsync(dst[k], r, size_t(nb) * g->npts * sizeof(Rl), kind_out(where), g->stream),
+                         "state copy");
+        if (rc) return rc;
     }
     return g->sync();
 }
 
 template <class Rl> int sg_conserved(pss_grid *g, double *out)
 {
+    const SgState<Rl> st = sg_state<Rl>(g, 0, g->batch);
+    Rl *X = reinterpret_cast<Rl *>(g->buf[3]), *Y = X + g->ntot;  // u^n, u^n - u^{n-1}
     int rc;
-    for (int k : {0, 1}) {
-        if ((rc = g->cuda(cudaMemcpyAsync(g->buf[3 + k], g->buf[k], g->field_bytes(), cudaMemcpyDeviceToDevice,
-                                          g->stream), "copy")) ||
-            (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 3 + k), +1), "inverse")))
+    for (int k = 0; k < 2; ++k) {
+        const V2<Rl> *src = k ? st.d : st.u;
+        if (sizeof(Rl) == 8) {
+            if ((rc = sg_real_of<Rl>(g, st, src, nullptr, k ? Y : X))) return rc;
+        } else if ((rc = g->cuda(rows_inverse<Rl>(src, B<Rl>(g, 4), g->nx, g->half ? g->sx : 0, g->ny, g->batch,
+                                                  Tw<Rl>(g->twx), g->stream), "inverse rows")) ||
+                   (rc = g->cuda(cols_to_real<Rl>(B<Rl>(g, 4), k ? Y : X, sg_scale<Rl>(g), g->nx, g->ny, g->batch,
+                                                  Tw<Rl>(g->twy), g->stream), "inverse columns"))) {
             return rc;
+        }
     }
-    if ((rc = g->cuda(sg_sums<Rl>(B<Rl>(g, 3), B<Rl>(g, 4), B<Rl>(g, 0), B<Rl>(g, 1), g->nx, g->ny, g->batch, g->kx2d,
-                                  g->ky2d, g->p.dt, g->partials, g->sums, g->stream), "sg sums")) ||
+    if ((rc = g->cuda(sg_sums<Rl>(X, Y, st.u, st.d, g->nx, g->ny, st.w, g->batch, g->kx2d, g->ky2d, g->p.dt,
+                                  g->partials, g->sums, g->stream), "sg sums")) ||
         (rc = finish_sums(g)))
         return rc;
     const double dA = g->dA(), inv_n = 1.0 / (double(g->nx) * double(g->ny));
@@ -678,7 +771,7 @@ template <class Rl> int ns_step_begin(pss_grid *g)
 template <class Rl> int ns_set(pss_grid *g, const void *w0, int where)
 {
     int rc;
-    if ((rc = load_real<Rl>(g, w0, where, 6, 0, false)) || (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 0), -1), "forward")) ||
+    if ((rc = load_real<Rl>(g, w0, where, 6, 0)) || (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 0), -1), "forward")) ||
         (rc = g->cuda(apply_mask<Rl>(B<Rl>(g, 0), Rt<Rl>(g->keepx), Rt<Rl>(g->keepy), g->nx, g->ny, g->batch, g->stream),
                       "mask")) ||
         (rc = g->cuda(cudaMemsetAsync(g->ns_field, 0, size_t(g->batch) * ns_field_bytes(), g->stream), "memset")) ||
@@ -858,12 +951,12 @@ template <class Rl> cudaError_t fft2_one(pss_grid *g, V2<Rl> *b, int dir)
 
 // real field (host or device) -> complex slot dst_buf[f], through raw scratch slot tmp_buf[f]
 template <class Rl>
-int load_real_one(pss_grid *g, int64_t f, const void *src, int where, int tmp, int dst, bool apply_sin)
+int load_real_one(pss_grid *g, int64_t f, const void *src, int where, int tmp, int dst)
 {
     Rl *t = reinterpret_cast<Rl *>(Bf<Rl>(g, tmp, f));
     int rc = g->cuda(cudaMemcpyAsync(t, src, size_t(g->npts) * sizeof(Rl), kind_in(where), g->stream), "copy");
     if (rc) return rc;
-    return g->cuda(real_to_complex<Rl>(t, Bf<Rl>(g, dst, f), g->npts, apply_sin, g->stream), "real to complex");
+    return g->cuda(real_to_complex<Rl>(t, Bf<Rl>(g, dst, f), g->npts, g->stream), "real to complex");
 }
 
 template <class Rl> int store_real_one(pss_grid *g, int64_t f, const V2<Rl> *a, void *dst, int where, int tmp)
@@ -883,27 +976,12 @@ template <class Rl> int field_set(pss_grid *g, int64_t f, const void *a, const v
             (rc = g->cuda(fft_rows<Rl>(Bf<Rl>(g, 0, f), g->nx, g->ny, 1, -1, Rl(1), Tw<Rl>(g->twx), g->stream), "row fft")))
             return rc;
     } else if (g->p.eq == PSS_EQ_SG) {
-        if ((rc = load_real_one<Rl>(g, f, a, where, 3, 0, false)) ||
-            (rc = g->cuda(real_to_complex<Rl>(reinterpret_cast<Rl *>(Bf<Rl>(g, 3, f)), Bf<Rl>(g, 2, f), g->npts, true,
-                                              g->stream), "sin")))
-            return rc;
-        if (b) rc = load_real_one<Rl>(g, f, b, where, 3, 1, false);
-        else rc = g->cuda(cudaMemsetAsync(Bf<Rl>(g, 1, f), 0, fb, g->stream), "memset");
-        if (rc) return rc;
-        for (int i : {0, 1, 2})
-            if ((rc = g->cuda(fft2_one<Rl>(g, Bf<Rl>(g, i, f), -1), "forward"))) return rc;
-        const Rl s = Rl(1.0 / (double(g->nx) * double(g->ny)));
-        if ((rc = g->cuda(sg_init<Rl>(Bf<Rl>(g, 0, f), Bf<Rl>(g, 1, f), Bf<Rl>(g, 2, f), g->kx2d, g->ky2d, g->p.dt,
-                                      g->nx, g->ny, 1, g->stream), "sg init")) ||
-            (rc = g->cuda(cudaMemcpyAsync(Bf<Rl>(g, 2, f), Bf<Rl>(g, 0, f), fb, cudaMemcpyDeviceToDevice, g->stream),
-                          "copy")) ||
-            (rc = g->cuda(fft_cols<Rl>(Bf<Rl>(g, 2, f), g->nx, g->ny, 1, +1, s, Tw<Rl>(g->twy), g->stream), "H")))
-            return rc;
+        return sg_set_fields<Rl>(g, f, 1, a, b, where);
     } else {
         // full spectrum of the field in buf[6] (half spectra) or buf[0], then
         // (half spectra) into the field's slot of the half-width buffer 0
         const int dst = g->ns_half ? 6 : 0;
-        if ((rc = load_real_one<Rl>(g, f, a, where, g->ns_half ? 3 : 6, dst, false)) ||
+        if ((rc = load_real_one<Rl>(g, f, a, where, g->ns_half ? 3 : 6, dst)) ||
             (rc = g->cuda(fft2_one<Rl>(g, Bf<Rl>(g, dst, f), -1), "forward")) ||
             (rc = g->cuda(apply_mask<Rl>(Bf<Rl>(g, dst, f), Rt<Rl>(g->keepx), Rt<Rl>(g->keepy), g->nx, g->ny, 1,
                                          g->stream), "mask")) ||
@@ -928,16 +1006,7 @@ template <class Rl> int field_get(pss_grid *g, int64_t f, void *a, void *b, int 
             (rc = g->cuda(cudaMemcpyAsync(a, Bf<Rl>(g, 1, f), fb, kind_out(where), g->stream), "copy")))
             return rc;
     } else if (g->p.eq == PSS_EQ_SG) {
-        if ((rc = g->cuda(cudaMemcpyAsync(Bf<Rl>(g, 3, f), Bf<Rl>(g, 0, f), fb, cudaMemcpyDeviceToDevice, g->stream),
-                          "copy")) ||
-            (rc = g->cuda(fft2_one<Rl>(g, Bf<Rl>(g, 3, f), +1), "inverse")) ||
-            (rc = store_real_one<Rl>(g, f, Bf<Rl>(g, 3, f), a, where, 4)))
-            return rc;
-        if (b && ((rc = g->cuda(cplx_axpy<Rl>(Bf<Rl>(g, 0, f), Bf<Rl>(g, 1, f), Rl(1), Bf<Rl>(g, 3, f), g->npts,
-                                              g->stream), "axpy")) ||
-                  (rc = g->cuda(fft2_one<Rl>(g, Bf<Rl>(g, 3, f), +1), "inverse")) ||
-                  (rc = store_real_one<Rl>(g, f, Bf<Rl>(g, 3, f), b, where, 4))))
-            return rc;
+        return sg_get_fields<Rl>(g, f, 1, a, b, where);
     } else {
         V2<Rl> *w[3];
         for (int i = 0; i < 3; ++i) w[i] = B<Rl>(g, i) + ns_off(g, f);  // field f's slot of each vorticity buffer
@@ -970,7 +1039,7 @@ int pss_grid::set_state(const void *a, const void *b, int where)
     nonconv_pending = false;
     int rc;
 #define NLS(R) nls_set<R>(this, a, where)
-#define SG(R) sg_set<R>(this, a, b, where)
+#define SG(R) sg_set_fields<R>(this, 0, batch, a, b, where)
 #define NS(R) ns_set<R>(this, a, where)
     rc = p.eq == PSS_EQ_NLS ? PSS_BY_PRECISION(NLS) : p.eq == PSS_EQ_SG ? PSS_BY_PRECISION(SG) : PSS_BY_PRECISION(NS);
 #undef NLS
@@ -978,8 +1047,8 @@ int pss_grid::set_state(const void *a, const void *b, int where)
 #undef NS
     if (!rc) {
         has_state = true;
-        full_valid = true;
-        half_valid = false;
+        full_valid = !half;
+        half_valid = half;
     }
     return rc;
 }
@@ -991,8 +1060,8 @@ int pss_grid::set_sg_levels(const void *u_n, const void *u_nm1, int where)
     if (rc) return rc;
     steps = 0;
     has_state = true;
-    full_valid = true;
-    half_valid = false;
+    full_valid = !half;
+    half_valid = half;
     return PSS_OK;
 }
 
@@ -1093,10 +1162,10 @@ int pss_grid::step_n(int64_t n)
 
 int pss_grid::get_state(void *a, void *b, int where)
 {
-    int rc = half_sync(false);
+    int rc = half_sync(true);
     if (rc) return rc;
 #define NLS(R) nls_get<R>(this, a, where)
-#define SG(R) sg_get<R>(this, a, b, where)
+#define SG(R) sg_get_fields<R>(this, 0, batch, a, b, where)
 #define NS(R) ns_get<R>(this, a, where)
     return p.eq == PSS_EQ_NLS ? PSS_BY_PRECISION(NLS) : p.eq == PSS_EQ_SG ? PSS_BY_PRECISION(SG) : PSS_BY_PRECISION(NS);
 #undef NLS
@@ -1106,26 +1175,24 @@ int pss_grid::get_state(void *a, void *b, int where)
 
 int pss_grid::set_field(int64_t f, const void *a, const void *b, int where)
 {
-    int rc = half_sync(false);  // the other fields' full state must be current
+    int rc = half_sync(true);  // the other fields' state must be current
     if (rc) return rc;
+    if (half) full_valid = false;
     rc = p.precision == PSS_FP32 ? field_set<float>(this, f, a, b, where) : field_set<double>(this, f, a, b, where);
-    if (!rc) {
-        has_state = true;
-        half_valid = false;
-    }
+    if (!rc) has_state = true;
     return rc;
 }
 
 int pss_grid::get_field(int64_t f, void *a, void *b, int where)
 {
-    int rc = half_sync(false);
+    int rc = half_sync(true);
     if (rc) return rc;
     return p.precision == PSS_FP32 ? field_get<float>(this, f, a, b, where) : field_get<double>(this, f, a, b, where);
 }
 
 int pss_grid::conserved(double *out)
 {
-    int rc = half_sync(false);
+    int rc = half_sync(true);
     if (rc) return rc;
 #define NLS(R) nls_conserved<R>(this, out)
 #define SG(R) sg_conserved<R>(this, out)
@@ -1178,7 +1245,9 @@ int pss_grid::checkpoint(void *buf_, int where, bool save)
     if (!save) {
         steps = meta[0];
         if (p.eq == PSS_EQ_SG) {
-            rc = p.precision == PSS_FP32 ? sg_make_h<float>(this) : sg_make_h<double>(this);
+            if (!half)  // half spectra: the next use packs them and makes H
+                rc = p.precision == PSS_FP32 ? sg_make_h<float>(this, sg_state<float>(this, 0, batch))
+                                             : sg_make_h<double>(this, sg_state<double>(this, 0, batch));
         } else if (p.eq == PSS_EQ_NS) {
             // all fields restart from buffer 0 with their update count
             NsFieldHost *h = static_cast<NsFieldHost *>(host_fields);

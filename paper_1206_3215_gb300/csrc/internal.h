@@ -60,6 +60,45 @@ cudaError_t sg_col_pass(V2<Rl> *h, V2<Rl> *u, V2<Rl> *d, int64_t nx, int64_t ny,
 template <class Rl>
 cudaError_t sg_row_pass_r2c(V2<Rl> *h, int64_t nx, int64_t sx, int64_t ny, int64_t batch, const TW<Rl> *twm,
                             const TW<Rl> *twn, cudaStream_t s);
+// Real rows and half spectra (k_sg_io.cu): row transform of a into h; of
+// dt v + (dt^2/2) sin u (v may be null) into h; inverse row transform of h into out.
+template <class Rl>
+cudaError_t sg_half_split(const Rl *a, V2<Rl> *h, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
+                          const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s);
+template <class Rl>
+cudaError_t sg_half_start(const Rl *u, const Rl *v, V2<Rl> *h, double dt, int64_t nx, int64_t sx, int64_t ny,
+                          int64_t batch, const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s);
+template <class Rl>
+cudaError_t sg_half_join(const V2<Rl> *h, Rl *out, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
+                         const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s);
+// dt v + (dt^2/2) sin u as a complex array of n points (full spectra).
+template <class Rl>
+cudaError_t sg_start_field(const Rl *u, const Rl *v, V2<Rl> *dst, double dt, int64_t n, cudaStream_t s);
+// Complex transforms between real arrays and spectra, sx = 0: full spectra,
+// sx > 0: half spectra in rows of sx.  Row transform of real rows; inverse row
+// transform into full complex rows; real parts of an inverse row transform, or
+// of an inverse column transform times scale, into real arrays.
+template <class Rl>
+cudaError_t rows_from_real(const Rl *src, V2<Rl> *dst, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
+                           const TW<Rl> *twx, cudaStream_t s);
+template <class Rl>
+cudaError_t rows_inverse(const V2<Rl> *src, V2<Rl> *dst, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
+                         const TW<Rl> *twx, cudaStream_t s);
+template <class Rl>
+cudaError_t rows_to_real(const V2<Rl> *src, Rl *dst, int64_t nx, int64_t ny, int64_t batch, const TW<Rl> *twx,
+                         cudaStream_t s);
+template <class Rl>
+cudaError_t cols_to_real(const V2<Rl> *src, Rl *dst, Rl scale, int64_t nx, int64_t ny, int64_t batch,
+                         const TW<Rl> *twy, cudaStream_t s);
+// Columns of width nx, full or half: out = scale * inverse transform of a - b
+// (b may be null); data = transform of data + (dt^2/2) |k|^2 u, cx and cy
+// holding (dt^2/2) k^2 per axis as {hi, lo}.
+template <class Rl>
+cudaError_t sg_level_cols(const V2<Rl> *a, const V2<Rl> *b, V2<Rl> *out, Rl scale, int64_t nx, int64_t ny,
+                          int64_t batch, const TW<Rl> *twy, cudaStream_t s);
+template <class Rl>
+cudaError_t sg_start_cols(V2<Rl> *data, const V2<Rl> *u, const V2<Rl> *cx, const V2<Rl> *cy, int64_t nx, int64_t ny,
+                          int64_t batch, const TW<Rl> *twy, cudaStream_t s);
 // full [batch][ny][nx] spectrum of real fields <-> half spectrum [batch][ny][sx]
 template <class Rl>
 cudaError_t pack_half(const V2<Rl> *full, V2<Rl> *half, int64_t nx, int64_t ny, int64_t sx, int64_t batch,
@@ -91,12 +130,9 @@ cudaError_t ns_decide(void *fs, const double *partials, int64_t groups, int64_t 
 cudaError_t ns_advance(int *ctl, bool use_graph, cudaGraphConditionalHandle h, cudaStream_t s);
 
 // ---- elementwise helpers (k_util.cu) ----------------------------------------
-template <class Rl> cudaError_t real_to_complex(const Rl *src, V2<Rl> *dst, int64_t n, bool apply_sin, cudaStream_t s);
+template <class Rl> cudaError_t real_to_complex(const Rl *src, V2<Rl> *dst, int64_t n, cudaStream_t s);
 template <class Rl>
 cudaError_t complex_to_real(const V2<Rl> *a, const V2<Rl> *b, Rl c, Rl *dst, int64_t n, cudaStream_t s);
-template <class Rl>
-cudaError_t sg_init(const V2<Rl> *u, V2<Rl> *d, const V2<Rl> *sn, const double *kx2, const double *ky2, double dt,
-                    int64_t nx, int64_t ny, int64_t batch, cudaStream_t s);
 template <class Rl>
 cudaError_t ns_gather(const void *fs, V2<Rl> *const w[3], V2<Rl> *dst, int64_t per_field, int64_t batch,
                       cudaStream_t s);
@@ -118,9 +154,11 @@ cudaError_t nls_sums(const V2<Rl> *psi, const V2<Rl> *psi_hat, int64_t nx, int64
 // message returned by pss_last_error(NULL) for calls without a grid handle
 void set_global_error(const char *msg);
 
-// SG: per field {sum (Y/dt)^2/2, sum 1 - cos(X - Y/2), sum |k|^2 |U - D/2|^2}
+// SG: per field {sum (Y/dt)^2/2, sum 1 - cos(X - Y/2), sum |k|^2 |U - D/2|^2};
+// X, Y real fields, U, D spectra with rows of w columns: w = nx, or (half
+// spectra) w > nx/2, columns 0 .. nx/2 standing for both halves
 template <class Rl>
-cudaError_t sg_sums(const V2<Rl> *X, const V2<Rl> *Y, const V2<Rl> *U, const V2<Rl> *D, int64_t nx, int64_t ny,
+cudaError_t sg_sums(const Rl *X, const Rl *Y, const V2<Rl> *U, const V2<Rl> *D, int64_t nx, int64_t ny, int64_t w,
                     int64_t batch, const double *kx2, const double *ky2, double dt, double *partials, double *out,
                     cudaStream_t s);
 // NS: per field {Re w_hat(0,0), sum |w_hat|^2, sum_{k != 0} |w_hat|^2 / |k|^2}

@@ -85,28 +85,60 @@ cudaError_t nls_sums(const V2<Rl> *psi, const V2<Rl> *psi_hat, int64_t nx, int64
     return cudaGetLastError();
 }
 
-// SG at t_{n-1/2}: X = u^n, Y = u^n - u^{n-1} (physical, real parts), U = uhat^n,
-// D = uhat^n - uhat^{n-1}.  Sums: (Y/dt)^2 / 2, 1 - cos(ubar) = 2 sin^2(ubar/2)
-// with ubar = X - Y/2, and |k|^2 |U - D/2|^2 (the spectrum of ubar).
+// 1 - cos x without cancellation: for |x| <= 1 its Taylor series in x^2 (the
+// first omitted term, x^20/20!, is below 1e-18 of the sum), else 2 sin^2(x/2)
+__device__ __forceinline__ double one_minus_cos(double x)
+{
+    if ((__double2hiint(x) & 0x7fffffff) < 0x3ff00000) {
+        const double t = x * x;
+        double p = 1.0 / 6402373705728000.0;
+        p = fma(-t, p, 1.0 / 20922789888000.0);
+        p = fma(-t, p, 1.0 / 87178291200.0);
+        p = fma(-t, p, 1.0 / 479001600.0);
+        p = fma(-t, p, 1.0 / 3628800.0);
+        p = fma(-t, p, 1.0 / 40320.0);
+        p = fma(-t, p, 1.0 / 720.0);
+        p = fma(-t, p, 1.0 / 24.0);
+        return t * fma(-t, p, 0.5);
+    }
+    const double s = sin(0.5 * x);
+    return 2.0 * s * s;
+}
+
+// SG at t_{n-1/2}: X = u^n, Y = u^n - u^{n-1} (real fields), U = uhat^n,
+// D = uhat^n - uhat^{n-1}.  Sums: (Y/dt)^2 / 2, 1 - cos(ubar) with
+// ubar = X - Y/2, and |k|^2 |U - D/2|^2 (the spectrum of ubar), over half
+// spectra where w < nx (columns 0 and nx/2 once, those between them twice).
+// Bound by the FP64 lanes (two per SM): the division by dt is taken out of
+// the sum and 1 - cos is a polynomial where it may be; with real fields and
+// half spectra 2048^2 x 8 takes 0.9 ms (2.85 ms with complex fields, full
+// spectra, a division and a sine per point).
 template <class Rl>
 __global__ void __launch_bounds__(RED_THREADS)
-    k_sg_sums(const V2<Rl> *X, const V2<Rl> *Y, const V2<Rl> *U, const V2<Rl> *D, int64_t nx, int64_t ny,
-              const double *kx2, const double *ky2, double dt, double *partials)
+    k_sg_sums(const Rl *__restrict__ X, const Rl *__restrict__ Y, const V2<Rl> *__restrict__ U,
+              const V2<Rl> *__restrict__ D, int64_t nx, int64_t ny, int64_t w, const double *__restrict__ kx2,
+              const double *__restrict__ ky2, double half_dt2inv, double *partials)
 {
     __shared__ double sh[3 * RED_THREADS];
-    const int64_t f = blockIdx.y, n = nx * ny, o = f * n;
-    const int lgx = __ffsll(nx) - 1;  // nx is a power of two
+    const int64_t f = blockIdx.y, n = nx * ny, o = f * n, ns = w * ny, os = f * ns;
     double a[3] = {0.0, 0.0, 0.0};
-    for (int64_t i = int64_t(blockIdx.x) * RED_THREADS + threadIdx.x; i < n;
-         i += int64_t(RED_BLOCKS) * RED_THREADS) {
-        const double du = double(Y[o + i].x), ub = double(X[o + i].x) - 0.5 * du;
-        const double sh2 = sin(0.5 * ub);
-        a[0] += 0.5 * (du / dt) * (du / dt);
-        a[1] += 2.0 * sh2 * sh2;
-        const V2<Rl> u = U[o + i], d = D[o + i];
-        const double br = double(u.x) - 0.5 * double(d.x), bi = double(u.y) - 0.5 * double(d.y);
-        a[2] += (kx2[i & (nx - 1)] + ky2[i >> lgx]) * (br * br + bi * bi);
+#pragma unroll 4
+    for (int64_t i = int64_t(blockIdx.x) * RED_THREADS + threadIdx.x; i < n; i += int64_t(RED_BLOCKS) * RED_THREADS) {
+        const double du = double(Y[o + i]);
+        a[0] = fma(du, du, a[0]);
+        a[1] += one_minus_cos(fma(-0.5, du, double(X[o + i])));
     }
+    const unsigned uw = unsigned(w), mid = unsigned(nx / 2);
+#pragma unroll 4
+    for (unsigned i = blockIdx.x * RED_THREADS + threadIdx.x; i < unsigned(ns); i += RED_BLOCKS * RED_THREADS) {
+        const unsigned y = i / uw, x = i - y * uw;
+        if (w < nx && x > mid) continue;  // padding of half spectra
+        const V2<Rl> u = U[os + i], d = D[os + i];
+        const double br = fma(-0.5, double(d.x), double(u.x)), bi = fma(-0.5, double(d.y), double(u.y));
+        const double e = (kx2[x] + ky2[y]) * fma(br, br, bi * bi);
+        a[2] += w < nx && x != 0 && x != mid ? 2.0 * e : e;
+    }
+    a[0] *= half_dt2inv;
     block_sum<3>(a, sh);
     if (threadIdx.x == 0)
 #pragma unroll
@@ -146,12 +178,12 @@ __global__ void __launch_bounds__(RED_THREADS)
 }
 
 template <class Rl>
-cudaError_t sg_sums(const V2<Rl> *X, const V2<Rl> *Y, const V2<Rl> *U, const V2<Rl> *D, int64_t nx, int64_t ny,
+cudaError_t sg_sums(const Rl *X, const Rl *Y, const V2<Rl> *U, const V2<Rl> *D, int64_t nx, int64_t ny, int64_t w,
                     int64_t batch, const double *kx2, const double *ky2, double dt, double *partials, double *out,
                     cudaStream_t s)
 {
-    k_sg_sums<Rl><<<dim3(RED_BLOCKS, unsigned(batch)), RED_THREADS, 0, s>>>(X, Y, U, D, nx, ny, kx2, ky2, dt,
-                                                                           partials);
+    k_sg_sums<Rl><<<dim3(RED_BLOCKS, unsigned(batch)), RED_THREADS, 0, s>>>(X, Y, U, D, nx, ny, w, kx2, ky2,
+                                                                           0.5 / (dt * dt), partials);
     k_fold<3><<<unsigned(batch), RED_THREADS, 0, s>>>(partials, out);
     return cudaGetLastError();
 }
@@ -166,11 +198,11 @@ cudaError_t ns_sums(const void *fs, V2<Rl> *const w[3], int64_t nx, int64_t ny, 
     return cudaGetLastError();
 }
 
-template cudaError_t sg_sums<float>(const float2 *, const float2 *, const float2 *, const float2 *, int64_t,
+template cudaError_t sg_sums<float>(const float *, const float *, const float2 *, const float2 *, int64_t, int64_t,
                                     int64_t, int64_t, const double *, const double *, double, double *, double *,
                                     cudaStream_t);
-template cudaError_t sg_sums<double>(const double2 *, const double2 *, const double2 *, const double2 *, int64_t,
-                                     int64_t, int64_t, const double *, const double *, double, double *,
+template cudaError_t sg_sums<double>(const double *, const double *, const double2 *, const double2 *, int64_t,
+                                     int64_t, int64_t, int64_t, const double *, const double *, double, double *,
                                      double *, cudaStream_t);
 template cudaError_t ns_sums<float>(const void *, float2 *const[3], int64_t, int64_t, int64_t, const double *,
                                     const double *, double *, double *, cudaStream_t);

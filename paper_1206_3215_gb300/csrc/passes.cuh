@@ -184,16 +184,6 @@ template <class Rl> __host__ __device__ constexpr bool short_variant(int n)
 {
     return Shape<Rl>::rowP(n, true) != Shape<Rl>::rowP(n, false);
 }
-// resident CTAs per SM a pass budgets its registers for (LEAN ops; else 1):
-// VS::CTAS, fewer where those exceed VS::TPS threads (512: 128 registers each);
-// the small CTAs of short FP32 lines as many (up to 16) as fill VS::TPS threads
-template <class Rl, int VAR> __host__ __device__ constexpr int lean_ctas(bool lean, int threads, int n)
-{
-    using VS = VarShape<Rl, VAR>;
-    const int fit = imax(VS::TPS / threads, 1);
-    if (!lean) return 1;
-    return sizeof(Rl) == 4 && n <= 256 ? imin(imax(VS::CTAS, fit), 16) : imin(VS::CTAS, fit);
-}
 
 // dynamic shared memory a pass may use per CTA (the GB300 limit is 227 KB)
 constexpr size_t SMEM_LIMIT = 200 * 1024;
@@ -246,7 +236,10 @@ template <class Rl, int N, int NIN, bool LEAN = false, int PMAX = 32, int VAR = 
     static constexpr int MAXB = LEAN ? Shape<Rl>::MAX_NBUF : 2;
     static constexpr int NBUF = (MAXB > 1 && size_t(2) * BUF * Shape<Rl>::ESZ <= SMEM_LIMIT) ? 2 : 1;
     static constexpr size_t SMEM = size_t(NBUF) * BUF * Shape<Rl>::ESZ;
-    static constexpr int MIN_CTAS = lean_ctas<Rl, VAR>(LEAN, THREADS, N);
+    // resident CTAs the registers are budgeted for: at most VS::TPS threads
+    // per SM (512: 128 registers each)
+    static constexpr int MIN_CTAS =
+        LEAN ? (THREADS * VS::CTAS <= VS::TPS ? VS::CTAS : (VS::TPS / THREADS > 1 ? VS::TPS / THREADS : 1)) : 1;
 };
 
 template <class Rl, int N, int NIN, bool LEAN = false, int PMAX = 32, int VAR = 0> struct ColCfg {
@@ -263,7 +256,10 @@ template <class Rl, int N, int NIN, bool LEAN = false, int PMAX = 32, int VAR = 
     static constexpr int MAXB = LEAN ? Shape<Rl>::MAX_NBUF : 2;
     static constexpr int NBUF = (MAXB > 1 && size_t(2) * BUF * Shape<Rl>::ESZ <= SMEM_LIMIT) ? 2 : 1;
     static constexpr size_t SMEM = size_t(NBUF) * BUF * Shape<Rl>::ESZ;
-    static constexpr int MIN_CTAS = lean_ctas<Rl, VAR>(LEAN, THREADS, N);
+    // resident CTAs the registers are budgeted for: at most VS::TPS threads
+    // per SM (512: 128 registers each)
+    static constexpr int MIN_CTAS =
+        LEAN ? (THREADS * VS::CTAS <= VS::TPS ? VS::CTAS : (VS::TPS / THREADS > 1 ? VS::TPS / THREADS : 1)) : 1;
 };
 
 // points per thread an op allows at length N: Op::pmax(N) where the op
@@ -338,6 +334,13 @@ template <class Op, class = void> struct EarlyNext : std::false_type {};
 template <class Op>
 struct EarlyNext<Op, std::void_t<decltype(Op::EARLY_NEXT)>> : std::integral_constant<bool, Op::EARLY_NEXT> {};
 
+// An op that sets DIRECT_LOAD reads its rows itself (op.load<N, P>(v, row, ok,
+// t): register m = element t + T m) instead of having them staged: rows that
+// are not complex arrays, or that one thread gathers from two places.
+template <class Op, class = void> struct DirectLoad : std::false_type {};
+template <class Op>
+struct DirectLoad<Op, std::void_t<decltype(Op::DIRECT_LOAD)>> : std::integral_constant<bool, Op::DIRECT_LOAD> {};
+
 // rows_total = batch * ny; row r of the batch starts at element r * NX
 template <class Rl, int N, class Op, int VAR>
 __global__ void __launch_bounds__(RowCfgOf<Rl, N, Op, VAR>::THREADS, RowCfgOf<Rl, N, Op, VAR>::MIN_CTAS)
@@ -353,12 +356,15 @@ __global__ void __launch_bounds__(RowCfgOf<Rl, N, Op, VAR>::THREADS, RowCfgOf<Rl
     const int64_t tiles = (rows_total + C::ROWS - 1) / C::ROWS;
 
     auto line = [&](int b, int k) { return Sm{buf + b * C::BUF + (k * C::ROWS + lr) * C::LINE}; };
+    constexpr bool DIRECT = DirectLoad<Op>::value;
     auto issue = [&](int64_t tile, int b) {
-        const int64_t row = tile * C::ROWS + lr;
-        if (tile < tiles && row < rows_total)
+        if constexpr (!DIRECT) {
+            const int64_t row = tile * C::ROWS + lr;
+            if (tile < tiles && row < rows_total)
 #pragma unroll
-            for (int k = 0; k < NIN; ++k) stage_line<C::P, C::T>(line(b, k), op.in(k) + row * N, 1, t);
-        cp_async_commit();
+                for (int k = 0; k < NIN; ++k) stage_line<C::P, C::T>(line(b, k), op.in(k) + row * N, 1, t);
+            cp_async_commit();
+        }
     };
 
     constexpr bool EARLY = EarlyNext<Op>::value && C::NBUF == 1;
@@ -385,8 +391,9 @@ __global__ void __launch_bounds__(RowCfgOf<Rl, N, Op, VAR>::THREADS, RowCfgOf<Rl
 #pragma unroll
         for (int k = 0; k < NIN; ++k) {
             sm[k] = line(b, k);
-            read_line<C::P, C::T>(v[k], sm[k], t);
+            if constexpr (!DIRECT) read_line<C::P, C::T>(v[k], sm[k], t);
         }
+        if constexpr (DIRECT) op.template load<N, C::P>(v[0], row, row < rows_total, t);
         if constexpr (EARLY) {
             const int64_t next = tile + gridDim.x;
             if (PSS_ROW_PREFETCH && t == 0 && next < tiles && next * C::ROWS + lr < rows_total)
