@@ -309,8 +309,9 @@ int pss_grid::profile_resolve()
 
 // per-field fixed-point record as written by the NS kernels
 struct NsFieldHost {
-    int idx, active, nonconv, pad;
+    int idx, active, nonconv, k;
     long long updates;
+    int left, pad;
 };
 
 int pss_grid::ns_update_count(int64_t *n)
@@ -730,7 +731,8 @@ template <class Rl> int ns_prep(pss_grid *g, bool per_step = false)
     ns_w<Rl>(g, w);
     return g->cuda(ns_prep_pass<Rl>(w, per_step ? g->ns_field : nullptr, B<Rl>(g, 4), B<Rl>(g, 5), Rt<Rl>(g->kxo),
                                     Rt<Rl>(g->kyo), Rt<Rl>(g->kx2), Rt<Rl>(g->ky2), g->nx, g->ny, g->batch,
-                                    Tw<Rl>(g->twy), g->stream, g->ns_half ? g->nsx : 0), "ns derivatives");
+                                    reinterpret_cast<int *>(g->flags), Tw<Rl>(g->twy), g->stream,
+                                    g->ns_half ? g->nsx : 0), "ns derivatives");
 }
 
 // offset of field f in a vorticity buffer (half spectra: rows of nsx)
@@ -741,7 +743,8 @@ template <class Rl> int ns_prep_one(pss_grid *g, int64_t f)
 {
     V2<Rl> *w[3] = {B<Rl>(g, 0) + ns_off(g, f), B<Rl>(g, 1) + ns_off(g, f), B<Rl>(g, 2) + ns_off(g, f)};
     return g->cuda(ns_prep_pass<Rl>(w, nullptr, Bf<Rl>(g, 4, f), Bf<Rl>(g, 5, f), Rt<Rl>(g->kxo), Rt<Rl>(g->kyo),
-                                    Rt<Rl>(g->kx2), Rt<Rl>(g->ky2), g->nx, g->ny, 1, Tw<Rl>(g->twy), g->stream,
+                                    Rt<Rl>(g->kx2), Rt<Rl>(g->ky2), g->nx, g->ny, 1,
+                                    reinterpret_cast<int *>(g->flags), Tw<Rl>(g->twy), g->stream,
                                     g->ns_half ? g->nsx : 0),
                    "ns derivatives");
 }
@@ -759,15 +762,6 @@ template <class Rl> int ns_to_half(pss_grid *g, V2<Rl> *src, V2<Rl> *dst, int64_
     return g->cuda(pack_half<Rl>(src, dst, g->nx, g->ny, g->nsx, batch, g->stream), "pack");
 }
 
-// start of a step: mark every field active; the midpoint scheme also needs
-// the derivatives of w^n (its last column pass wrote those of the midpoint)
-template <class Rl> int ns_step_begin(pss_grid *g)
-{
-    int rc = g->cuda(ns_begin(g->ns_field, g->batch, reinterpret_cast<int *>(g->flags), g->stream), "ns begin");
-    if (!rc && g->p.scheme == PSS_NS_MIDPOINT) rc = ns_prep<Rl>(g, true);
-    return rc;
-}
-
 template <class Rl> int ns_set(pss_grid *g, const void *w0, int where)
 {
     int rc;
@@ -780,34 +774,44 @@ template <class Rl> int ns_set(pss_grid *g, const void *w0, int where)
     return where == PSS_HOST ? g->cuda(cudaStreamSynchronize(g->stream), "sync") : PSS_OK;
 }
 
-// the passes of one fixed-point update (row pass, column pass, decide, advance)
-template <class Rl> int ns_update(pss_grid *g, bool in_graph)
+// Updates in one body of the captured loop: an iteration of the WHILE node
+// costs about 5 us beside its kernels, so a body holds the two updates most
+// steps take (four gain another 1 % on long calls and leave up to three
+// updates to run empty at the end of a call, 3 kernels of 2 us each).
+constexpr int NS_BODY = 2;
+
+// one loop body: (midpoint) the derivatives of w^n of the fields that start a
+// step, then `updates` times row pass, column pass and decision
+template <class Rl> int ns_body(pss_grid *g, int updates, bool in_graph)
 {
     V2<Rl> *w[3];
     ns_w<Rl>(g, w);
     int *ctl = reinterpret_cast<int *>(g->flags);
+    const bool mid = g->p.scheme == PSS_NS_MIDPOINT;
     const double parseval = g->p.lx * g->p.ly / (double(g->npts) * double(g->npts));
     int rc;
-    if (!in_graph && (rc = g->pass_begin(0))) return rc;
-    cudaError_t e = ns_row_pass<Rl>(B<Rl>(g, 4), B<Rl>(g, 5), g->ns_field, g->nx, g->ny, g->batch,
-                                    Tw<Rl>(g->twx), g->stream, g->p.dealias != 0, g->ns_half);
-    if ((!in_graph && (rc = g->pass_end())) || (rc = g->cuda(e, "ns row pass"))) return rc;
-    int groups = 0;
-    if (!in_graph && (rc = g->pass_begin(1))) return rc;
-    e = ns_col_pass<Rl>(B<Rl>(g, 4), B<Rl>(g, 5), w, B<Rl>(g, 3), g->ns_field, g->partials, Rt<Rl>(g->kxo),
-                        Rt<Rl>(g->kyo), Rt<Rl>(g->kx2), Rt<Rl>(g->ky2), Rt<Rl>(g->keepx), Rt<Rl>(g->keepy), g->p.dt,
-                        g->p.nu, g->nx, g->ny, g->batch, ctl, g->p.scheme == PSS_NS_MIDPOINT ? 1 : 0, Tw<Rl>(g->twy),
-                        &groups, g->stream, g->p.dealias != 0, g->ns_half ? g->nsx : 0);
-    if ((!in_graph && (rc = g->pass_end())) || (rc = g->cuda(e, "ns column pass"))) return rc;
-    if (!in_graph && (rc = g->pass_begin(2))) return rc;
-    e = ns_decide(g->ns_field, g->partials, groups, g->batch, ctl, parseval, g->p.tol, g->p.max_iter, g->stream);
-    if (e == cudaSuccess) e = ns_advance(ctl, in_graph, g->ns_cond, g->stream);
-    if ((!in_graph && (rc = g->pass_end())) || (rc = g->cuda(e, "ns decide"))) return rc;
+    if (mid && (rc = ns_prep<Rl>(g, true))) return rc;
+    for (int u = 0; u < updates; ++u) {
+        if (!in_graph && (rc = g->pass_begin(0))) return rc;
+        cudaError_t e = ns_row_pass<Rl>(B<Rl>(g, 4), B<Rl>(g, 5), g->ns_field, g->nx, g->ny, g->batch, ctl,
+                                        Tw<Rl>(g->twx), g->stream, g->p.dealias != 0, g->ns_half);
+        if ((!in_graph && (rc = g->pass_end())) || (rc = g->cuda(e, "ns row pass"))) return rc;
+        int groups = 0;
+        if (!in_graph && (rc = g->pass_begin(1))) return rc;
+        e = ns_col_pass<Rl>(B<Rl>(g, 4), B<Rl>(g, 5), w, B<Rl>(g, 3), g->ns_field, g->partials, Rt<Rl>(g->kxo),
+                            Rt<Rl>(g->kyo), Rt<Rl>(g->kx2), Rt<Rl>(g->ky2), Rt<Rl>(g->keepx), Rt<Rl>(g->keepy),
+                            g->p.dt, g->p.nu, g->nx, g->ny, g->batch, ctl, mid ? 1 : 0, Tw<Rl>(g->twy), &groups,
+                            g->stream, g->p.dealias != 0, g->ns_half ? g->nsx : 0);
+        if ((!in_graph && (rc = g->pass_end())) || (rc = g->cuda(e, "ns column pass"))) return rc;
+        if (!in_graph && (rc = g->pass_begin(2))) return rc;
+        e = ns_decide(g->ns_field, g->partials, groups, g->batch, ctl, parseval, g->p.tol, g->p.max_iter, mid,
+                      u + 1 == updates, in_graph, g->ns_cond, g->stream);
+        if ((!in_graph && (rc = g->pass_end())) || (rc = g->cuda(e, "ns decide"))) return rc;
+    }
     return PSS_OK;
 }
 
-// One step as a graph: begin (and, midpoint scheme, the derivatives of w^n),
-// then WHILE(some field active) { one update }.
+// the steps of a call as a graph: WHILE(some field has steps left) { body }
 template <class Rl> int ns_build_graph(pss_grid *g)
 {
     cudaGraph_t graph = nullptr;
@@ -817,22 +821,6 @@ template <class Rl> int ns_build_graph(pss_grid *g)
     if ((rc = g->cuda(cudaGraphConditionalHandleCreate(&g->ns_cond, graph, 1, cudaGraphCondAssignDefault),
                       "conditional handle")))
         return rc;
-    if ((rc = g->cuda(cudaStreamBeginCaptureToGraph(g->stream, graph, nullptr, nullptr, 0,
-                                                    cudaStreamCaptureModeRelaxed), "capture")))
-        return rc;
-    rc = ns_step_begin<Rl>(g);
-    // the last node captured so far: the WHILE node depends on it
-    cudaGraphNode_t begin_node = nullptr;
-    cudaStreamCaptureStatus status;
-    const cudaGraphNode_t *deps = nullptr;
-    size_t ndeps = 0;
-    cudaError_t e = cudaStreamGetCaptureInfo(g->stream, &status, nullptr, nullptr, &deps, nullptr, &ndeps);
-    if (e == cudaSuccess && ndeps == 1) begin_node = deps[0];
-    cudaGraph_t out = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(g->stream, &out);
-    if (rc) return rc;
-    if ((rc = g->cuda(e != cudaSuccess ? e : e2, "capture begin"))) return rc;
-    if (!begin_node) return g->fail(PSS_E_CUDA, "step graph: expected one node before the loop, found %zu", ndeps);
     // zero-initialised node parameters (the struct's union has no default constructor)
     alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)] = {};
     cudaGraphNodeParams &cp = *reinterpret_cast<cudaGraphNodeParams *>(raw);
@@ -841,15 +829,16 @@ template <class Rl> int ns_build_graph(pss_grid *g)
     cp.conditional.type = cudaGraphCondTypeWhile;
     cp.conditional.size = 1;
     cudaGraphNode_t cnode = nullptr;
-    if ((rc = g->cuda(cudaGraphAddNode(&cnode, graph, &begin_node, nullptr, 1, &cp), "conditional node"))) return rc;
+    if ((rc = g->cuda(cudaGraphAddNode(&cnode, graph, nullptr, nullptr, 0, &cp), "conditional node"))) return rc;
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     if ((rc = g->cuda(cudaStreamBeginCaptureToGraph(g->stream, body, nullptr, nullptr, 0,
                                                     cudaStreamCaptureModeRelaxed), "capture body")))
         return rc;
-    rc = ns_update<Rl>(g, true);
-    e2 = cudaStreamEndCapture(g->stream, &out);
+    rc = ns_body<Rl>(g, NS_BODY, true);
+    cudaGraph_t out = nullptr;
+    const cudaError_t e = cudaStreamEndCapture(g->stream, &out);
     if (rc) return rc;
-    if ((rc = g->cuda(e2, "capture body end"))) return rc;
+    if ((rc = g->cuda(e, "capture body end"))) return rc;
     return g->cuda(cudaGraphInstantiate(&g->ns_exec, graph, 0), "graph instantiate");
 }
 
@@ -864,22 +853,23 @@ template <class Rl> int ns_step(pss_grid *g, int64_t n)
         cudaGetLastError();
         g->err.clear();
     }
-    if (g->use_graphs && !g->profiling) {
-        for (int64_t s = 0; s < n; ++s)
+    const int64_t most = 1 << 30;  // steps per launch of the loop (the records count in 32 bits)
+    for (int64_t done = 0; done < n; done += most) {
+        const int part = int(std::min(most, n - done));
+        if ((rc = g->cuda(ns_begin(g->ns_field, g->batch, ctl, part, g->stream), "ns begin"))) return rc;
+        if (g->use_graphs && !g->profiling) {
             if ((rc = g->cuda(cudaGraphLaunch(g->ns_exec, g->stream), "graph launch"))) return rc;
-        return PSS_OK;  // a field that reached max_iter is reported by the next synchronising call
-    }
-    for (int64_t s = 0; s < n; ++s) {
-        if ((rc = ns_step_begin<Rl>(g))) return rc;
-        for (int k = 0; k < g->p.max_iter; ++k) {
-            if ((rc = ns_update<Rl>(g, false))) return rc;
+            continue;
+        }
+        do {
+            if ((rc = ns_body<Rl>(g, 1, false))) return rc;
             if ((rc = g->cuda(cudaMemcpyAsync(hctl, ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, g->stream),
                               "ctl copy")) ||
                 (rc = g->cuda(cudaStreamSynchronize(g->stream), "ns sync")))
                 return rc;
-            if (hctl[2] == 0) break;
-        }
+        } while (hctl[2] != 0);
     }
+    if (g->use_graphs && !g->profiling) return PSS_OK;  // a field that reached max_iter: the next synchronising call
     rc = g->check_ns_nonconv();
     if (rc == PSS_E_NOT_CONVERGED) g->steps += n;  // the steps were taken; pss_grid::step_n adds n only on success
     return rc;
@@ -1251,7 +1241,7 @@ int pss_grid::checkpoint(void *buf_, int where, bool save)
         } else if (p.eq == PSS_EQ_NS) {
             // all fields restart from buffer 0 with their update count
             NsFieldHost *h = static_cast<NsFieldHost *>(host_fields);
-            for (int64_t i = 0; i < batch; ++i) h[i] = NsFieldHost{0, 0, 0, 0, i == 0 ? meta[1] : 0};
+            for (int64_t i = 0; i < batch; ++i) h[i] = NsFieldHost{0, 0, 0, 0, i == 0 ? meta[1] : 0, 0, 0};
             rc = cuda(cudaMemcpyAsync(ns_field, h, size_t(batch) * ns_field_bytes(), cudaMemcpyHostToDevice, stream),
                       "fields");
             if (!rc && ns_half)

@@ -82,7 +82,7 @@ struct pss_grid {
     // captured CUDA graphs (NLS/SG: also while profiling; NS: off while
     // profiling; all off with PSS_GRAPHS=0)
     bool use_graphs = true;
-    cudaGraph_t ns_graph = nullptr;       // one NS step: begin -> WHILE(active) { passes }
+    cudaGraph_t ns_graph = nullptr;       // NS: WHILE(steps left) { updates }
     cudaGraphExec_t ns_exec = nullptr;
     cudaGraphConditionalHandle ns_cond = 0;
     // NLS/SG step_n(n) as one graph, by (n, profiling stride).  A profiling

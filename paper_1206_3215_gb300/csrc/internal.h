@@ -111,7 +111,7 @@ cudaError_t unpack_half(const V2<Rl> *half, V2<Rl> *full, int64_t nx, int64_t ny
 size_t ns_field_bytes();  // bytes of the per-field fixed-point record
 template <class Rl>
 cudaError_t ns_row_pass(V2<Rl> *c1, V2<Rl> *c2, const void *fs, int64_t nx, int64_t ny, int64_t batch,
-                        const TW<Rl> *twx, cudaStream_t s, bool dealias, bool half = false);
+                        const int *ctl, const TW<Rl> *twx, cudaStream_t s, bool dealias, bool half = false);
 template <class Rl>
 cudaError_t ns_col_pass(V2<Rl> *c1, V2<Rl> *c2, V2<Rl> *const w[3], V2<Rl> *jn, void *fs, double *partials,
                         const Rl *kxo, const Rl *kyo, const Rl *kx2, const Rl *ky2, const Rl *keepx,
@@ -121,13 +121,13 @@ cudaError_t ns_col_pass(V2<Rl> *c1, V2<Rl> *c2, V2<Rl> *const w[3], V2<Rl> *jn, 
 template <class Rl>
 cudaError_t ns_prep_pass(V2<Rl> *const w[3], const void *fs, V2<Rl> *c1, V2<Rl> *c2, const Rl *kxo, const Rl *kyo,
                          const Rl *kx2, const Rl *ky2, int64_t nx, int64_t ny, int64_t batch,
-                         const TW<Rl> *twy, cudaStream_t s, int64_t sx = 0);
-// loop control ctl (4 ints on the device): [0] update index, [1] any field
-// active after the current update, [2] its value at the last advance
-cudaError_t ns_begin(void *fs, int64_t batch, int *ctl, cudaStream_t s);
+                         const int *ctl, const TW<Rl> *twy, cudaStream_t s, int64_t sx = 0);
+// Loop control (ctl: ints of the grid's flag block, k_ns.cuh): n steps of every
+// field; the decision after an update (`last`: the last one of a loop body).
+cudaError_t ns_begin(void *fs, int64_t batch, int *ctl, int n, cudaStream_t s);
 cudaError_t ns_decide(void *fs, const double *partials, int64_t groups, int64_t batch, int *ctl, double parseval,
-                      double tol, int max_iter, cudaStream_t s);
-cudaError_t ns_advance(int *ctl, bool use_graph, cudaGraphConditionalHandle h, cudaStream_t s);
+                      double tol, int max_iter, bool restart_at_end, bool last, bool use_graph,
+                      cudaGraphConditionalHandle h, cudaStream_t s);
 
 // ---- elementwise helpers (k_util.cu) ----------------------------------------
 template <class Rl> cudaError_t real_to_complex(const Rl *src, V2<Rl> *dst, int64_t n, cudaStream_t s);
@@ -171,10 +171,10 @@ constexpr unsigned FLAG_NONFINITE = 1u;
 constexpr unsigned FLAG_NOT_CONVERGED = 2u;
 
 // int slot of the grid's 64-byte device flag block that pass kernels report
-// a lost tile copy in (slots 0 .. 3 carry the NS step control)
+// a lost tile copy in (slots 0 .. 3 and 6 carry the NS loop control, k_ns.cuh)
 constexpr int FLAG_SLOT_PASS_STATUS = 8;
 // NS split column pass: slot 4 its item counter (zeroed by k_ns_begin and
-// k_ns_advance), slot 5 the column-pass epoch (never reset; k_ns_advance
+// k_ns_decide), slot 5 the column-pass epoch (never reset; k_ns_decide
 // adds one), and from int FLAG_TILE_DONE on one word per column tile
 // (batch x nx words, allocated after the 64-byte block for NS grids)
 constexpr int FLAG_SLOT_SPLIT_CLAIM = 4;

@@ -4,79 +4,96 @@
 
 namespace pss {
 
-// Device-side loop control, 4 ints: [0] update index k of the current pass,
-// [1] any field still active after this update (built by k_ns_decide),
-// [2] the value of [1] at the last k_ns_advance (read by the host loop); and
-// the split column pass's item counter and epoch (FLAG_SLOT_SPLIT_CLAIM,
-// FLAG_SLOT_EPOCH).
-// one block per field: fold the partials of update k in a fixed order (a
-// strided sum per thread, then a tree), decide, count
+// One block per field: fold the partials of its update in a fixed order (a
+// strided sum per thread, then a tree), decide, count.  A field whose step is
+// done goes on with its next one in the next update, whatever the batch's
+// other fields do; with `restart_at_end` (midpoint: a step starts with the
+// derivatives of w^n, formed once per loop body) it pauses until the body's
+// last update (`last`).  The block that finishes last resets the control
+// words for the next column pass and, inside a captured loop, sets the WHILE
+// node's condition: some field is active.  Every field stops at max_iter at
+// the latest, so the loop always ends; after a lost tile copy it ends at once.
 constexpr int NS_DECIDE_THREADS = 256;
 __global__ void __launch_bounds__(NS_DECIDE_THREADS)
     k_ns_decide(NsField *fs, const double *partials, int64_t groups, int64_t batch, int *ctl, double parseval,
-                double tol, int max_iter)
+                double tol, int max_iter, int restart_at_end, int last, int use_graph, cudaGraphConditionalHandle h)
 {
     __shared__ double red[NS_DECIDE_THREADS];
+    const bool idle = ctl[NS_CTL_MORE] == 0;
     const int64_t f = blockIdx.x;
-    if (f >= batch) return;
     NsField s = fs[f];
-    if (!s.active) return;  // the same for every thread of the block
-    double sum = 0.0;
-    for (int64_t g = threadIdx.x; g < groups; g += NS_DECIDE_THREADS) sum += partials[f * groups + g];
-    red[threadIdx.x] = sum;
-    __syncthreads();
-    for (int w = NS_DECIDE_THREADS / 2; w > 0; w >>= 1) {
-        if (int(threadIdx.x) < w) red[threadIdx.x] += red[threadIdx.x + w];
+    if (!idle && s.active) {  // the same for every thread of the block
+        double sum = 0.0;
+        for (int64_t g = threadIdx.x; g < groups; g += NS_DECIDE_THREADS) sum += partials[f * groups + g];
+        red[threadIdx.x] = sum;
         __syncthreads();
+        for (int w = NS_DECIDE_THREADS / 2; w > 0; w >>= 1) {
+            if (int(threadIdx.x) < w) red[threadIdx.x] += red[threadIdx.x + w];
+            __syncthreads();
+        }
     }
     if (threadIdx.x != 0) return;
-    const int k = ctl[0];
-    int *any_active = ctl + 1;
-    const double norm = parseval * red[0];
-    s.updates += 1;
-    const bool done = norm < tol;
-    if (done || k + 1 >= max_iter) {
-        if (!done) s.nonconv = 1;
-        s.idx = ns_buf(s.idx, k + 1);
-        s.active = 0;
-    } else {
-        atomicOr(any_active, 1);
+    if (!idle) {
+        if (s.active) {
+            const double norm = parseval * red[0];
+            s.updates += 1;
+            const bool done = norm < tol;
+            if (done || s.k + 1 >= max_iter) {
+                if (!done) s.nonconv = 1;
+                s.idx = ns_buf(s.idx, s.k + 1);
+                s.k = 0;
+                s.left -= 1;
+                s.active = s.left > 0 && !restart_at_end;
+            } else {
+                s.k += 1;
+            }
+        }
+        if (restart_at_end && last && !s.active && s.left > 0) s.active = 1;
+        fs[f] = s;
+        const int any = (s.left > 0 ? 1 : 0) | (s.active && s.k == 0 ? 2 : 0) | (s.active ? 4 : 0);
+        if (any) atomicOr(ctl + NS_CTL_ANY, any);
     }
-    fs[f] = s;
-}
-
-__global__ void k_ns_begin(NsField *fs, int64_t batch, int *ctl)
-{
-    const int64_t f = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (f == 0) {
-        ctl[0] = 0;
-        ctl[1] = 0;
-        ctl[FLAG_SLOT_SPLIT_CLAIM] = 0;
-    }
-    if (f < batch) fs[f].active = 1;
-}
-
-// next update: k += 1; the loop continues while some field is active.  Inside
-// a captured step graph this sets the WHILE node's condition; every field
-// stops at max_iter at the latest, so the loop always ends.
-__global__ void k_ns_advance(int *ctl, int use_graph, cudaGraphConditionalHandle h)
-{
-    const int more = ctl[1] != 0;
-    ctl[2] = more;
-    ctl[1] = 0;
-    ctl[0] += 1;
+    __threadfence();
+    if (atomicAdd(ctl + NS_CTL_TICKET, 1) + 1 < int(gridDim.x)) return;
+    __threadfence();
+    const int any = atomicExch(ctl + NS_CTL_ANY, 0);
+    const int more = (any & 1) && ctl[FLAG_SLOT_PASS_STATUS] == 0;
+    ctl[NS_CTL_TICKET] = 0;
+    ctl[NS_CTL_MORE] = more;
+    ctl[NS_CTL_START] = (any & 2) != 0;
+    ctl[NS_CTL_ACTIVE] = more && (any & 4) != 0;
     ctl[FLAG_SLOT_SPLIT_CLAIM] = 0;  // the next column pass claims its items from 0
     ctl[FLAG_SLOT_EPOCH] += 1;       // and publishes its tiles under a new value
     if (use_graph) cudaGraphSetConditional(h, more ? 1u : 0u);
 }
 
+// start of a call of n steps
+__global__ void k_ns_begin(NsField *fs, int64_t batch, int *ctl, int n)
+{
+    const int64_t f = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (f == 0) {
+        ctl[NS_CTL_ANY] = 0;
+        ctl[NS_CTL_TICKET] = 0;
+        ctl[NS_CTL_MORE] = 1;
+        ctl[NS_CTL_START] = 1;
+        ctl[NS_CTL_ACTIVE] = 1;
+        ctl[FLAG_SLOT_SPLIT_CLAIM] = 0;
+    }
+    if (f < batch) {
+        fs[f].active = 1;
+        fs[f].k = 0;
+        fs[f].left = n;
+    }
+}
+
 template <class Rl>
 cudaError_t ns_row_pass(V2<Rl> *c1, V2<Rl> *c2, const void *fs, int64_t nx, int64_t ny, int64_t batch,
-                        const TW<Rl> *twx, cudaStream_t s, bool dealias, bool half)
+                        const int *ctl, const TW<Rl> *twx, cudaStream_t s, bool dealias, bool half)
 {
     int lgy = 0;
     while ((int64_t(1) << lgy) < ny) ++lgy;  // ny is a power of two
-    return launch_row<Rl>(nx, ny, NsRow<Rl>{c1, c2, static_cast<const NsField *>(fs), lgy, dealias ? 1 : 0, half ? 1 : 0},
+    return launch_row<Rl>(nx, ny, NsRow<Rl>{c1, c2, static_cast<const NsField *>(fs), lgy, dealias ? 1 : 0, half ? 1 : 0,
+                                            ctl},
                           twx, batch, s);
 }
 
@@ -99,31 +116,27 @@ cudaError_t ns_col_pass(V2<Rl> *c1, V2<Rl> *c2, V2<Rl> *const w[3], V2<Rl> *jn, 
 template <class Rl>
 cudaError_t ns_prep_pass(V2<Rl> *const w[3], const void *fs, V2<Rl> *c1, V2<Rl> *c2, const Rl *kxo, const Rl *kyo,
                          const Rl *kx2, const Rl *ky2, int64_t nx, int64_t ny, int64_t batch,
-                         const TW<Rl> *twy, cudaStream_t s, int64_t sx)
+                         const int *ctl, const TW<Rl> *twy, cudaStream_t s, int64_t sx)
 {
-    if (sx > 0) return ns_prep_half<Rl>(w, fs, c1, c2, kxo, kyo, kx2, ky2, nx, sx, ny, batch, twy, s);
+    if (sx > 0) return ns_prep_half<Rl>(w, fs, c1, c2, kxo, kyo, kx2, ky2, nx, sx, ny, batch, ctl, twy, s);
     NsPrep<Rl> op{w[0], w[1], w[2], static_cast<const NsField *>(fs), c1, c2, kxo, kyo, kx2, ky2,
-                  Rl(1.0 / (double(nx) * double(ny))), nx, nx};
+                  Rl(1.0 / (double(nx) * double(ny))), nx, nx, ctl};
     return launch_col<Rl>(ny, nx, op, twy, batch, s);
 }
 
-cudaError_t ns_begin(void *fs, int64_t batch, int *ctl, cudaStream_t s)
+cudaError_t ns_begin(void *fs, int64_t batch, int *ctl, int n, cudaStream_t s)
 {
-    k_ns_begin<<<unsigned((batch + 255) / 256), 256, 0, s>>>(static_cast<NsField *>(fs), batch, ctl);
+    k_ns_begin<<<unsigned((batch + 255) / 256), 256, 0, s>>>(static_cast<NsField *>(fs), batch, ctl, n);
     return cudaGetLastError();
 }
 
 cudaError_t ns_decide(void *fs, const double *partials, int64_t groups, int64_t batch, int *ctl, double parseval,
-                      double tol, int max_iter, cudaStream_t s)
+                      double tol, int max_iter, bool restart_at_end, bool last, bool use_graph,
+                      cudaGraphConditionalHandle h, cudaStream_t s)
 {
     k_ns_decide<<<unsigned(batch), NS_DECIDE_THREADS, 0, s>>>(static_cast<NsField *>(fs), partials, groups,
-                                                             batch, ctl, parseval, tol, max_iter);
-    return cudaGetLastError();
-}
-
-cudaError_t ns_advance(int *ctl, bool use_graph, cudaGraphConditionalHandle h, cudaStream_t s)
-{
-    k_ns_advance<<<1, 1, 0, s>>>(ctl, use_graph ? 1 : 0, h);
+                                                             batch, ctl, parseval, tol, max_iter,
+                                                             restart_at_end ? 1 : 0, last ? 1 : 0, use_graph ? 1 : 0, h);
     return cudaGetLastError();
 }
 
@@ -131,7 +144,7 @@ size_t ns_field_bytes() { return sizeof(NsField); }
 
 #define PSS_INST(Rl)                                                                                         \
     template cudaError_t ns_row_pass<Rl>(V2<Rl> *, V2<Rl> *, const void *, int64_t, int64_t, int64_t,       \
-                                         const TW<Rl> *, cudaStream_t, bool, bool);                          \
+                                         const int *, const TW<Rl> *, cudaStream_t, bool, bool);             \
     template cudaError_t ns_col_pass<Rl>(V2<Rl> *, V2<Rl> *, V2<Rl> *const[3], V2<Rl> *, void *, double *,  \
                                          const Rl *, const Rl *, const Rl *, const Rl *, const Rl *,         \
                                          const Rl *, double, double, int64_t, int64_t, int64_t,             \
@@ -139,8 +152,8 @@ size_t ns_field_bytes() { return sizeof(NsField); }
                                          int64_t);                                                           \
     template cudaError_t ns_prep_pass<Rl>(V2<Rl> *const[3], const void *, V2<Rl> *, V2<Rl> *, const Rl *,     \
                                           const Rl *,                                                         \
-                                          const Rl *, const Rl *, int64_t, int64_t, int64_t, const TW<Rl> *, \
-                                          cudaStream_t, int64_t);
+                                          const Rl *, const Rl *, int64_t, int64_t, int64_t, const int *,    \
+                                          const TW<Rl> *, cudaStream_t, int64_t);
 PSS_INST(float)
 PSS_INST(double)
 

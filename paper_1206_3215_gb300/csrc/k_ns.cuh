@@ -57,12 +57,22 @@ __host__ __device__ constexpr int ns_pmax(int n) { return n <= 1024 ? NS_PMAX : 
 __device__ __forceinline__ float ns_rcp(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double ns_rcp(double x) { return __drcp_rn(x); }
 
+// Device-side loop control, ints of the grid's flag block: what the blocks of
+// k_ns_decide found so far and how many of them are done; then, for the
+// passes that follow, whether any field has steps left (the loop's
+// condition), stands at the start of a step whose derivatives are still to be
+// formed (midpoint), takes part in the next update (else the passes return at
+// once).
+constexpr int NS_CTL_ANY = 0, NS_CTL_TICKET = 1, NS_CTL_MORE = 2, NS_CTL_START = 3, NS_CTL_ACTIVE = 6;
+
 struct NsField {
     int idx;        // buffer holding w^n
-    int active;     // still iterating in this step
+    int active;     // takes part in the next update
     int nonconv;    // reached max_iter in some step (sticky)
-    int pad;
+    int k;          // index of the next update within its step
     long long updates;  // CN updates (= Jacobian evaluations) summed over steps
+    int left;       // steps still to take in this call
+    int pad;
 };
 
 __host__ __device__ __forceinline__ int ns_buf(int idx, int k)
@@ -106,6 +116,8 @@ template <class Rl> struct NsRow {
     int dealias;  // 2/3 rule: columns with 3 |mx| >= nx are not written (they stay
                   // zero: the column pass skips them and the mask discards J there)
     int half;     // half spectra: only columns 0 .. nx/2 of J are read, so only they are written
+    const int *ctl;
+    __device__ __forceinline__ bool idle() const { return ctl[NS_CTL_ACTIVE] == 0; }
     __device__ const V2<Rl> *in(int k) const { return k == 0 ? c1 : c2; }
     template <int N, int P, int BLOCK, class Sm>
     __device__ __forceinline__ void row(V2<Rl> (&v)[2][P], int64_t r, bool ok, int t, const Sm (&sm)[2],
@@ -175,7 +187,7 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
     const Rl *kxo, *kyo, *kx2, *ky2, *keepx, *keepy;
     Rl half_dt, half_dt_nu, inv_n2;
     int64_t nx;             // row stride of w and J_hat^n (half spectra: nxf/2 + 8)
-    const int *kptr;  // fixed-point update index of this pass (device, set by k_ns_advance)
+    const int *ctl;  // loop control (k_ns.cu)
     int W;
     int64_t in_stride;      // row stride of J, C1, C2 (= nxf)
     // 2/3 rule: column groups skip_lo .. skip_lo + skip_n - 1 hold only modes
@@ -188,6 +200,7 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
     int *claim;
     const int *epoch;
     unsigned *tile_done;
+    __device__ __forceinline__ bool idle() const { return ctl[NS_CTL_ACTIVE] == 0; }
     static constexpr bool midpoint = MID;  // implicit midpoint, else trapezoidal Jacobian
     __host__ __device__ const V2<Rl> *in(int) const { return c1; }
     __device__ V2<Rl> *wb(int b) const { return b == 0 ? w0 : b == 1 ? w1 : w2; }
@@ -220,8 +233,8 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
                                               const TW<Rl> *tw, int o0, int o1) const
     {
         constexpr int T = N / P;
-        const int k = *kptr;
         const NsField f = fs[field];
+        const int k = f.k;
         const int64_t nxf = in_stride;
         // half spectra: the padding columns beyond nxf/2 carry nothing
         const bool valid = !HALF || 2 * int64_t(x) <= nxf;
@@ -390,12 +403,14 @@ template <class Rl, bool HALF = false> struct NsPrep {
     static constexpr int NOUT = HALF ? 4 : 2;
     __host__ __device__ static constexpr int pmax(int n) { return n < 1024 ? NS_PMAX : NS_PREP_PMAX_BIG; }
     const V2<Rl> *w0, *w1, *w2;
-    const NsField *fs;
+    const NsField *fs;  // null: every field, from buffer 0; else the fields at the start of a step
     V2<Rl> *c1, *c2;
     const Rl *kxo, *kyo, *kx2, *ky2;
     Rl inv_n2;
     int64_t nx;   // row stride of w (half spectra: nxf/2 + 8)
     int64_t nxf;  // row stride of C1, C2
+    const int *ctl;
+    __device__ __forceinline__ bool idle() const { return fs && ctl[NS_CTL_START] == 0; }
     __device__ const V2<Rl> *in(int, int64_t field) const
     {
         const int b = fs ? fs[field].idx : 0;
@@ -409,7 +424,7 @@ template <class Rl, bool HALF = false> struct NsPrep {
         V2<Rl>(&v)[P] = vv[0];
         const int64_t base = field * N * nx + x;
         const V2<Rl> *w = in(0, field) + base;
-        const bool valid = !HALF || 2 * int64_t(x) <= nxf;
+        const bool valid = (!HALF || 2 * int64_t(x) <= nxf) && (!fs || (fs[field].active && fs[field].k == 0));
         const int xs = valid ? x : 0;
         const Rl kx = __ldg(kxo + xs), kxx = __ldg(kx2 + xs);
         // the first output from the staged column, the others from the column
@@ -506,6 +521,6 @@ cudaError_t ns_col_half(V2<Rl> *c1, V2<Rl> *c2, V2<Rl> *const w[3], V2<Rl> *jn, 
 template <class Rl>
 cudaError_t ns_prep_half(V2<Rl> *const w[3], const void *fs, V2<Rl> *c1, V2<Rl> *c2, const Rl *kxo, const Rl *kyo,
                          const Rl *kx2, const Rl *ky2, int64_t nxf, int64_t sx, int64_t ny, int64_t batch,
-                         const TW<Rl> *twy, cudaStream_t s);
+                         const int *ctl, const TW<Rl> *twy, cudaStream_t s);
 
 }  // namespace pss

@@ -24,10 +24,10 @@ cudaError_t ns_col_half(V2<Rl> *c1, V2<Rl> *c2, V2<Rl> *const w[3], V2<Rl> *jn, 
 template <class Rl>
 cudaError_t ns_prep_half(V2<Rl> *const w[3], const void *fs, V2<Rl> *c1, V2<Rl> *c2, const Rl *kxo, const Rl *kyo,
                          const Rl *kx2, const Rl *ky2, int64_t nxf, int64_t sx, int64_t ny, int64_t batch,
-                         const TW<Rl> *twy, cudaStream_t s)
+                         const int *ctl, const TW<Rl> *twy, cudaStream_t s)
 {
     NsPrep<Rl, true> op{w[0], w[1], w[2], static_cast<const NsField *>(fs), c1, c2, kxo, kyo, kx2, ky2,
-                        Rl(1.0 / (double(nxf) * double(ny))), sx, nxf};
+                        Rl(1.0 / (double(nxf) * double(ny))), sx, nxf, ctl};
     return launch_col<Rl>(ny, sx, op, twy, batch, s);
 }
 
@@ -38,7 +38,7 @@ cudaError_t ns_prep_half(V2<Rl> *const w[3], const void *fs, V2<Rl> *c1, V2<Rl> 
                                          const int *, int, const TW<Rl> *, int *, cudaStream_t, bool);      \
     template cudaError_t ns_prep_half<Rl>(V2<Rl> *const[3], const void *, V2<Rl> *, V2<Rl> *, const Rl *,     \
                                           const Rl *, const Rl *, const Rl *, int64_t, int64_t, int64_t,     \
-                                          int64_t, const TW<Rl> *, cudaStream_t);
+                                          int64_t, const int *, const TW<Rl> *, cudaStream_t);
 PSS_INST(float)
 PSS_INST(double)
 

@@ -148,8 +148,9 @@ __global__ void __launch_bounds__(RED_THREADS)
 // NS from the spectrum w_hat of each field (buffer fs[f].idx): Re w_hat(0,0)
 // (= sum of w), sum |w_hat|^2, sum over k != 0 of |w_hat|^2 / |k|^2.
 struct NsFieldRd {
-    int idx, active, nonconv, pad;
+    int idx, active, nonconv, k;
     long long updates;
+    int left, pad;
 };
 template <class Rl>
 __global__ void __launch_bounds__(RED_THREADS)

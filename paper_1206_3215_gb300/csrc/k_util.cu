@@ -20,8 +20,9 @@ __global__ void k_complex_to_real(const V2<Rl> *a, const V2<Rl> *b, Rl c, Rl *ds
 
 // copy every field's current vorticity (buffer fs[f].idx) into dst
 struct NsFieldView {
-    int idx, active, nonconv, pad;
+    int idx, active, nonconv, k;
     long long updates;
+    int left, pad;
 };
 template <class Rl>
 __global__ void k_ns_gather(const NsFieldView *fs, const V2<Rl> *w0, const V2<Rl> *w1, const V2<Rl> *w2,

@@ -334,6 +334,17 @@ template <class Op, class = void> struct EarlyNext : std::false_type {};
 template <class Op>
 struct EarlyNext<Op, std::void_t<decltype(Op::EARLY_NEXT)>> : std::integral_constant<bool, Op::EARLY_NEXT> {};
 
+// An op may define idle(): its pass has nothing to do (passes of a captured
+// loop that has ended); every CTA then returns before its first tile.
+template <class Op, class = void> struct HasIdle : std::false_type {};
+template <class Op>
+struct HasIdle<Op, std::void_t<decltype(std::declval<const Op &>().idle())>> : std::true_type {};
+template <class Op> __device__ __forceinline__ bool op_idle(const Op &op)
+{
+    if constexpr (HasIdle<Op>::value) return op.idle();
+    else return false;
+}
+
 // An op that sets DIRECT_LOAD reads its rows itself (op.load<N, P>(v, row, ok,
 // t): register m = element t + T m) instead of having them staged: rows that
 // are not complex arrays, or that one thread gathers from two places.
@@ -351,6 +362,7 @@ __global__ void __launch_bounds__(RowCfgOf<Rl, N, Op, VAR>::THREADS, RowCfgOf<Rl
     using Sm = SmemLine<V, C::PADLOG>;
     constexpr int NIN = Op::NIN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (op_idle(op)) return;
     V *const buf = reinterpret_cast<V *>(smem_raw);
     const int lr = threadIdx.x / C::T, t = threadIdx.x % C::T;
     const int64_t tiles = (rows_total + C::ROWS - 1) / C::ROWS;
@@ -462,6 +474,7 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, VAR>::THREADS, ColCfgOf<Rl
     using Sm = SmemLine<V, C::PADLOG>;
     constexpr int NIN = Op::NIN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (op_idle(op)) return;
     V *const buf = reinterpret_cast<V *>(smem_raw);
     const int c = threadIdx.x % C::W, t = threadIdx.x / C::W;
     const int64_t groups = kept_groups(op, nx / C::W), tiles = groups * batch;
@@ -574,6 +587,7 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, 0>::THREADS, ColCfgOf<Rl, 
     using Sm = SmemLine<V, C::PADLOG>;
     static_assert(C::NBUF == 1, "one staging buffer");
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (op_idle(op)) return;
     // align to 128 bytes by an offset from the shared array itself (an
     // address rebuilt from an integer would lose the shared state space and
     // turn every exchange access into a generic one)
@@ -731,6 +745,7 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, 0>::THREADS, ColCfgOf<Rl, 
     using Sm = SmemLine<V, C::PADLOG>;
     static_assert(C::NBUF == 1 && C::BLOCK == 1, "one staging buffer; transforms span the CTA");
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (op_idle(op)) return;
     V *const buf = reinterpret_cast<V *>(smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u));
     const unsigned sbar = smem_addr(buf + C::BUF);
     __shared__ int item_s;
@@ -891,6 +906,7 @@ __global__ void __launch_bounds__(2 * ColCfgOf<Rl, N, Op, 0>::THREADS,
     constexpr bool TST = TmaStoreOp<Op>::value;
     constexpr int GB = land_gbuf<C>();  // elements per group buffer (128-byte multiple)
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (op_idle(op)) return;
     V *const xbuf = reinterpret_cast<V *>(smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u));
     V *const land = xbuf + 2 * GB;                      // the dense [N][W] landing block
     const unsigned sbar = smem_addr(land + N * C::W);   // mbarrier of group g at sbar + 8 g
