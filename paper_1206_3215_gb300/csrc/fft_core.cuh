@@ -227,6 +227,32 @@ __device__ __forceinline__ void prefetch_l2(const void *p)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
+// The passes of a step form a chain in which each kernel reads what the one
+// before it wrote.  They are launched so that a kernel's CTAs may start while
+// its predecessor still runs (launch_chain in launch.cuh): a kernel fills its
+// tables and barriers, which depend on no earlier kernel, waits until the
+// earlier kernels of the chain have completed and their stores are visible
+// (grid_wait), and then lets its own successor start (grid_trigger).  Every
+// CTA waits, also one without work, so that a kernel never completes before
+// its predecessors; the trigger comes after the wait, so that only the next
+// kernel's CTAs sit waiting, not those of the whole chain.  Only grids of one
+// wave, with at most one CTA per SM of at most half an SM's shared memory,
+// give it: beside fuller grids the early CTAs pile up on the SMs that have
+// room first and the next kernel runs unevenly spread (a trigger in every
+// kernel: NLS 4096^2 x 2 447 -> 474 us per step, SG 512^2 x 8 27 -> 31;
+// without the limit on shared memory NLS 1024^2 19.0 -> 21.2).  Per step, plain
+// launches -> these: NLS 64^2 10.9 -> 8.2 us, 256^2 12.1 -> 9.0, 512^2 15.3 -> 12.7,
+// SG 512^2 x 2 26.6 -> 22.1; where no kernel gives the trigger, 0 - 3 %.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+constexpr unsigned GRID_SMS = 152, GRID_EARLY_SMEM = 114 * 1024;
+__device__ __forceinline__ void grid_trigger(int64_t tiles)
+{
+    unsigned smem;
+    asm("mov.u32 %0, %dynamic_smem_size;" : "=r"(smem));
+    if (gridDim.x <= GRID_SMS && tiles <= int64_t(gridDim.x) && smem <= GRID_EARLY_SMEM)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Load of streamed state (read once per pass, or re-read from L2 right after
 // this thread stored it): cached in L2 only, so that it does not evict the
 // small tables (wavenumbers, masks, twiddles) the pass keeps reading through

@@ -19,6 +19,8 @@ __global__ void __launch_bounds__(NS_DECIDE_THREADS)
                 double tol, int max_iter, int restart_at_end, int last, int use_graph, cudaGraphConditionalHandle h)
 {
     __shared__ double red[NS_DECIDE_THREADS];
+    grid_wait();
+    grid_trigger(1);
     const bool idle = ctl[NS_CTL_MORE] == 0;
     const int64_t f = blockIdx.x;
     NsField s = fs[f];
@@ -134,10 +136,9 @@ cudaError_t ns_decide(void *fs, const double *partials, int64_t groups, int64_t 
                       double tol, int max_iter, bool restart_at_end, bool last, bool use_graph,
                       cudaGraphConditionalHandle h, cudaStream_t s)
 {
-    k_ns_decide<<<unsigned(batch), NS_DECIDE_THREADS, 0, s>>>(static_cast<NsField *>(fs), partials, groups,
-                                                             batch, ctl, parseval, tol, max_iter,
-                                                             restart_at_end ? 1 : 0, last ? 1 : 0, use_graph ? 1 : 0, h);
-    return cudaGetLastError();
+    return launch_chain(k_ns_decide, unsigned(batch), NS_DECIDE_THREADS, 0, s, static_cast<NsField *>(fs), partials,
+                        groups, batch, ctl, parseval, tol, max_iter, restart_at_end ? 1 : 0, last ? 1 : 0,
+                        use_graph ? 1 : 0, h);
 }
 
 size_t ns_field_bytes() { return sizeof(NsField); }

@@ -83,6 +83,8 @@ __global__ void __launch_bounds__(R2cCfg<Rl, M, SMALL>::THREADS, R2cCfg<Rl, M, S
     const int rl = threadIdx.x / T, t = threadIdx.x % T;
     const Sm sm{reinterpret_cast<V *>(smem_raw) + rl * C::LINE};
     fill_stage_tw<M, P>(twm);
+    grid_wait();
+    grid_trigger((rows_total + C::ROWS - 1) / C::ROWS);
     __syncthreads();
     for (int64_t r0 = int64_t(blockIdx.x) * C::ROWS; r0 < rows_total; r0 += int64_t(gridDim.x) * C::ROWS) {
         const int64_t row = r0 + rl;
@@ -174,8 +176,7 @@ cudaError_t launch_half_row(const HalfRowArgs<Rl> &g, int64_t rows_total, const 
     int grid = 0;
     if ((e = resident_ctas(k, C::THREADS, C::SMEM, ctas, &grid)) != cudaSuccess) return e;
     if (tiles < grid) grid = int(tiles);
-    k<<<dim3(unsigned(grid)), C::THREADS, C::SMEM, s>>>(g, rows_total, twm, twn);
-    return cudaGetLastError();
+    return launch_chain(k, unsigned(grid), C::THREADS, C::SMEM, s, g, rows_total, twm, twn);
 }
 
 // rows of nx real points, nx/2 = M

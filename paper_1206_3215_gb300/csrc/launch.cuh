@@ -53,6 +53,25 @@ template <class K> inline cudaError_t resident_ctas(K kernel, int threads, size_
     return cudaSuccess;
 }
 
+// Launch of a kernel of a chain (grid_wait, grid_trigger in fft_core.cuh): it
+// may start while the kernel before it on the stream still runs, also as a
+// node of a captured graph.
+template <class... KA, class... A>
+inline cudaError_t launch_chain(void (*k)(KA...), unsigned grid, int threads, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1] = {};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, KA(args)...);
+}
+
 template <class Rl, int N, class Op> constexpr bool tunable()
 {
     return sizeof(Rl) == 4 && Op::LEAN && N >= 512 && !SkipsGroups<Op>::value;
@@ -91,8 +110,7 @@ inline cudaError_t launch_row_v(Op op, const TW<Rl> *tw, int64_t rows_total, cud
     int grid = 0;
     if ((e = resident_ctas(k, C::THREADS, C::SMEM, ctas, &grid)) != cudaSuccess) return e;
     if (tiles < grid) grid = int(tiles);
-    k<<<dim3(unsigned(grid)), C::THREADS, C::SMEM, s>>>(op, tw, rows_total);
-    return cudaGetLastError();
+    return launch_chain(k, unsigned(grid), C::THREADS, C::SMEM, s, op, tw, rows_total);
 }
 
 template <class Rl, int N, class Op, int VAR>
@@ -109,8 +127,7 @@ inline cudaError_t launch_col_v(Op op, const TW<Rl> *tw, int64_t nx, int64_t bat
     int grid = 0;
     if ((e = resident_ctas(k, C::THREADS, C::SMEM, ctas, &grid)) != cudaSuccess) return e;
     if (tiles < grid) grid = int(tiles);
-    k<<<dim3(unsigned(grid)), C::THREADS, C::SMEM, s>>>(op, tw, nx, batch);
-    return cudaGetLastError();
+    return launch_chain(k, unsigned(grid), C::THREADS, C::SMEM, s, op, tw, nx, batch);
 }
 
 // PSS_TMA=0 stages column tiles with per-point cp.async copies instead of
@@ -161,9 +178,8 @@ inline cudaError_t launch_col_tma(Op op, const TW<Rl> *tw, int64_t nx, int64_t b
     // returns (a bounded wait that runs out; nothing is left in flight)
     const char *f = getenv("PSS_FAULT");
     const bool inject = f && strcmp(f, "tma_timeout") == 0;
-    k<<<dim3(unsigned(grid)), C::THREADS, smem, s>>>(map, map_half, op, tw, nx, batch, inject ? 64u : TMA_WAIT_LIMIT,
-                                                      inject ? 1 : 0);
-    return cudaGetLastError();
+    return launch_chain(k, unsigned(grid), C::THREADS, smem, s, map, map_half, op, tw, nx, batch,
+                        inject ? 64u : TMA_WAIT_LIMIT, inject ? 1 : 0);
 }
 
 // PSS_COL_LAND=0 keeps the one-buffer tensor-copy column pass for ops that
@@ -205,9 +221,8 @@ inline cudaError_t launch_col_land(Op op, const TW<Rl> *tw, int64_t nx, int64_t 
     if (tiles < grid) grid = int(tiles);
     const char *f = getenv("PSS_FAULT");
     const bool inject = f && strcmp(f, "tma_timeout") == 0;
-    k<<<dim3(unsigned(grid)), 2 * C::THREADS, smem, s>>>(map, op, tw, nx, batch, inject ? 64u : TMA_WAIT_LIMIT,
-                                                          inject ? 1 : 0);
-    return cudaGetLastError();
+    return launch_chain(k, unsigned(grid), 2 * C::THREADS, smem, s, map, op, tw, nx, batch,
+                        inject ? 64u : TMA_WAIT_LIMIT, inject ? 1 : 0);
 }
 
 // PSS_COL_SPLIT=0 keeps the one-part column pass for ops that opted into the
@@ -248,9 +263,8 @@ inline cudaError_t launch_col_split(Op op, const TW<Rl> *tw, int64_t nx, int64_t
     if (2 * tiles < grid) grid = int(2 * tiles);
     const char *f = getenv("PSS_FAULT");
     const bool inject = f && strcmp(f, "tma_timeout") == 0;
-    k<<<dim3(unsigned(grid)), C::THREADS, smem, s>>>(map, op, tw, nx, batch, inject ? 64u : TMA_WAIT_LIMIT,
-                                                      inject ? 1 : 0);
-    return cudaGetLastError();
+    return launch_chain(k, unsigned(grid), C::THREADS, smem, s, map, op, tw, nx, batch,
+                        inject ? 64u : TMA_WAIT_LIMIT, inject ? 1 : 0);
 }
 
 template <class Rl, int N, class Op>

@@ -362,7 +362,6 @@ __global__ void __launch_bounds__(RowCfgOf<Rl, N, Op, VAR>::THREADS, RowCfgOf<Rl
     using Sm = SmemLine<V, C::PADLOG>;
     constexpr int NIN = Op::NIN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (op_idle(op)) return;
     V *const buf = reinterpret_cast<V *>(smem_raw);
     const int lr = threadIdx.x / C::T, t = threadIdx.x % C::T;
     const int64_t tiles = (rows_total + C::ROWS - 1) / C::ROWS;
@@ -381,9 +380,12 @@ __global__ void __launch_bounds__(RowCfgOf<Rl, N, Op, VAR>::THREADS, RowCfgOf<Rl
 
     constexpr bool EARLY = EarlyNext<Op>::value && C::NBUF == 1;
     int64_t tile = blockIdx.x;
-    if (C::NBUF == 2 || EARLY) issue(tile, 0);
     fill_stage_tw<N, C::P>(tw);
     op_prologue<N>(op);
+    grid_wait();
+    grid_trigger(tiles);
+    if (op_idle(op)) return;
+    if (C::NBUF == 2 || EARLY) issue(tile, 0);
     __syncthreads();
     for (int it = 0; tile < tiles; ++it, tile += gridDim.x) {
         int b = 0;
@@ -474,7 +476,6 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, VAR>::THREADS, ColCfgOf<Rl
     using Sm = SmemLine<V, C::PADLOG>;
     constexpr int NIN = Op::NIN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (op_idle(op)) return;
     V *const buf = reinterpret_cast<V *>(smem_raw);
     const int c = threadIdx.x % C::W, t = threadIdx.x / C::W;
     const int64_t groups = kept_groups(op, nx / C::W), tiles = groups * batch;
@@ -492,9 +493,12 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, VAR>::THREADS, ColCfgOf<Rl
     };
 
     int64_t tile = blockIdx.x;
-    if (C::NBUF == 2) issue(tile, 0);
     fill_stage_tw<N, C::P>(tw);
     op_prologue<N>(op);
+    grid_wait();
+    grid_trigger(tiles);
+    if (op_idle(op)) return;
+    if (C::NBUF == 2) issue(tile, 0);
     __syncthreads();
     for (int it = 0; tile < tiles; ++it, tile += gridDim.x) {
         int b = 0;
@@ -587,7 +591,6 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, 0>::THREADS, ColCfgOf<Rl, 
     using Sm = SmemLine<V, C::PADLOG>;
     static_assert(C::NBUF == 1, "one staging buffer");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (op_idle(op)) return;
     // align to 128 bytes by an offset from the shared array itself (an
     // address rebuilt from an integer would lose the shared state space and
     // turn every exchange access into a generic one)
@@ -602,6 +605,9 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, 0>::THREADS, ColCfgOf<Rl, 
     if (threadIdx.x == 0) mbar_init(sbar, 1);
     fill_stage_tw<N, C::P>(tw);
     op_prologue<N>(op);
+    grid_wait();
+    grid_trigger(tiles);
+    if (op_idle(op)) return;
     __syncthreads();
     // thread 0: ask for tile `tl` (the buffer's earlier shared-memory accesses
     // come first)
@@ -745,16 +751,18 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, 0>::THREADS, ColCfgOf<Rl, 
     using Sm = SmemLine<V, C::PADLOG>;
     static_assert(C::NBUF == 1 && C::BLOCK == 1, "one staging buffer; transforms span the CTA");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (op_idle(op)) return;
     V *const buf = reinterpret_cast<V *>(smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u));
     const unsigned sbar = smem_addr(buf + C::BUF);
     __shared__ int item_s;
     const int c = threadIdx.x % C::W, t = threadIdx.x / C::W;
     const int groups = int(kept_groups(op, nx / C::W)), tiles = groups * int(batch);
-    const unsigned epoch = unsigned(*op.epoch) + 1u;
     if (threadIdx.x == 0) mbar_init(sbar, 1);
     fill_stage_tw<N, C::P>(tw);
     op_prologue<N>(op);
+    grid_wait();
+    grid_trigger(2 * tiles);
+    if (op_idle(op)) return;
+    const unsigned epoch = unsigned(*op.epoch) + 1u;
     __syncthreads();
     unsigned parity = 0;
     const int lag = imin(int(gridDim.x), tiles);
@@ -906,7 +914,6 @@ __global__ void __launch_bounds__(2 * ColCfgOf<Rl, N, Op, 0>::THREADS,
     constexpr bool TST = TmaStoreOp<Op>::value;
     constexpr int GB = land_gbuf<C>();  // elements per group buffer (128-byte multiple)
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (op_idle(op)) return;
     V *const xbuf = reinterpret_cast<V *>(smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u));
     V *const land = xbuf + 2 * GB;                      // the dense [N][W] landing block
     const unsigned sbar = smem_addr(land + N * C::W);   // mbarrier of group g at sbar + 8 g
@@ -933,10 +940,13 @@ __global__ void __launch_bounds__(2 * ColCfgOf<Rl, N, Op, 0>::THREADS,
         sts_vol(ctrl, 0);
         sts_vol(ctrl + 4, 0);
         sts_vol(ctrl + 8, 0);
-        issue(int(blockIdx.x), 0);
     }
     fill_stage_tw<N, C::P>(tw);
     op_prologue<N>(op);
+    grid_wait();
+    grid_trigger(tiles);
+    if (op_idle(op)) return;
+    if (threadIdx.x == 0) issue(int(blockIdx.x), 0);
     __syncthreads();
 
     const Sm sm[1] = {Sm{xbuf + grp * GB + c * C::STRIDE}};
