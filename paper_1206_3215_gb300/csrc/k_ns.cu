@@ -88,15 +88,153 @@ __global__ void k_ns_begin(NsField *fs, int64_t batch, int *ctl, int n)
     }
 }
 
+// Row pass of one update for FP32 rows of up to 2048 points: row inverse
+// transforms of C1 and C2, J = Re C1 Re C2 + Im C1 Im C2, row forward
+// transform into c1.
+//
+// All three run through one forward-transform body (F^-1 x = conj(F conj x),
+// exact), and a thread holds one array of P points (at most 128 registers, 16
+// warps per SM; with both arrays in registers 215 and 8): C1's result waits
+// in the second shared-memory line of the row, at the thread's own points,
+// where C2 was staged.  That line is read and written at own points only, so
+// it needs no barrier; its next copy is issued once J is formed, the first
+// line's from the start of the last stage.  NS per step, both arrays in
+// registers -> this: 1024^2 x 4 half spectra 256 -> 234 us, 512^2 x 8
+// 157 -> 152, 512 x 256 x 5 midpoint 89 -> 86; 2048^2 the same.  80 registers
+// (24 warps) spill: 1024^2 x 4 267 us.  Two halves of a CTA carrying C1 and C2
+// side by side: 246 us, 4096^2 940 (64 registers: 280, 1067).
+//
+// Dealiasing (2/3 rule): the columns with 3 |mx| >= nx hold zeros in C1 and C2
+// and are not read, and J is not written there (the column pass skips them,
+// the mask discards J); half spectra: J is written for columns 0 .. nx/2.
+constexpr int NS_ROW_MAX = 2048;
+template <int N> struct NsRowCfg {
+    static constexpr int P = imin(Shape<float>::rowP(N), 16);
+    static constexpr int T = N / P;
+    static constexpr int RT = N <= 256 ? 64 : 256;
+    static constexpr int ROWS = T >= RT ? 1 : RT / T;
+    static constexpr int THREADS = ROWS * T;
+    static constexpr int BLOCK = T <= 32 ? 0 : (ROWS > 1 ? T : 1);  // the barrier of one row's threads
+    static constexpr int PADLOG = pad_log(P);
+    static constexpr int LINE = N + (N >> PADLOG);
+    static constexpr size_t SMEM = size_t(2) * ROWS * LINE * sizeof(float2);
+    static constexpr int MIN_CTAS = imin(imax(512 / THREADS, 1), 16);
+};
+
+template <int N>
+__global__ void __launch_bounds__(NsRowCfg<N>::THREADS, NsRowCfg<N>::MIN_CTAS)
+    k_ns_row(float2 *c1, const float2 *c2, const NsField *fs, int lgy, int dealias, int half, const int *ctl,
+             const float4 *__restrict__ tw, int64_t rows_total)
+{
+    using C = NsRowCfg<N>;
+    using V = float2;
+    using Sm = SmemLine<V, C::PADLOG>;
+    constexpr int P = C::P, T = C::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V *const lines = reinterpret_cast<V *>(smem_raw);
+    const int lr = threadIdx.x / T, t = threadIdx.x % T;
+    const Sm sm{lines + lr * C::LINE}, park{lines + (C::ROWS + lr) * C::LINE};
+    const int64_t tiles = (rows_total + C::ROWS - 1) / C::ROWS;
+    // column x of C1, C2 is not known to be zero
+    auto live_col = [&](int x) { return !dealias || 3 * (x < N / 2 ? x : N - x) < N; };
+    auto issue = [&](int64_t tile, const V *in, const Sm &line) {
+        const int64_t row = tile * C::ROWS + lr;
+        if (tile < tiles && row < rows_total) {
+            const V *p = in + row * N + t;
+#pragma unroll
+            for (int m = 0; m < P; ++m)
+                if (live_col(t + T * m)) cp_async<sizeof(V)>(&line[t + T * m], p + T * m);
+        }
+        cp_async_commit();
+    };
+    fill_stage_tw<N, P>(tw);
+    grid_wait();
+    grid_trigger(tiles);
+    if (ctl[NS_CTL_ACTIVE] == 0) return;
+    int64_t tile = blockIdx.x;
+    issue(tile, c2, park);
+    issue(tile, c1, sm);
+    __syncthreads();
+    for (; tile < tiles; tile += gridDim.x) {
+        const int64_t row = tile * C::ROWS + lr, next = tile + gridDim.x;
+        cp_async_wait<0>();
+        V v[P];
+#pragma unroll
+        for (int m = 0; m < P; ++m) {
+            const V x = sm[t + T * m];
+            v[m] = live_col(t + T * m) ? V{x.x, -x.y} : V{0.0f, 0.0f};
+        }
+        // pass 0: C1, pass 1: C2 (each as F of the conjugate, which leaves the
+        // conjugate of the inverse transform), pass 2: J
+#pragma unroll 1
+        for (int pass = 0; pass < 3; ++pass) {
+            block_fft<N, P, -1, C::BLOCK>(v, sm, t, tw, [&]() {
+                if (pass == 2) {
+                    fft_sync<C::BLOCK>();  // the row's last shared-memory reads are done
+                    issue(next, c1, sm);
+                }
+            });
+            if (pass == 0) {
+#pragma unroll
+                for (int m = 0; m < P; ++m) {
+                    const V w = park[t + T * m];
+                    park[t + T * m] = v[m];
+                    v[m] = live_col(t + T * m) ? V{w.x, -w.y} : V{0.0f, 0.0f};
+                }
+            } else if (pass == 1) {
+#pragma unroll
+                for (int m = 0; m < P; ++m) {
+                    const V w = park[t + T * m];
+                    v[m] = V{fma_rn(w.x, v[m].x, mul_rn(w.y, v[m].y)), 0.0f};
+                }
+                issue(next, c2, park);
+            }
+        }
+        if (row < rows_total && fs[row >> lgy].active) {
+            V *p = c1 + row * N + t;
+#pragma unroll
+            for (int m = 0; m < P; ++m) {
+                const int x = t + T * m;
+                if (live_col(x) && (!half || x <= N / 2)) p[T * m] = v[m];
+            }
+        }
+    }
+    cp_async_wait<0>();
+}
+
 template <class Rl>
 cudaError_t ns_row_pass(V2<Rl> *c1, V2<Rl> *c2, const void *fs, int64_t nx, int64_t ny, int64_t batch,
                         const int *ctl, const TW<Rl> *twx, cudaStream_t s, bool dealias, bool half)
 {
+    const NsField *f = static_cast<const NsField *>(fs);
     int lgy = 0;
-    while ((int64_t(1) << lgy) < ny) ++lgy;  // ny is a power of two
-    return launch_row<Rl>(nx, ny, NsRow<Rl>{c1, c2, static_cast<const NsField *>(fs), lgy, dealias ? 1 : 0, half ? 1 : 0,
-                                            ctl},
-                          twx, batch, s);
+    while ((int64_t(1) << lgy) < ny) ++lgy;  // ny is a power of two: row r belongs to field r >> lgy
+    auto short_rows = [&](auto n) -> cudaError_t {
+        constexpr int N = decltype(n)::value;
+        using C = NsRowCfg<N>;
+        auto k = k_ns_row<N>;
+        static std::atomic<unsigned> done{0};
+        static int ctas[32] = {};
+        cudaError_t e = allow_smem(k, C::SMEM, done);
+        if (e != cudaSuccess) return e;
+        const int64_t rows_total = batch * ny, tiles = (rows_total + C::ROWS - 1) / C::ROWS;
+        int grid = 0;
+        if ((e = resident_ctas(k, C::THREADS, C::SMEM, ctas, &grid)) != cudaSuccess) return e;
+        if (tiles < grid) grid = int(tiles);
+        return launch_chain(k, unsigned(grid), C::THREADS, C::SMEM, s, reinterpret_cast<float2 *>(c1),
+                            reinterpret_cast<const float2 *>(c2), f, lgy, dealias ? 1 : 0, half ? 1 : 0, ctl,
+                            reinterpret_cast<const float4 *>(twx), rows_total);
+    };
+    const NsRow<Rl> op{c1, c2, f, lgy, dealias ? 1 : 0, half ? 1 : 0, ctl};
+    switch (nx) {
+#define PSS_CASE(N)                                                                                       \
+    case N:                                                                                               \
+        if constexpr (sizeof(Rl) == 4 && N <= NS_ROW_MAX) return short_rows(std::integral_constant<int, N>{}); \
+        else return launch_row_n<Rl, N>(op, twx, ny, batch, s);
+        PSS_FOR_EACH_N(PSS_CASE)
+#undef PSS_CASE
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <class Rl>

@@ -119,6 +119,11 @@ template <class Rl> struct NsRow {
     const int *ctl;
     __device__ __forceinline__ bool idle() const { return ctl[NS_CTL_ACTIVE] == 0; }
     __device__ const V2<Rl> *in(int k) const { return k == 0 ? c1 : c2; }
+    // the columns with 3 |mx| >= nx hold zeros in C1 and C2 (dealiasing)
+    template <int N> __device__ __forceinline__ bool live_col(int x) const
+    {
+        return !dealias || 3 * (x < N / 2 ? x : N - x) < N;
+    }
     template <int N, int P, int BLOCK, class Sm>
     __device__ __forceinline__ void row(V2<Rl> (&v)[2][P], int64_t r, bool ok, int t, const Sm (&sm)[2],
                                         const TW<Rl> *tw) const
@@ -137,7 +142,7 @@ template <class Rl> struct NsRow {
 #pragma unroll
         for (int m = 0; m < P; ++m, p += T) {
             const int x = t + T * m;
-            const bool kept = (!dealias || 3 * (x < N / 2 ? x : N - x) < N) && (!half || x <= N / 2);
+            const bool kept = live_col<N>(x) && (!half || x <= N / 2);
             if (live && kept) *p = v[0][m];
         }
     }
