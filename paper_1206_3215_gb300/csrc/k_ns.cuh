@@ -103,9 +103,10 @@ template <class V, class R> __device__ __forceinline__ V ns_deriv(int which, V w
     return V{mul_rn(-fma_rn(kx, w.y, mul_rn(ky, w.x)), s), mul_rn(fma_rn(kx, w.x, -mul_rn(ky, w.y)), s)};
 }
 
-// The row pass keeps both inputs in registers (measured at 4096^2: 0.22 ms
-// with 16 points per thread, double buffer and up to 255 registers, against
-// 0.34 ms in the lean shape with the C1 row parked in shared memory)
+// Row pass of FP64 grids and of rows of 4096 points and more: both inputs in
+// registers, their two transforms interleaved (16 points per thread, double
+// buffer, up to 255 registers).  Shorter FP32 rows run k_ns_row (k_ns.cu).
+// At 4096^2 this form takes 157 us per update, k_ns_row 182.
 template <class Rl> struct NsRow {
     static constexpr int NIN = 2;
     static constexpr bool LEAN = false;
@@ -183,6 +184,11 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
     static constexpr bool LEAN = NS_LEAN;
     static constexpr int PMAX = NS_PMAX;
     static constexpr int NOUT = HALF ? 4 : 2;  // inverse transforms per column
+    // groups of threads that can share a tile (k_col_fan): half spectra in FP32.
+    // With full spectra (two outputs) it is even at best (512 x 256 x 5 midpoint
+    // 88 -> 85 us per step, 256^2 x 8 66 -> 70), in FP64 the repeated transforms
+    // cost what they save (256^2 x 4 229 -> 254)
+    static constexpr int COL_FAN = HALF && sizeof(Rl) == 4 ? NOUT : 0;
     __host__ __device__ static constexpr int pmax(int n) { return ns_pmax(n); }
     V2<Rl> *c1, *c2;        // in: J row transforms (c1); out: C1, C2 of w^{k+1}
     V2<Rl> *w0, *w1, *w2;   // vorticity buffers
@@ -238,30 +244,19 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
                                               const TW<Rl> *tw, int o0, int o1) const
     {
         constexpr int T = N / P;
-        const NsField f = fs[field];
-        const int k = f.k;
-        const int64_t nxf = in_stride;
-        // half spectra: the padding columns beyond nxf/2 carry nothing
-        const bool valid = !HALF || 2 * int64_t(x) <= nxf;
-        const bool live = f.active != 0 && valid;
-        const int64_t base = field * N * nx + x;
-        const V2<Rl> *wn = wb(f.idx) + base;
-        const V2<Rl> *wk = wb(ns_buf(f.idx, k)) + base;
-        V2<Rl> *wk1 = wb(ns_buf(f.idx, k + 1)) + base;
-        const int xs = valid ? x : 0;  // table index (the padding reads column 0's entries)
-        const Rl kx = __ldg(kxo + xs), kxx = __ldg(kx2 + xs), mx = __ldg(keepx + xs);
+        const Point q = point<N>(field, x, t);
         double acc = 0.0;
         float acc_hi = 0.0f, acc_lo = 0.0f;  // FP32: double-float partial of this thread
-        if (f.active && o0 == 0) {  // the update reads w^n, w^k (and J_hat^n) after the forward transform
+        if (q.f.active && o0 == 0) {  // the update reads w^n, w^k (and J_hat^n) after the forward transform
             // by row: thread i of the tile's T W threads asks for rows i, i + T W, ...
             // (one 32-byte row segment of the tile per request)
             const int64_t tb = field * N * nx + (x - x % W);
 #pragma unroll
             for (int r = t * W + x % W; r < N; r += T * W) {
                 const int64_t o = tb + int64_t(r) * nx;
-                prefetch_l2(wb(f.idx) + o);
-                prefetch_l2(wb(ns_buf(f.idx, k)) + o);
-                if (!MID && k > 0) prefetch_l2(jn + o);
+                prefetch_l2(wb(q.f.idx) + o);
+                prefetch_l2(wb(ns_buf(q.f.idx, q.f.k)) + o);
+                if (!MID && q.f.k > 0) prefetch_l2(jn + o);
             }
         }
         // pass 0: J_hat and the update; pass p > 0: output p - 1, a derivative
@@ -272,103 +267,182 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
         // SM than the part that stored it)
 #pragma unroll 1
         for (int pass = o0 == 0 ? 0 : o0 + 1; pass <= o1; ++pass) {
-            if (pass >= 2) {
-                const int out = pass - 1;
-                const int nwhich = HALF ? out >> 1 : out;
-                const bool nmirror = HALF && (out & 1);
-                const Rl sx = nmirror ? -kx : kx;
-                // at -kx a field's transform is conj(IFFT(conj(d(-kx, -ky)) w_hat(kx, ky))):
-                // d(-kx, ky) itself for C1, its negative for C2 = i (kx + i ky) w_hat
-                const Rl sg = (nmirror && nwhich == 1) ? Rl(-1) : Rl(1);
-#pragma unroll
-                for (int m = 0; m < P; ++m) {
-                    const int y = t + T * m;
-                    const int64_t o = int64_t(y) * nx;
-                    const V2<Rl> w1v = live ? __ldcg(wk1 + o) : V2<Rl>{0, 0};
-                    const V2<Rl> a_n = (MID && live) ? ld_stream(wn + o) : V2<Rl>{0, 0};
-                    const V2<Rl> d = ns_deriv(nwhich, jfield(w1v, a_n), sx, __ldg(kyo + y), kxx + __ldg(ky2 + y),
-                                              inv_n2);
-                    v[m] = V2<Rl>{sg * d.x, sg * d.y};
-                }
-            }
+            if (pass >= 2) rebuild<N, P>(v, q, pass - 1);
             if (pass > 0) conj_all(v);
             block_fft<N, P, -1, BLOCK>(v, sm, t, tw);
-            if (pass == 0) {
-                // loads of CH points ahead of their stores (the buffers may alias
-                // as far as the compiler knows, so it would not reorder them)
-                constexpr int CH = 4;
-                V2<Rl> ln[CH], lk[CH], lj[CH];
-#pragma unroll
-                for (int m = 0; m < P; ++m) {
-                    const int y = t + T * m;
-                    const int64_t o = int64_t(y) * nx;
-                    if (m % CH == 0)
-#pragma unroll
-                        for (int c = 0; c < CH && m + c < P; ++c) {
-                            const int64_t oc = int64_t(t + T * (m + c)) * nx;
-                            ln[c] = live ? ld_stream(wn + oc) : V2<Rl>{0, 0};
-                            lk[c] = live ? ld_stream(wk + oc) : V2<Rl>{0, 0};
-                            if (!MID && k > 0) lj[c] = live ? ld_stream(jn + base + oc) : V2<Rl>{0, 0};
-                        }
-                    const Rl mask = mul_rn(mx, __ldg(keepy + y));
-                    const V2<Rl> jk{mul_rn(v[m].x, mask), mul_rn(v[m].y, mask)};
-                    // midpoint: jk is already J((w^k + w^n)/2), used twice below
-                    V2<Rl> jnv = jk;
-                    if constexpr (!MID) {
-                        if (k == 0) {
-                            if (live) jn[base + o] = jk;
-                        } else {
-                            jnv = live ? lj[m % CH] : jk;
-                        }
-                    }
-                    const V2<Rl> a_n = ln[m % CH];
-                    const V2<Rl> a_k = lk[m % CH];
-                    const Rl kk = kxx + __ldg(ky2 + y);
-                    // w^{k+1} = [(1 - a) w^n - dt/2 (J^k + J^n)] / (1 + a), a = dt nu |k|^2 / 2,
-                    // formed as w^n minus a small increment so that FP32 rounds
-                    // the increment, not the nearly-unit decay factor, every step
-                    const Rl a = mul_rn(half_dt_nu, kk);
-                    const Rl inv = ns_rcp(Rl(1) + a);  // correctly rounded, as 1 / (1 + a)
-                    const Rl a2 = Rl(2) * a;           // exact
-                    const V2<Rl> inc{mul_rn(fma_rn(a2, a_n.x, mul_rn(half_dt, jk.x + jnv.x)), inv),
-                                     mul_rn(fma_rn(a2, a_n.y, mul_rn(half_dt, jk.y + jnv.y)), inv)};
-                    const V2<Rl> w1v{a_n.x - inc.x, a_n.y - inc.y};
-                    if constexpr (sizeof(Rl) == 4) {
-                        // w^{k+1} - w^k: exact in FP32 once the iterates agree to a
-                        // factor of two (Sterbenz), one rounding before that
-                        if (valid) {
-                            df_add_sq(acc_hi, acc_lo, w1v.x - a_k.x);
-                            df_add_sq(acc_hi, acc_lo, w1v.y - a_k.y);
-                        }
-                    } else {
-                        const double ex = double(w1v.x) - double(a_k.x), ey = double(w1v.y) - double(a_k.y);
-                        if (valid) acc += ex * ex + ey * ey;
-                    }
-                    if (live) wk1[o] = w1v;
-                    v[m] = ns_deriv(0, jfield(w1v, a_n), kx, __ldg(kyo + y), kk, inv_n2);
-                }
-            } else {
-                // output pass - 1: C1 or C2, at kx or (half spectra) mirrored at nxf - kx
-                const int out = pass - 1;
-                const int which = HALF ? out >> 1 : out;
-                const bool mirror = HALF && (out & 1);
-                if (!mirror) conj_all(v);  // the mirrored column stores the conjugate
-                const bool dup = mirror && (x == 0 || 2 * int64_t(x) == nxf);
-                V2<Rl> *dst = (which == 0 ? c1 : c2) + field * N * nxf + (mirror ? nxf - x : x);
-                store_line<P, T>(v, dst, nxf, t, live && !dup);
-            }
+            if (pass == 0) update<N, P>(v, q, 0, true, acc, acc_hi, acc_lo);
+            else store_output<N, P>(v, q, pass - 1);
         }
-        if (o0 == 0) {
-            // FP64 partial of |w^{k+1} - w^k|^2 over this tile, folded in a fixed order
-            const int64_t g = x / W;
-            if constexpr (sizeof(Rl) == 4) acc = double(acc_hi) + double(acc_lo);
-            block_partial<BLOCK>(acc, partials + field * (nx / W - skip_n) + (g < skip_lo ? g : g - skip_n));
+        if (o0 == 0) write_partial<BLOCK>(q, acc, acc_hi, acc_lo);
+    }
+    // Column pass of a tile by F groups of threads (k_col_fan): each group
+    // transforms J and makes the update by itself, group 0 stores it, and
+    // group g forms and transforms outputs g, g + F, ...; all groups of the
+    // CTA call this together.
+    template <int N, int P, int BLOCK, int F, class Sm>
+    __device__ __forceinline__ void col_fan(V2<Rl> (&v)[P], int64_t field, int x, int t, const Sm &sm,
+                                            const TW<Rl> *tw, int grp) const
+    {
+        const Point q = point<N>(field, x, t);
+        double acc = 0.0;
+        float acc_hi = 0.0f, acc_lo = 0.0f;
+        block_fft<N, P, -1, BLOCK>(v, sm, t, tw);
+        update<N, P>(v, q, grp, grp == 0, acc, acc_hi, acc_lo);
+        if constexpr (F < NOUT) __syncthreads();  // the stored iterate is complete
+#pragma unroll 1
+        for (int out = grp; out < NOUT; out += F) {
+            if (out != grp) rebuild<N, P>(v, q, out);
+            conj_all(v);
+            block_fft<N, P, -1, BLOCK>(v, sm, t, tw);
+            store_output<N, P>(v, q, out);
+        }
+        if (grp == 0) write_partial<BLOCK>(q, acc, acc_hi, acc_lo);
+    }
+
+    // what a thread needs to know of its column
+    struct Point {
+        NsField f;
+        bool valid, live;
+        int64_t field, base;
+        int x, t;
+        Rl kx, kxx, mx;
+        const V2<Rl> *wn, *wk;  // w^n, w^k at the column's row 0
+        V2<Rl> *wk1;            // w^{k+1}
+    };
+    template <int N> __device__ __forceinline__ Point point(int64_t field, int x, int t) const
+    {
+        Point q;
+        q.f = fs[field];
+        // half spectra: the padding columns beyond nxf/2 carry nothing
+        q.valid = !HALF || 2 * int64_t(x) <= in_stride;
+        q.live = q.f.active != 0 && q.valid;
+        q.field = field;
+        q.base = field * N * nx + x;
+        q.x = x;
+        q.t = t;
+        q.wn = wb(q.f.idx) + q.base;
+        q.wk = wb(ns_buf(q.f.idx, q.f.k)) + q.base;
+        q.wk1 = wb(ns_buf(q.f.idx, q.f.k + 1)) + q.base;
+        const int xs = q.valid ? x : 0;  // table index (the padding reads column 0's entries)
+        q.kx = __ldg(kxo + xs);
+        q.kxx = __ldg(kx2 + xs);
+        q.mx = __ldg(keepx + xs);
+        return q;
+    }
+    // output `out`: C1 or C2 (which), at kx or (half spectra) mirrored at nxf - kx
+    static __device__ __forceinline__ int out_which(int out) { return HALF ? out >> 1 : out; }
+    static __device__ __forceinline__ bool out_mirror(int out) { return HALF && (out & 1); }
+    // the spectrum of output `out` of the column's field w1v (a_n: w^n), at row y
+    __device__ __forceinline__ V2<Rl> out_spectrum(const Point &q, int out, V2<Rl> w1v, V2<Rl> a_n, int y, Rl kk) const
+    {
+        const int nwhich = out_which(out);
+        const bool nmirror = out_mirror(out);
+        const Rl sx = nmirror ? -q.kx : q.kx;
+        // at -kx a field's transform is conj(IFFT(conj(d(-kx, -ky)) w_hat(kx, ky))):
+        // d(-kx, ky) itself for C1, its negative for C2 = i (kx + i ky) w_hat
+        const Rl sg = (nmirror && nwhich == 1) ? Rl(-1) : Rl(1);
+        const V2<Rl> d = ns_deriv(nwhich, jfield(w1v, a_n), sx, __ldg(kyo + y), kk, inv_n2);
+        return V2<Rl>{sg * d.x, sg * d.y};
+    }
+    template <int N, int P> __device__ __forceinline__ void rebuild(V2<Rl> (&v)[P], const Point &q, int out) const
+    {
+        constexpr int T = N / P;
+#pragma unroll
+        for (int m = 0; m < P; ++m) {
+            const int y = q.t + T * m;
+            const int64_t o = int64_t(y) * nx;
+            const V2<Rl> w1v = q.live ? __ldcg(q.wk1 + o) : V2<Rl>{0, 0};
+            const V2<Rl> a_n = (MID && q.live) ? ld_stream(q.wn + o) : V2<Rl>{0, 0};
+            v[m] = out_spectrum(q, out, w1v, a_n, y, q.kxx + __ldg(ky2 + y));
         }
     }
+    template <int N, int P> __device__ __forceinline__ void store_output(V2<Rl> (&v)[P], const Point &q, int out) const
+    {
+        const bool mirror = out_mirror(out);
+        if (!mirror) conj_all(v);  // the mirrored column stores the conjugate
+        const int64_t nxf = in_stride;
+        const bool dup = mirror && (q.x == 0 || 2 * int64_t(q.x) == nxf);
+        V2<Rl> *dst = (out_which(out) == 0 ? c1 : c2) + q.field * N * nxf + (mirror ? nxf - q.x : q.x);
+        store_line<P, N / P>(v, dst, nxf, q.t, q.live && !dup);
+    }
+    // the update of a column whose J_hat (before the mask) is in v; leaves the
+    // spectrum of output `out` there.  `store`: the new iterate and (k = 0) J_hat^n
+    // are stored
+    template <int N, int P>
+    __device__ __forceinline__ void update(V2<Rl> (&v)[P], const Point &q, int out, bool store, double &acc,
+                                           float &acc_hi, float &acc_lo) const
+    {
+        constexpr int T = N / P;
+        const int k = q.f.k, t = q.t;
+        const V2<Rl> *wn = q.wn, *wk = q.wk;
+        V2<Rl> *wk1 = q.wk1;
+        const bool live = q.live, valid = q.valid;
+        // loads of CH points ahead of their stores (the buffers may alias
+        // as far as the compiler knows, so it would not reorder them)
+        constexpr int CH = 4;
+        V2<Rl> ln[CH], lk[CH], lj[CH];
+#pragma unroll
+        for (int m = 0; m < P; ++m) {
+            const int y = t + T * m;
+            const int64_t o = int64_t(y) * nx;
+            if (m % CH == 0)
+#pragma unroll
+                for (int c = 0; c < CH && m + c < P; ++c) {
+                    const int64_t oc = int64_t(t + T * (m + c)) * nx;
+                    ln[c] = live ? ld_stream(wn + oc) : V2<Rl>{0, 0};
+                    lk[c] = live ? ld_stream(wk + oc) : V2<Rl>{0, 0};
+                    if (!MID && k > 0) lj[c] = live ? ld_stream(jn + q.base + oc) : V2<Rl>{0, 0};
+                }
+            const Rl mask = mul_rn(q.mx, __ldg(keepy + y));
+            const V2<Rl> jk{mul_rn(v[m].x, mask), mul_rn(v[m].y, mask)};
+            // midpoint: jk is already J((w^k + w^n)/2), used twice below
+            V2<Rl> jnv = jk;
+            if constexpr (!MID) {
+                if (k == 0) {
+                    if (live && store) jn[q.base + o] = jk;
+                } else {
+                    jnv = live ? lj[m % CH] : jk;
+                }
+            }
+            const V2<Rl> a_n = ln[m % CH];
+            const V2<Rl> a_k = lk[m % CH];
+            const Rl kk = q.kxx + __ldg(ky2 + y);
+            // w^{k+1} = [(1 - a) w^n - dt/2 (J^k + J^n)] / (1 + a), a = dt nu |k|^2 / 2,
+            // formed as w^n minus a small increment so that FP32 rounds
+            // the increment, not the nearly-unit decay factor, every step
+            const Rl a = mul_rn(half_dt_nu, kk);
+            const Rl inv = ns_rcp(Rl(1) + a);  // correctly rounded, as 1 / (1 + a)
+            const Rl a2 = Rl(2) * a;           // exact
+            const V2<Rl> inc{mul_rn(fma_rn(a2, a_n.x, mul_rn(half_dt, jk.x + jnv.x)), inv),
+                             mul_rn(fma_rn(a2, a_n.y, mul_rn(half_dt, jk.y + jnv.y)), inv)};
+            const V2<Rl> w1v{a_n.x - inc.x, a_n.y - inc.y};
+            if constexpr (sizeof(Rl) == 4) {
+                // w^{k+1} - w^k: exact in FP32 once the iterates agree to a
+                // factor of two (Sterbenz), one rounding before that
+                if (valid) {
+                    df_add_sq(acc_hi, acc_lo, w1v.x - a_k.x);
+                    df_add_sq(acc_hi, acc_lo, w1v.y - a_k.y);
+                }
+            } else {
+                const double ex = double(w1v.x) - double(a_k.x), ey = double(w1v.y) - double(a_k.y);
+                if (valid) acc += ex * ex + ey * ey;
+            }
+            if (live && store) wk1[o] = w1v;
+            v[m] = out_spectrum(q, out, w1v, a_n, y, kk);
+        }
+    }
+    // FP64 partial of |w^{k+1} - w^k|^2 over this tile, folded in a fixed order
+    template <int BLOCK>
+    __device__ __forceinline__ void write_partial(const Point &q, double acc, float acc_hi, float acc_lo) const
+    {
+        const int64_t g = q.x / W;
+        if constexpr (sizeof(Rl) == 4) acc = double(acc_hi) + double(acc_lo);
+        block_partial<BLOCK>(acc, partials + q.field * (nx / W - skip_n) + (g < skip_lo ? g : g - skip_n));
+    }
     // sum over the threads of the tile in a fixed tree; the tile's first
-    // thread writes.  BLOCK <= 1: the tile is the CTA; BLOCK > 1: a group of
-    // BLOCK threads of a CTA that holds two tiles (its own named barrier, its
-    // own warps' slots)
+    // thread writes.  BLOCK = 0: the tile is one warp; 1: the CTA; BLOCK > 1: a
+    // group of BLOCK threads of a CTA (its own named barrier, its own warps'
+    // slots)
     template <int BLOCK> __device__ __forceinline__ void block_partial(double acc, double *out) const
     {
         __shared__ double red[32];
@@ -384,6 +458,8 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
                 for (int i = 0; i < BLOCK / 32; ++i) s += red[warp + i];
                 *out = s;
             }
+        } else if constexpr (BLOCK == 0) {
+            if (lane == 0) *out = acc;  // the tile is one warp (or less)
         } else {
             __syncthreads();
             if (lane == 0) red[warp] = acc;

@@ -267,6 +267,40 @@ inline cudaError_t launch_col_split(Op op, const TW<Rl> *tw, int64_t nx, int64_t
                         inject ? 64u : TMA_WAIT_LIMIT, inject ? 1 : 0);
 }
 
+// PSS_COL_FAN=0 keeps one group of threads per tile (read per launch)
+inline bool fan_enabled()
+{
+    const char *e = getenv("PSS_COL_FAN");
+    return !(e && e[0] == '0' && e[1] == 0);
+}
+
+// Several groups per tile (k_col_fan): the most (NOUT or half of them) with
+// which all tiles run at once, 512 threads per SM (more threads than that
+// take turns, and the repeated forward transforms and updates are lost);
+// whole warps per group, CTAs of at most 512 threads.  Returns false where it
+// does not apply.
+template <class Rl, int N, class Op, int F>
+inline bool launch_col_fan(Op op, const TW<Rl> *tw, int64_t nx, int64_t batch, cudaStream_t s, cudaError_t *out)
+{
+    using C = ColCfgOf<Rl, N, Op, 0>;
+    constexpr size_t smem = size_t(F) * C::BUF * sizeof(V2<Rl>);
+    if constexpr (F < 2 || C::THREADS % 32 != 0 || F * C::THREADS > 512 || smem > SMEM_LIMIT) {
+        if constexpr (F > 2) return launch_col_fan<Rl, N, Op, F / 2>(op, tw, nx, batch, s, out);
+        else return false;
+    } else {
+        const int64_t tiles = kept_groups(op, nx / C::W) * batch;
+        if (tiles * F * C::THREADS > int64_t(GRID_SMS) * 512) {
+            if constexpr (F > 2) return launch_col_fan<Rl, N, Op, F / 2>(op, tw, nx, batch, s, out);
+            else return false;
+        }
+        auto k = k_col_fan<Rl, N, Op, F>;
+        static std::atomic<unsigned> done{0};
+        if ((*out = allow_smem(k, smem, done)) != cudaSuccess || tiles <= 0) return true;
+        *out = launch_chain(k, unsigned(tiles), F * C::THREADS, smem, s, op, tw, nx, batch);
+        return true;
+    }
+}
+
 template <class Rl, int N, class Op>
 inline cudaError_t launch_row_n(Op op, const TW<Rl> *tw, int64_t ny, int64_t batch, cudaStream_t s)
 {
@@ -287,6 +321,10 @@ inline cudaError_t launch_col_n(Op op, const TW<Rl> *tw, int64_t nx, int64_t bat
     if constexpr (short_variant<Rl>(N)) {
         static_assert(!tma_col<Rl, N, Op>(), "variant 2 has no tensor-copy pass");
         if (N * nx <= SMALL_FIELD) return launch_col_v<Rl, N, Op, 2>(op, tw, nx, batch, s);
+    }
+    if constexpr (FanOp<Op>::value > 0) {
+        cudaError_t e;
+        if (fan_enabled() && launch_col_fan<Rl, N, Op, FanOp<Op>::value>(op, tw, nx, batch, s, &e)) return e;
     }
     if constexpr (tunable<Rl, N, Op>()) {
         static PlanSlot slot;

@@ -1019,6 +1019,50 @@ __global__ void __launch_bounds__(2 * ColCfgOf<Rl, N, Op, 0>::THREADS,
 }
 
 // ----------------------------------------------------------------------------
+// Column pass with F groups of threads per tile, for ops with several
+// transforms per tile (Navier-Stokes: one forward, two or four inverse) on
+// grids too small to fill the SMs with one group per tile: every group holds
+// the tile (C::THREADS threads, its own exchange buffer), does the forward
+// transform by itself and then its share of the outputs, so that a tile takes
+// 1 + NOUT / F transforms one after the other instead of 1 + NOUT.  An op opts
+// in with COL_FAN = its largest F.  The tile is read straight into registers;
+// the CTA barrier after that orders the reads of the input before the outputs
+// that overwrite it.
+template <class Op, class = void> struct FanOp : std::integral_constant<int, 0> {};
+template <class Op> struct FanOp<Op, std::void_t<decltype(Op::COL_FAN)>> : std::integral_constant<int, Op::COL_FAN> {};
+
+template <class Rl, int N, class Op, int F>
+__global__ void __launch_bounds__(F *ColCfgOf<Rl, N, Op, 0>::THREADS,
+                                  imax(1, 512 / (F * ColCfgOf<Rl, N, Op, 0>::THREADS)))
+    k_col_fan(Op op, const TW<Rl> *__restrict__ tw, int64_t nx, int64_t batch)
+{
+    using C = ColCfgOf<Rl, N, Op, 0>;
+    using V = V2<Rl>;
+    using Sm = SmemLine<V, C::PADLOG>;
+    constexpr int G = C::THREADS, BLOCK = G == 32 ? 0 : G;
+    static_assert(G % 32 == 0 && F * G <= 512 && Op::NIN == 1, "whole warps per group");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int grp = threadIdx.x / G, tg = threadIdx.x % G, c = tg % C::W, t = tg / C::W;
+    const Sm sm{reinterpret_cast<V *>(smem_raw) + grp * C::BUF + c * C::STRIDE};
+    const int64_t groups = kept_groups(op, nx / C::W), tiles = groups * batch;
+    fill_stage_tw<N, C::P>(tw);
+    grid_wait();
+    grid_trigger(tiles);
+    if (op_idle(op)) return;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t field = tile / groups;
+        const int x = int(group_index(op, tile % groups) * C::W + c);
+        V v[C::P];
+        const V *p = col_in(op, 0, field) + (field * N + t) * in_stride(op, nx) + x;
+        const int64_t step = int64_t(C::T) * in_stride(op, nx);
+#pragma unroll
+        for (int m = 0; m < C::P; ++m, p += step) v[m] = *p;
+        __syncthreads();  // (also: the twiddle copy is filled)
+        op.template col_fan<N, C::P, BLOCK, F>(v, field, x, t, sm, tw, grp);
+    }
+}
+
+// ----------------------------------------------------------------------------
 // Store helper: register m -> element t + T m of a line with stride st
 template <int P, int T, class V>
 __device__ __forceinline__ void store_line(const V (&v)[P], V *__restrict__ p, int64_t st, int t,
