@@ -50,9 +50,15 @@ template <class Rl> struct SgRow {
                 block_fft<N, P, -1, BLOCK>(v, sm[0], t, tw, [&]() {
                     if (pass == 1) hook();
                 });
-                if (pass == 0)  // u = Re F^-1 H = Re conj(F conj H) = Re F conj H
+                if (pass == 0) {  // u = Re F^-1 H = Re conj(F conj H) = Re F conj H
+                    if (sg_all_small(v, false)) {
 #pragma unroll
-                    for (int m = 0; m < P; ++m) v[m] = V2<Rl>{sin_(v[m].x), Rl(0)};
+                        for (int m = 0; m < P; ++m) v[m] = V2<Rl>{sg_sin_poly(v[m].x), Rl(0)};
+                    } else {
+#pragma unroll
+                        for (int m = 0; m < P; ++m) v[m] = V2<Rl>{sin_(v[m].x), Rl(0)};
+                    }
+                }
             }
         } else {
             block_fft<N, P, +1, BLOCK>(v, sm[0], t, tw);
@@ -79,7 +85,12 @@ template <class Rl> struct SgCol {
     int64_t nx;
     int *status;        // set when a tile copy did not arrive
     __host__ __device__ const V2<Rl> *in(int) const { return h; }
-    template <int N, int P, int BLOCK, class Sm>
+    // arrays of the tile that the update reads after the forward transform: the
+    // tensor-copy pass asks for them to be brought into L2, one request each
+    // (PF: it has done so; else every thread asks for its points)
+    static constexpr bool COL_PREFETCH = true;
+    __host__ __device__ const V2<Rl> *later(int k) const { return k == 0 ? u : d; }
+    template <int N, int P, int BLOCK, class Sm, bool PF = false>
     __device__ __forceinline__ void col(V2<Rl> (&vv)[1][P], int64_t field, int x, int t,
                                         const Sm (&sm)[1], const TW<Rl> *tw) const
     {
@@ -87,7 +98,7 @@ template <class Rl> struct SgCol {
         V2<Rl>(&v)[P] = vv[0];
         const int64_t base = field * N * nx + x;
         const int64_t step = int64_t(T) * nx;
-        {
+        if constexpr (!PF) {
             // u and d are read only after the forward transform: have them in L2 by then
             const V2<Rl> *qu = u + base + int64_t(t) * nx, *qd = d + base + int64_t(t) * nx;
 #pragma unroll

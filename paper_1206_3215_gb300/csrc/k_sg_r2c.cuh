@@ -127,9 +127,16 @@ __global__ void __launch_bounds__(R2cCfg<Rl, M, SMALL>::THREADS, R2cCfg<Rl, M, S
 #pragma unroll 1
         for (int pass = MODE == HalfRow::STEP ? 0 : 1; pass < 2; ++pass) {
             block_fft<M, P, -1, C::BLOCK>(v, sm, t, twm);
-            if (MODE == HalfRow::STEP && pass == 0)  // z = conj(F conj Z): u_{2j} = Re z, u_{2j+1} = Im z = -Im(F conj Z)
+            if (MODE == HalfRow::STEP && pass == 0) {
+                // z = conj(F conj Z): u_{2j} = Re z, u_{2j+1} = Im z = -Im(F conj Z)
+                if (sg_all_small(v, true)) {
 #pragma unroll
-                for (int m = 0; m < P; ++m) v[m] = V{sg_sin(v[m].x), sg_sin(-v[m].y)};
+                    for (int m = 0; m < P; ++m) v[m] = V{sg_sin_poly(v[m].x), sg_sin_poly(-v[m].y)};
+                } else {
+#pragma unroll
+                    for (int m = 0; m < P; ++m) v[m] = V{sg_sin(v[m].x), sg_sin(-v[m].y)};
+                }
+            }
         }
         if constexpr (MODE == HalfRow::JOIN) {
             if (ok)

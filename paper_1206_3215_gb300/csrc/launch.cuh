@@ -159,7 +159,7 @@ inline cudaError_t launch_col_tma(Op op, const TW<Rl> *tw, int64_t nx, int64_t b
     const int64_t tiles = kept_groups(op, nx / C::W) * batch;
     if (tiles <= 0) return cudaSuccess;
     if (tiles > INT32_MAX - 2 * 65536) return cudaErrorInvalidValue;  // the kernel counts tiles in 32 bits
-    CUtensorMap map, map_half;
+    CUtensorMap map, map_half, map_later;
     if ((e = encode_col_map(&map, op.in(0), int(sizeof(V2<Rl>)), in_stride(op, nx), N, batch, C::W)) != cudaSuccess)
         return e;
     // the half-tile store box (the op writes its input array in place)
@@ -170,6 +170,15 @@ inline cudaError_t launch_col_tma(Op op, const TW<Rl> *tw, int64_t nx, int64_t b
     } else {
         map_half = map;
     }
+    map_later = map;
+    if constexpr (ColPrefetch<Op>::value) {
+        static_assert(!HS::ON, "map_half is the first later array's");
+        if ((e = encode_col_map(&map_half, op.later(0), int(sizeof(V2<Rl>)), in_stride(op, nx), N, batch, C::W)) !=
+                cudaSuccess ||
+            (e = encode_col_map(&map_later, op.later(1), int(sizeof(V2<Rl>)), in_stride(op, nx), N, batch, C::W)) !=
+                cudaSuccess)
+            return e;
+    }
     int grid = 0;
     if ((e = resident_ctas(k, C::THREADS, smem, ctas, &grid)) != cudaSuccess) return e;
     if (tiles < grid) grid = int(tiles);
@@ -178,7 +187,7 @@ inline cudaError_t launch_col_tma(Op op, const TW<Rl> *tw, int64_t nx, int64_t b
     // returns (a bounded wait that runs out; nothing is left in flight)
     const char *f = getenv("PSS_FAULT");
     const bool inject = f && strcmp(f, "tma_timeout") == 0;
-    return launch_chain(k, unsigned(grid), C::THREADS, smem, s, map, map_half, op, tw, nx, batch,
+    return launch_chain(k, unsigned(grid), C::THREADS, smem, s, map, map_half, map_later, op, tw, nx, batch,
                         inject ? 64u : TMA_WAIT_LIMIT, inject ? 1 : 0);
 }
 

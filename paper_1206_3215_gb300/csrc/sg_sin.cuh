@@ -23,6 +23,27 @@ constexpr float C3 = float((HI - double(C1) - double(C2)) + LO);
 #define PSS_SG_LIBM_SIN 0
 #endif
 
+// sin r on [-pi/4, pi/4]
+__device__ __forceinline__ float sg_sin_poly(float r)
+{
+    const float r2 = r * r;
+    return __fmaf_rn(r * r2, -1.0f / 6 + r2 * (1.0f / 120 + r2 * (-1.0f / 5040 + r2 * (1.0f / 362880))), r);
+}
+// largest |u| that needs no reduction (k = 0 below): sg_sin is sg_sin_poly there
+constexpr float sg_sin_small = 0.785f;
+// whether every value of a thread is that small: its passes then run the sine
+// polynomial alone, 6 instead of 22 instructions per point (2048^2 x 8 half
+// spectra row pass 127 -> 117 us)
+template <int P> __device__ __forceinline__ bool sg_all_small(const float2 (&v)[P], bool both)
+{
+    float big = 0.0f;
+#pragma unroll
+    for (int m = 0; m < P; ++m) big = fmaxf(big, both ? fmaxf(fabsf(v[m].x), fabsf(v[m].y)) : fabsf(v[m].x));
+    return big <= sg_sin_small;
+}
+template <int P> __device__ __forceinline__ bool sg_all_small(const double2 (&)[P], bool) { return false; }
+__device__ __forceinline__ double sg_sin_poly(double x) { return sin(x); }
+
 __device__ __forceinline__ float sg_sin(float x)
 {
     if constexpr (PSS_SG_LIBM_SIN) return sinf(x);
@@ -31,7 +52,7 @@ __device__ __forceinline__ float sg_sin(float x)
     r = __fmaf_rn(-k, sgsin::C2, r);
     r = __fmaf_rn(-k, sgsin::C3, r);
     const float r2 = r * r;
-    const float sn = __fmaf_rn(r * r2, -1.0f / 6 + r2 * (1.0f / 120 + r2 * (-1.0f / 5040 + r2 * (1.0f / 362880))), r);
+    const float sn = sg_sin_poly(r);
     const float cs = 1.0f + r2 * (-0.5f + r2 * (1.0f / 24 + r2 * (-1.0f / 720 + r2 * (1.0f / 40320 + r2 * (-1.0f / 3628800)))));
     const int q = int(k) & 3;
     const float v = (q & 1) ? cs : sn;
