@@ -367,12 +367,19 @@ int pss_grid::check_ns_nonconv()
 
 namespace {
 
-template <class Rl> int nls_set(pss_grid *g, const void *a, int where)
+// fields f .. f + nb - 1 from the caller's array: straight through the row
+// transform where a kernel can read it, else copied first
+template <class Rl> int nls_set(pss_grid *g, int64_t f, int64_t nb, const void *a, int where)
 {
-    int rc = g->cuda(cudaMemcpyAsync(g->buf[0], a, g->field_bytes(), kind_in(where), g->stream), "set_state copy");
-    if (rc) return rc;
-    rc = g->cuda(fft_rows<Rl>(B<Rl>(g, 0), g->nx, g->ny, g->batch, -1, Rl(1), Tw<Rl>(g->twx), g->stream),
-                 "set_state row fft");
+    V2<Rl> *dst = B<Rl>(g, 0) + f * g->npts;
+    const V2<Rl> *src = dst;
+    int rc;
+    if (where == PSS_DEVICE && kernel_access(a, sizeof(V2<Rl>)))
+        src = C<Rl>(a);
+    else if ((rc = g->cuda(cudaMemcpyAsync(dst, a, size_t(nb * g->npts) * g->esz, kind_in(where), g->stream),
+                           "set_state copy")))
+        return rc;
+    rc = g->cuda(fft_rows<Rl>(src, dst, g->nx, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twx), g->stream), "set_state row fft");
     if (rc) return rc;
     if (where == PSS_HOST) return g->cuda(cudaStreamSynchronize(g->stream), "set_state sync");
     return PSS_OK;
@@ -405,34 +412,30 @@ template <class Rl> int nls_step(pss_grid *g, int64_t n)
     return g->cuda(e, "nls step");
 }
 
-// psi (physical) into buf[1]
-template <class Rl> int nls_physical(pss_grid *g)
+// psi (physical) of fields f .. f + nb - 1 into dst
+template <class Rl> int nls_physical(pss_grid *g, int64_t f, int64_t nb, V2<Rl> *dst)
 {
-    int rc = g->cuda(cudaMemcpyAsync(g->buf[1], g->buf[0], g->field_bytes(), cudaMemcpyDeviceToDevice, g->stream),
-                     "copy");
-    if (rc) return rc;
-    return g->cuda(fft_rows<Rl>(B<Rl>(g, 1), g->nx, g->ny, g->batch, +1, Rl(1.0 / double(g->nx)),
+    return g->cuda(fft_rows<Rl>(B<Rl>(g, 0) + f * g->npts, dst, g->nx, g->ny, nb, +1, Rl(1.0 / double(g->nx)),
                                 Tw<Rl>(g->twx), g->stream),
                    "row inverse");
 }
 
-template <class Rl> int nls_get(pss_grid *g, void *a, int where)
+template <class Rl> int nls_get(pss_grid *g, int64_t f, int64_t nb, void *a, int where)
 {
-    int rc = nls_physical<Rl>(g);
-    if (rc) return rc;
-    rc = g->cuda(cudaMemcpyAsync(a, g->buf[1], g->field_bytes(), kind_out(where), g->stream), "get_state copy");
-    if (rc) return rc;
-    return g->sync();
+    const bool direct = where == PSS_DEVICE && kernel_access(a, sizeof(V2<Rl>));
+    V2<Rl> *dst = direct ? static_cast<V2<Rl> *>(a) : B<Rl>(g, 1) + f * g->npts;
+    int rc = nls_physical<Rl>(g, f, nb, dst);
+    if (!rc && !direct)
+        rc = g->cuda(cudaMemcpyAsync(a, dst, size_t(nb * g->npts) * g->esz, kind_out(where), g->stream),
+                     "get_state copy");
+    return rc ? rc : g->sync();
 }
 
 template <class Rl> int nls_conserved(pss_grid *g, double *out)
 {
-    int rc = nls_physical<Rl>(g);
+    int rc = nls_physical<Rl>(g, 0, g->batch, B<Rl>(g, 1));
     if (rc) return rc;
-    rc = g->cuda(cudaMemcpyAsync(g->buf[2], g->buf[0], g->field_bytes(), cudaMemcpyDeviceToDevice, g->stream),
-                 "copy");
-    if (rc) return rc;
-    rc = g->cuda(fft_cols<Rl>(B<Rl>(g, 2), g->nx, g->ny, g->batch, -1, Rl(1), Tw<Rl>(g->twy), g->stream),
+    rc = g->cuda(fft_cols<Rl>(B<Rl>(g, 0), B<Rl>(g, 2), g->nx, g->ny, g->batch, -1, Rl(1), Tw<Rl>(g->twy), g->stream),
                  "col fft");
     if (rc) return rc;
     rc = g->cuda(nls_sums<Rl>(B<Rl>(g, 1), B<Rl>(g, 2), g->nx, g->ny, g->batch, g->kx2d, g->ky2d, g->partials,
@@ -464,10 +467,10 @@ namespace {
 // forward (-1) or inverse (+1, with 1/(nx ny)) 2D transform of buffer b
 template <class Rl> cudaError_t fft2(pss_grid *g, V2<Rl> *b, int dir)
 {
-    cudaError_t e = fft_rows<Rl>(b, g->nx, g->ny, g->batch, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
+    cudaError_t e = fft_rows<Rl>(b, b, g->nx, g->ny, g->batch, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
     if (e != cudaSuccess) return e;
     const Rl sc = dir > 0 ? Rl(1.0 / (double(g->nx) * double(g->ny))) : Rl(1);
-    return fft_cols<Rl>(b, g->nx, g->ny, g->batch, dir, sc, Tw<Rl>(g->twy), g->stream);
+    return fft_cols<Rl>(b, b, g->nx, g->ny, g->batch, dir, sc, Tw<Rl>(g->twy), g->stream);
 }
 
 // real caller array (host or device) -> complex buffer dst (imaginary part 0),
@@ -568,10 +571,10 @@ template <class Rl> int sg_set_fields(pss_grid *g, int64_t f, int64_t nb, const 
     } else {
         e = sg_start_field<Rl>(u, v, st.d, g->p.dt, nb * g->npts, g->stream);
         if (e == cudaSuccess)
-            e = fft_rows<Rl>(st.d, g->nx, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twx), g->stream);
+            e = fft_rows<Rl>(st.d, st.d, g->nx, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twx), g->stream);
     }
     if ((rc = g->cuda(e, "start-up rows")) || (rc = g->cuda(sg_split<Rl>(g, st, u, st.u), "forward rows")) ||
-        (rc = g->cuda(fft_cols<Rl>(st.u, st.w, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
+        (rc = g->cuda(fft_cols<Rl>(st.u, st.u, st.w, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
         (rc = g->cuda(sg_start_cols<Rl>(st.d, st.u, C<Rl>(g->sgcx), C<Rl>(g->sgcy), st.w, g->ny, nb, Tw<Rl>(g->twy),
                                         g->stream), "start-up columns")) ||
         (rc = sg_make_h<Rl>(g, st)))
@@ -589,8 +592,8 @@ template <class Rl> int sg_set_levels(pss_grid *g, const void *un, const void *u
         (rc = sg_real_in<Rl>(g, unm1, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), g->ntot, &b)) ||
         (rc = g->cuda(sg_split<Rl>(g, st, a, st.u), "forward rows")) ||
         (rc = g->cuda(sg_split<Rl>(g, st, b, st.d), "forward rows")) ||
-        (rc = g->cuda(fft_cols<Rl>(st.u, st.w, g->ny, st.nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
-        (rc = g->cuda(fft_cols<Rl>(st.d, st.w, g->ny, st.nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
+        (rc = g->cuda(fft_cols<Rl>(st.u, st.u, st.w, g->ny, st.nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
+        (rc = g->cuda(fft_cols<Rl>(st.d, st.d, st.w, g->ny, st.nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
         (rc = g->cuda(cplx_axpy<Rl>(st.u, st.d, Rl(1), st.d, st.w * g->ny * st.nb, g->stream), "d")) ||
         (rc = sg_make_h<Rl>(g, st)))
         return rc;
@@ -933,10 +936,10 @@ namespace {
 
 template <class Rl> cudaError_t fft2_one(pss_grid *g, V2<Rl> *b, int dir)
 {
-    cudaError_t e = fft_rows<Rl>(b, g->nx, g->ny, 1, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
+    cudaError_t e = fft_rows<Rl>(b, b, g->nx, g->ny, 1, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
     if (e != cudaSuccess) return e;
     const Rl sc = dir > 0 ? Rl(1.0 / (double(g->nx) * double(g->ny))) : Rl(1);
-    return fft_cols<Rl>(b, g->nx, g->ny, 1, dir, sc, Tw<Rl>(g->twy), g->stream);
+    return fft_cols<Rl>(b, b, g->nx, g->ny, 1, dir, sc, Tw<Rl>(g->twy), g->stream);
 }
 
 // real field (host or device) -> complex slot dst_buf[f], through raw scratch slot tmp_buf[f]
@@ -960,11 +963,8 @@ template <class Rl> int store_real_one(pss_grid *g, int64_t f, const V2<Rl> *a, 
 template <class Rl> int field_set(pss_grid *g, int64_t f, const void *a, const void *b, int where)
 {
     int rc = PSS_OK;
-    const size_t fb = size_t(g->npts) * g->esz;
     if (g->p.eq == PSS_EQ_NLS) {
-        if ((rc = g->cuda(cudaMemcpyAsync(Bf<Rl>(g, 0, f), a, fb, kind_in(where), g->stream), "copy")) ||
-            (rc = g->cuda(fft_rows<Rl>(Bf<Rl>(g, 0, f), g->nx, g->ny, 1, -1, Rl(1), Tw<Rl>(g->twx), g->stream), "row fft")))
-            return rc;
+        return nls_set<Rl>(g, f, 1, a, where);
     } else if (g->p.eq == PSS_EQ_SG) {
         return sg_set_fields<Rl>(g, f, 1, a, b, where);
     } else {
@@ -987,14 +987,8 @@ template <class Rl> int field_set(pss_grid *g, int64_t f, const void *a, const v
 template <class Rl> int field_get(pss_grid *g, int64_t f, void *a, void *b, int where)
 {
     int rc;
-    const size_t fb = size_t(g->npts) * g->esz;
     if (g->p.eq == PSS_EQ_NLS) {
-        if ((rc = g->cuda(cudaMemcpyAsync(Bf<Rl>(g, 1, f), Bf<Rl>(g, 0, f), fb, cudaMemcpyDeviceToDevice, g->stream),
-                          "copy")) ||
-            (rc = g->cuda(fft_rows<Rl>(Bf<Rl>(g, 1, f), g->nx, g->ny, 1, +1, Rl(1.0 / double(g->nx)), Tw<Rl>(g->twx),
-                                       g->stream), "row inverse")) ||
-            (rc = g->cuda(cudaMemcpyAsync(a, Bf<Rl>(g, 1, f), fb, kind_out(where), g->stream), "copy")))
-            return rc;
+        return nls_get<Rl>(g, f, 1, a, where);
     } else if (g->p.eq == PSS_EQ_SG) {
         return sg_get_fields<Rl>(g, f, 1, a, b, where);
     } else {
@@ -1028,7 +1022,7 @@ int pss_grid::set_state(const void *a, const void *b, int where)
     steps = 0;
     nonconv_pending = false;
     int rc;
-#define NLS(R) nls_set<R>(this, a, where)
+#define NLS(R) nls_set<R>(this, 0, batch, a, where)
 #define SG(R) sg_set_fields<R>(this, 0, batch, a, b, where)
 #define NS(R) ns_set<R>(this, a, where)
     rc = p.eq == PSS_EQ_NLS ? PSS_BY_PRECISION(NLS) : p.eq == PSS_EQ_SG ? PSS_BY_PRECISION(SG) : PSS_BY_PRECISION(NS);
@@ -1154,7 +1148,7 @@ int pss_grid::get_state(void *a, void *b, int where)
 {
     int rc = half_sync(true);
     if (rc) return rc;
-#define NLS(R) nls_get<R>(this, a, where)
+#define NLS(R) nls_get<R>(this, 0, batch, a, where)
 #define SG(R) sg_get_fields<R>(this, 0, batch, a, b, where)
 #define NS(R) ns_get<R>(this, a, where)
     return p.eq == PSS_EQ_NLS ? PSS_BY_PRECISION(NLS) : p.eq == PSS_EQ_SG ? PSS_BY_PRECISION(SG) : PSS_BY_PRECISION(NS);
@@ -1383,13 +1377,13 @@ extern "C" int pss_fft2d(void *data, int64_t nx, int64_t ny, int64_t batch, int 
     cudaError_t e;
     const double inv = direction > 0 ? 1.0 / (double(nx) * double(ny)) : 1.0;
     if (precision == PSS_FP32) {
-        e = fft_rows<float>(static_cast<float2 *>(data), nx, ny, batch, direction, 1.0f, static_cast<float4 *>(twx), s);
+        e = fft_rows<float>(static_cast<float2 *>(data), static_cast<float2 *>(data), nx, ny, batch, direction, 1.0f, static_cast<float4 *>(twx), s);
         if (e == cudaSuccess)
-            e = fft_cols<float>(static_cast<float2 *>(data), nx, ny, batch, direction, float(inv), static_cast<float4 *>(twy), s);
+            e = fft_cols<float>(static_cast<float2 *>(data), static_cast<float2 *>(data), nx, ny, batch, direction, float(inv), static_cast<float4 *>(twy), s);
     } else {
-        e = fft_rows<double>(static_cast<double2 *>(data), nx, ny, batch, direction, 1.0, static_cast<double2 *>(twx), s);
+        e = fft_rows<double>(static_cast<double2 *>(data), static_cast<double2 *>(data), nx, ny, batch, direction, 1.0, static_cast<double2 *>(twx), s);
         if (e == cudaSuccess)
-            e = fft_cols<double>(static_cast<double2 *>(data), nx, ny, batch, direction, inv, static_cast<double2 *>(twy), s);
+            e = fft_cols<double>(static_cast<double2 *>(data), static_cast<double2 *>(data), nx, ny, batch, direction, inv, static_cast<double2 *>(twy), s);
     }
     return e == cudaSuccess ? PSS_OK : PSS_E_CUDA;
 }

@@ -22,11 +22,12 @@ template <class Rl> using TW = typename twid<Rl>::type;
 
 // ---- plain transforms (k_fft.cu) -------------------------------------------
 // dir -1 forward, +1 inverse (unnormalised); the result is multiplied by scale.
+// src == dst: in place.
 template <class Rl>
-cudaError_t fft_rows(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, int dir, Rl scale,
+cudaError_t fft_rows(const V2<Rl> *src, V2<Rl> *dst, int64_t nx, int64_t ny, int64_t batch, int dir, Rl scale,
                      const TW<Rl> *twx, cudaStream_t s);
 template <class Rl>
-cudaError_t fft_cols(V2<Rl> *data, int64_t nx, int64_t ny, int64_t batch, int dir, Rl scale,
+cudaError_t fft_cols(const V2<Rl> *src, V2<Rl> *dst, int64_t nx, int64_t ny, int64_t batch, int dir, Rl scale,
                      const TW<Rl> *twy, cudaStream_t s);
 
 // ---- NLS passes (k_nls.cu) ---------------------------------------------------

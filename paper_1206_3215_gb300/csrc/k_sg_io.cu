@@ -32,14 +32,15 @@ template <class Rl> struct SgLevelCol {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
+    static constexpr bool EARLY_NEXT = true;
     const V2<Rl> *a, *b;
     V2<Rl> *out;
     Rl scale;
     int64_t nx;
     __device__ const V2<Rl> *in(int) const { return a; }
-    template <int N, int P, int BLOCK, class Sm>
+    template <int N, int P, int BLOCK, class Sm, class H = NoHook>
     __device__ __forceinline__ void col(V2<Rl> (&vv)[1][P], int64_t field, int x, int t, const Sm (&sm)[1],
-                                        const TW<Rl> *tw) const
+                                        const TW<Rl> *tw, const H &hook = H{}) const
     {
         constexpr int T = N / P;
         V2<Rl>(&v)[P] = vv[0];
@@ -51,10 +52,10 @@ template <class Rl> struct SgLevelCol {
         for (int m = 0; m < P; ++m) v[m] = cscale(v[m], scale);
         if constexpr (sizeof(Rl) == 4) {
             conj_all(v);
-            block_fft<N, P, -1, BLOCK>(v, sm[0], t, tw);
+            block_fft<N, P, -1, BLOCK>(v, sm[0], t, tw, hook);
             conj_all(v);
         } else {
-            block_fft<N, P, +1, BLOCK>(v, sm[0], t, tw);
+            block_fft<N, P, +1, BLOCK>(v, sm[0], t, tw, hook);
         }
         store_line<P, T>(v, out + base, nx, t, true);
     }
@@ -66,19 +67,20 @@ template <class Rl> struct SgStartCol {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
+    static constexpr bool EARLY_NEXT = true;
     V2<Rl> *data;
     const V2<Rl> *u;
     const V2<Rl> *cx, *cy;  // {hi, lo} of (dt^2/2) k^2 per axis
     int64_t nx;
     __device__ const V2<Rl> *in(int) const { return data; }
-    template <int N, int P, int BLOCK, class Sm>
+    template <int N, int P, int BLOCK, class Sm, class H = NoHook>
     __device__ __forceinline__ void col(V2<Rl> (&vv)[1][P], int64_t field, int x, int t, const Sm (&sm)[1],
-                                        const TW<Rl> *tw) const
+                                        const TW<Rl> *tw, const H &hook = H{}) const
     {
         constexpr int T = N / P;
         V2<Rl>(&v)[P] = vv[0];
         const int64_t base = field * N * nx + x;
-        block_fft<N, P, -1, BLOCK>(v, sm[0], t, tw);
+        block_fft<N, P, -1, BLOCK>(v, sm[0], t, tw, hook);
         const V2<Rl> kx = __ldg(cx + x);
 #pragma unroll
         for (int m = 0; m < P; ++m) {
@@ -99,14 +101,15 @@ template <class Rl> struct RowToReal {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
+    static constexpr bool EARLY_NEXT = true;
     const V2<Rl> *src;
     Rl *dst;
     __device__ const V2<Rl> *in(int) const { return src; }
-    template <int N, int P, int BLOCK, class Sm>
+    template <int N, int P, int BLOCK, class Sm, class H = NoHook>
     __device__ __forceinline__ void row(V2<Rl> (&v)[1][P], int64_t r, bool ok, int t, const Sm (&sm)[1],
-                                        const TW<Rl> *tw) const
+                                        const TW<Rl> *tw, const H &hook = H{}) const
     {
-        block_fft<N, P, +1, BLOCK>(v[0], sm[0], t, tw);
+        block_fft<N, P, +1, BLOCK>(v[0], sm[0], t, tw, hook);
         if (!ok) return;
 #pragma unroll
         for (int m = 0; m < P; ++m) dst[r * N + t + (N / P) * m] = v[0][m].x;
@@ -192,17 +195,18 @@ template <class Rl> struct ColToReal {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
+    static constexpr bool EARLY_NEXT = true;
     const V2<Rl> *src;
     Rl *dst;
     Rl scale;
     int64_t nx;
     __device__ const V2<Rl> *in(int) const { return src; }
-    template <int N, int P, int BLOCK, class Sm>
+    template <int N, int P, int BLOCK, class Sm, class H = NoHook>
     __device__ __forceinline__ void col(V2<Rl> (&v)[1][P], int64_t field, int x, int t, const Sm (&sm)[1],
-                                        const TW<Rl> *tw) const
+                                        const TW<Rl> *tw, const H &hook = H{}) const
     {
         constexpr int T = N / P;
-        block_fft<N, P, +1, BLOCK>(v[0], sm[0], t, tw);
+        block_fft<N, P, +1, BLOCK>(v[0], sm[0], t, tw, hook);
         Rl *p = dst + field * N * nx + x + int64_t(t) * nx;
         const int64_t step = int64_t(T) * nx;
 #pragma unroll

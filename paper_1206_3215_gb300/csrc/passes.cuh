@@ -326,8 +326,8 @@ template <int N, class Op> __device__ __forceinline__ void op_prologue(const Op 
     if constexpr (HasPrologue<Op>::value) op.template prologue<N>();
 }
 
-// An op that sets EARLY_NEXT takes a hook as the last argument of row() and
-// calls it once its last transform has made its last shared-memory access
+// An op that sets EARLY_NEXT takes a hook as the last argument of row() (or
+// col(), k_col) and calls it once its last transform has made its last shared-memory access
 // (block_fft's hook): a single-buffered row pass then issues the copies of
 // its next tile there, under the rest of the tile's arithmetic and stores.
 template <class Op, class = void> struct EarlyNext : std::false_type {};
@@ -434,8 +434,11 @@ __global__ void __launch_bounds__(RowCfgOf<Rl, N, Op, VAR>::THREADS, RowCfgOf<Rl
             const int64_t next = tile + gridDim.x;
             if (PSS_ROW_PREFETCH && t == 0 && next < tiles && next * C::ROWS + lr < rows_total)
 #pragma unroll
-                for (int k = 0; k < NIN; ++k)
-                    bulk_prefetch_l2(op.in(k) + (next * C::ROWS + lr) * N, unsigned(N * sizeof(V)));
+                for (int k = 0; k < NIN; ++k) {
+                    // (a caller's array may be aligned for its points only)
+                    const V *p = op.in(k) + (next * C::ROWS + lr) * N;
+                    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) bulk_prefetch_l2(p, unsigned(N * sizeof(V)));
+                }
             const auto hook = [&]() {
                 fft_sync<C::BLOCK>();  // the row's last shared-memory reads are done
                 issue(next, 0);
@@ -514,13 +517,14 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, VAR>::THREADS, ColCfgOf<Rl
         cp_async_commit();
     };
 
+    constexpr bool EARLY = EarlyNext<Op>::value && C::NBUF == 1;
     int64_t tile = blockIdx.x;
     fill_stage_tw<N, C::P>(tw);
     op_prologue<N>(op);
     grid_wait();
     grid_trigger(tiles);
     if (op_idle(op)) return;
-    if (C::NBUF == 2) issue(tile, 0);
+    if (C::NBUF == 2 || EARLY) issue(tile, 0);
     __syncthreads();
     for (int it = 0; tile < tiles; ++it, tile += gridDim.x) {
         int b = 0;
@@ -528,6 +532,8 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, VAR>::THREADS, ColCfgOf<Rl
             b = it & 1;
             issue(tile + gridDim.x, b ^ 1);
             cp_async_wait<1>();
+        } else if constexpr (EARLY) {
+            cp_async_wait<0>();  // issued during the previous tile (or above)
         } else {
             issue(tile, 0);
             cp_async_wait<0>();
@@ -541,8 +547,16 @@ __global__ void __launch_bounds__(ColCfgOf<Rl, N, Op, VAR>::THREADS, ColCfgOf<Rl
             sm[k] = line(b, k);
             read_line<C::P, C::T>(v[k], sm[k], t);
         }
-        op.template col<N, C::P, C::BLOCK>(v, field, x, t, sm, tw);
-        fft_sync<C::BLOCK>();
+        if constexpr (EARLY) {
+            const int64_t next = tile + gridDim.x;
+            op.template col<N, C::P, C::BLOCK>(v, field, x, t, sm, tw, [&]() {
+                fft_sync<C::BLOCK>();  // the tile's last shared-memory reads are done
+                issue(next, 0);
+            });
+        } else {
+            op.template col<N, C::P, C::BLOCK>(v, field, x, t, sm, tw);
+            fft_sync<C::BLOCK>();
+        }
     }
     cp_async_wait<0>();
 }
@@ -1093,24 +1107,28 @@ __device__ __forceinline__ void store_line(const V (&v)[P], V *__restrict__ p, i
 }
 
 // ----------------------------------------------------------------------------
-// Plain transforms (the 2D FFT of every step, Section 4)
+// Plain transforms (the 2D FFT of every step, Section 4), in place or from
+// src into dst.  The next tile's copies are issued from the start of the last
+// stage (EARLY_NEXT).
 
 template <class Rl, int DIR> struct RowFft {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
-    V2<Rl> *data;
+    static constexpr bool EARLY_NEXT = true;
+    const V2<Rl> *src;
+    V2<Rl> *dst;
     Rl scale;  // applied after the transform when != 1
-    __device__ const V2<Rl> *in(int) const { return data; }
-    template <int N, int P, int BLOCK, class Sm>
+    __device__ const V2<Rl> *in(int) const { return src; }
+    template <int N, int P, int BLOCK, class Sm, class H = NoHook>
     __device__ __forceinline__ void row(V2<Rl> (&v)[1][P], int64_t r, bool ok, int t, const Sm (&sm)[1],
-                                        const TW<Rl> *tw) const
+                                        const TW<Rl> *tw, const H &hook = H{}) const
     {
-        block_fft<N, P, DIR, BLOCK>(v[0], sm[0], t, tw);
+        block_fft<N, P, DIR, BLOCK>(v[0], sm[0], t, tw, hook);
         if (scale != Rl(1))
 #pragma unroll
             for (int m = 0; m < P; ++m) v[0][m] = cscale(v[0][m], scale);
-        store_line<P, N / P>(v[0], data + r * N, 1, t, ok);
+        store_line<P, N / P>(v[0], dst + r * N, 1, t, ok);
     }
 };
 
@@ -1118,19 +1136,21 @@ template <class Rl, int DIR> struct ColFft {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
-    V2<Rl> *data;
+    static constexpr bool EARLY_NEXT = true;
+    const V2<Rl> *src;
+    V2<Rl> *dst;
     int64_t nx;
     Rl scale;
-    __device__ const V2<Rl> *in(int) const { return data; }
-    template <int N, int P, int BLOCK, class Sm>
-    __device__ __forceinline__ void col(V2<Rl> (&v)[1][P], int64_t field, int x, int t,
-                                        const Sm (&sm)[1], const TW<Rl> *tw) const
+    __device__ const V2<Rl> *in(int) const { return src; }
+    template <int N, int P, int BLOCK, class Sm, class H = NoHook>
+    __device__ __forceinline__ void col(V2<Rl> (&v)[1][P], int64_t field, int x, int t, const Sm (&sm)[1],
+                                        const TW<Rl> *tw, const H &hook = H{}) const
     {
-        block_fft<N, P, DIR, BLOCK>(v[0], sm[0], t, tw);
+        block_fft<N, P, DIR, BLOCK>(v[0], sm[0], t, tw, hook);
         if (scale != Rl(1))
 #pragma unroll
             for (int m = 0; m < P; ++m) v[0][m] = cscale(v[0][m], scale);
-        store_line<P, N / P>(v[0], data + field * N * nx + x, nx, t, true);
+        store_line<P, N / P>(v[0], dst + field * N * nx + x, nx, t, true);
     }
 };
 
