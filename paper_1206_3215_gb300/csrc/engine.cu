@@ -142,6 +142,7 @@ int pss_grid::init()
     if (p.eq == PSS_EQ_NS && p.rfft) {
         ns_half = true;
         nsx = nx / 2 + 8;  // a multiple of every column-tile width
+        if ((rc = upload_twiddles(this, nx / 2, &twm))) return rc;
     }
     if (p.eq == PSS_EQ_SG && p.rfft) {
         half = true;
@@ -464,37 +465,6 @@ template <class Rl> int nls_conserved(pss_grid *g, double *out)
 
 namespace {
 
-// forward (-1) or inverse (+1, with 1/(nx ny)) 2D transform of buffer b
-template <class Rl> cudaError_t fft2(pss_grid *g, V2<Rl> *b, int dir)
-{
-    cudaError_t e = fft_rows<Rl>(b, b, g->nx, g->ny, g->batch, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
-    if (e != cudaSuccess) return e;
-    const Rl sc = dir > 0 ? Rl(1.0 / (double(g->nx) * double(g->ny))) : Rl(1);
-    return fft_cols<Rl>(b, b, g->nx, g->ny, g->batch, dir, sc, Tw<Rl>(g->twy), g->stream);
-}
-
-// real caller array (host or device) -> complex buffer dst (imaginary part 0),
-// through the raw scratch buffer `tmp`
-template <class Rl> int load_real(pss_grid *g, const void *src, int where, int tmp, int dst)
-{
-    const size_t bytes = size_t(g->ntot) * sizeof(Rl);
-    int rc = g->cuda(cudaMemcpyAsync(g->buf[tmp], src, bytes, kind_in(where), g->stream), "state copy");
-    if (rc) return rc;
-    return g->cuda(real_to_complex<Rl>(static_cast<const Rl *>(g->buf[tmp]), B<Rl>(g, dst), g->ntot, g->stream),
-                   "real to complex");
-}
-
-// Re(a - c b) of complex buffers into the caller array (through `tmp` for HOST)
-template <class Rl>
-int store_real(pss_grid *g, const V2<Rl> *a, const V2<Rl> *b, Rl c, void *dst, int where, int tmp)
-{
-    Rl *d = where == PSS_DEVICE ? static_cast<Rl *>(dst) : static_cast<Rl *>(g->buf[tmp]);
-    int rc = g->cuda(complex_to_real<Rl>(a, b, c, d, g->ntot, g->stream), "complex to real");
-    if (rc || where == PSS_DEVICE) return rc;
-    return g->cuda(cudaMemcpyAsync(dst, d, size_t(g->ntot) * sizeof(Rl), cudaMemcpyDeviceToHost, g->stream),
-                   "state copy");
-}
-
 template <class Rl> const Rl *Rt(const void *p) { return static_cast<const Rl *>(p); }
 
 int finish_sums(pss_grid *g)
@@ -539,7 +509,7 @@ template <class Rl> int sg_make_h(pss_grid *g, const SgState<Rl> &st)
 
 // A caller's real array as the row kernels read it (pairs): the array itself
 // where it is device memory aligned for that, else a copy in `tmp`.
-template <class Rl> int sg_real_in(pss_grid *g, const void *src, int where, Rl *tmp, int64_t n, const Rl **out)
+template <class Rl> int real_in(pss_grid *g, const void *src, int where, Rl *tmp, int64_t n, const Rl **out)
 {
     if (where == PSS_DEVICE && kernel_access(src, 2 * sizeof(Rl))) {
         *out = static_cast<const Rl *>(src);
@@ -562,8 +532,8 @@ template <class Rl> int sg_set_fields(pss_grid *g, int64_t f, int64_t nb, const 
     const SgState<Rl> st = sg_state<Rl>(g, f, nb);
     const Rl *u = nullptr, *v = nullptr;
     int rc;
-    if ((rc = sg_real_in<Rl>(g, u0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), nb * g->npts, &u)) ||
-        (v0 && (rc = sg_real_in<Rl>(g, v0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), nb * g->npts, &v))))
+    if ((rc = real_in<Rl>(g, u0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), nb * g->npts, &u)) ||
+        (v0 && (rc = real_in<Rl>(g, v0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), nb * g->npts, &v))))
         return rc;
     cudaError_t e;
     if (g->half) {
@@ -588,8 +558,8 @@ template <class Rl> int sg_set_levels(pss_grid *g, const void *un, const void *u
     const SgState<Rl> st = sg_state<Rl>(g, 0, g->batch);
     const Rl *a = nullptr, *b = nullptr;
     int rc;
-    if ((rc = sg_real_in<Rl>(g, un, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), g->ntot, &a)) ||
-        (rc = sg_real_in<Rl>(g, unm1, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), g->ntot, &b)) ||
+    if ((rc = real_in<Rl>(g, un, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), g->ntot, &a)) ||
+        (rc = real_in<Rl>(g, unm1, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), g->ntot, &b)) ||
         (rc = g->cuda(sg_split<Rl>(g, st, a, st.u), "forward rows")) ||
         (rc = g->cuda(sg_split<Rl>(g, st, b, st.d), "forward rows")) ||
         (rc = g->cuda(fft_cols<Rl>(st.u, st.u, st.w, g->ny, st.nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
@@ -765,15 +735,25 @@ template <class Rl> int ns_to_half(pss_grid *g, V2<Rl> *src, V2<Rl> *dst, int64_
     return g->cuda(pack_half<Rl>(src, dst, g->nx, g->ny, g->nsx, batch, g->stream), "pack");
 }
 
-template <class Rl> int ns_set(pss_grid *g, const void *w0, int where)
+// vorticity of fields f .. f + nb - 1: masked spectra into buffer 0, their
+// records cleared, derivatives formed
+template <class Rl> int ns_set(pss_grid *g, int64_t f, int64_t nb, const void *w0, int where)
 {
+    const int64_t width = g->ns_half ? g->nsx : g->nx;
+    V2<Rl> *w = B<Rl>(g, 0) + ns_off(g, f);
+    const Rl *src = nullptr;
     int rc;
-    if ((rc = load_real<Rl>(g, w0, where, 6, 0)) || (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 0), -1), "forward")) ||
-        (rc = g->cuda(apply_mask<Rl>(B<Rl>(g, 0), Rt<Rl>(g->keepx), Rt<Rl>(g->keepy), g->nx, g->ny, g->batch, g->stream),
-                      "mask")) ||
-        (rc = g->cuda(cudaMemsetAsync(g->ns_field, 0, size_t(g->batch) * ns_field_bytes(), g->stream), "memset")) ||
-        (g->ns_half && (rc = ns_to_half<Rl>(g, B<Rl>(g, 0), B<Rl>(g, 0), g->batch))) || (rc = ns_prep<Rl>(g)))
+    if ((rc = real_in<Rl>(g, w0, where, reinterpret_cast<Rl *>(Bf<Rl>(g, 6, f)), nb * g->npts, &src)) ||
+        (rc = g->cuda(rows_from_real<Rl>(src, w, g->nx, g->ns_half ? g->nsx : 0, g->ny, nb, Tw<Rl>(g->twx), g->stream),
+                      "forward rows")) ||
+        (rc = g->cuda(fft_cols<Rl>(w, w, width, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
+        (rc = g->cuda(apply_mask<Rl>(w, Rt<Rl>(g->keepx), Rt<Rl>(g->keepy), width, g->ny, nb, g->stream), "mask")) ||
+        (rc = g->cuda(cudaMemsetAsync(static_cast<char *>(g->ns_field) + f * ns_field_bytes(), 0,
+                                      size_t(nb) * ns_field_bytes(), g->stream), "memset")))
         return rc;
+    for (int64_t i = f; i < f + nb && nb < g->batch; ++i)
+        if ((rc = ns_prep_one<Rl>(g, i))) return rc;
+    if (nb == g->batch && (rc = ns_prep<Rl>(g))) return rc;
     return where == PSS_HOST ? g->cuda(cudaStreamSynchronize(g->stream), "sync") : PSS_OK;
 }
 
@@ -892,11 +872,27 @@ template <class Rl> int ns_current(pss_grid *g)
     return g->cuda(unpack_half<Rl>(B<Rl>(g, 3), B<Rl>(g, 6), g->nx, g->ny, g->nsx, g->batch, g->stream), "unpack");
 }
 
-template <class Rl> int ns_get(pss_grid *g, void *a, int where)
+// vorticity of fields f .. f + nb - 1 into a: column pass into buf[6], row pass
+// into the real array
+template <class Rl> int ns_get(pss_grid *g, int64_t f, int64_t nb, void *a, int where)
 {
+    V2<Rl> *w[3];
+    for (int i = 0; i < 3; ++i) w[i] = B<Rl>(g, i) + ns_off(g, f);
+    const bool direct = where == PSS_DEVICE && kernel_access(a, 2 * sizeof(Rl));
+    // (J_hat^n in buf[3] is rebuilt at the start of every step)
+    Rl *dst = direct ? static_cast<Rl *>(a) : reinterpret_cast<Rl *>(g->buf[3]) + f * g->npts;
+    V2<Rl> *t = Bf<Rl>(g, 6, f);
+    const Rl s = Rl(1.0 / (double(g->nx) * double(g->ny)));
     int rc;
-    if ((rc = ns_current<Rl>(g)) || (rc = g->cuda(fft2<Rl>(g, B<Rl>(g, 6), +1), "inverse")) ||
-        (rc = store_real<Rl>(g, B<Rl>(g, 6), nullptr, Rl(0), a, where, 3)))
+    if ((rc = g->cuda(ns_level_cols<Rl>(static_cast<char *>(g->ns_field) + f * ns_field_bytes(), w, t, s,
+                                        g->ns_half ? g->nsx : g->nx, g->ny, nb, Tw<Rl>(g->twy), g->stream),
+                      "inverse columns")) ||
+        (rc = g->cuda(g->ns_half ? sg_half_join<Rl>(t, dst, g->nx, g->nsx, g->ny, nb, Tw<Rl>(g->twm), Tw<Rl>(g->twx),
+                                                    g->stream)
+                                 : rows_to_real<Rl>(t, dst, g->nx, g->ny, nb, Tw<Rl>(g->twx), g->stream),
+                      "inverse rows")) ||
+        (!direct && (rc = g->cuda(cudaMemcpyAsync(a, dst, size_t(nb) * g->npts * sizeof(Rl), kind_out(where),
+                                                  g->stream), "state copy"))))
         return rc;
     return g->sync();
 }
@@ -934,80 +930,18 @@ template <class Rl> int ns_conserved(pss_grid *g, double *out)
 
 namespace {
 
-template <class Rl> cudaError_t fft2_one(pss_grid *g, V2<Rl> *b, int dir)
-{
-    cudaError_t e = fft_rows<Rl>(b, b, g->nx, g->ny, 1, dir, Rl(1), Tw<Rl>(g->twx), g->stream);
-    if (e != cudaSuccess) return e;
-    const Rl sc = dir > 0 ? Rl(1.0 / (double(g->nx) * double(g->ny))) : Rl(1);
-    return fft_cols<Rl>(b, b, g->nx, g->ny, 1, dir, sc, Tw<Rl>(g->twy), g->stream);
-}
-
-// real field (host or device) -> complex slot dst_buf[f], through raw scratch slot tmp_buf[f]
-template <class Rl>
-int load_real_one(pss_grid *g, int64_t f, const void *src, int where, int tmp, int dst)
-{
-    Rl *t = reinterpret_cast<Rl *>(Bf<Rl>(g, tmp, f));
-    int rc = g->cuda(cudaMemcpyAsync(t, src, size_t(g->npts) * sizeof(Rl), kind_in(where), g->stream), "copy");
-    if (rc) return rc;
-    return g->cuda(real_to_complex<Rl>(t, Bf<Rl>(g, dst, f), g->npts, g->stream), "real to complex");
-}
-
-template <class Rl> int store_real_one(pss_grid *g, int64_t f, const V2<Rl> *a, void *dst, int where, int tmp)
-{
-    Rl *d = where == PSS_DEVICE ? static_cast<Rl *>(dst) : reinterpret_cast<Rl *>(Bf<Rl>(g, tmp, f));
-    int rc = g->cuda(complex_to_real<Rl>(a, nullptr, Rl(0), d, g->npts, g->stream), "complex to real");
-    if (rc || where == PSS_DEVICE) return rc;
-    return g->cuda(cudaMemcpyAsync(dst, d, size_t(g->npts) * sizeof(Rl), cudaMemcpyDeviceToHost, g->stream), "copy");
-}
-
 template <class Rl> int field_set(pss_grid *g, int64_t f, const void *a, const void *b, int where)
 {
-    int rc = PSS_OK;
-    if (g->p.eq == PSS_EQ_NLS) {
-        return nls_set<Rl>(g, f, 1, a, where);
-    } else if (g->p.eq == PSS_EQ_SG) {
-        return sg_set_fields<Rl>(g, f, 1, a, b, where);
-    } else {
-        // full spectrum of the field in buf[6] (half spectra) or buf[0], then
-        // (half spectra) into the field's slot of the half-width buffer 0
-        const int dst = g->ns_half ? 6 : 0;
-        if ((rc = load_real_one<Rl>(g, f, a, where, g->ns_half ? 3 : 6, dst)) ||
-            (rc = g->cuda(fft2_one<Rl>(g, Bf<Rl>(g, dst, f), -1), "forward")) ||
-            (rc = g->cuda(apply_mask<Rl>(Bf<Rl>(g, dst, f), Rt<Rl>(g->keepx), Rt<Rl>(g->keepy), g->nx, g->ny, 1,
-                                         g->stream), "mask")) ||
-            (g->ns_half && (rc = ns_to_half<Rl>(g, Bf<Rl>(g, 6, f), B<Rl>(g, 0) + ns_off(g, f), 1))) ||
-            (rc = g->cuda(cudaMemsetAsync(static_cast<char *>(g->ns_field) + f * ns_field_bytes(), 0, ns_field_bytes(),
-                                          g->stream), "record")) ||
-            (rc = ns_prep_one<Rl>(g, f)))
-            return rc;
-    }
-    return where == PSS_HOST ? g->cuda(cudaStreamSynchronize(g->stream), "sync") : PSS_OK;
+    if (g->p.eq == PSS_EQ_NLS) return nls_set<Rl>(g, f, 1, a, where);
+    if (g->p.eq == PSS_EQ_SG) return sg_set_fields<Rl>(g, f, 1, a, b, where);
+    return ns_set<Rl>(g, f, 1, a, where);
 }
 
 template <class Rl> int field_get(pss_grid *g, int64_t f, void *a, void *b, int where)
 {
-    int rc;
-    if (g->p.eq == PSS_EQ_NLS) {
-        return nls_get<Rl>(g, f, 1, a, where);
-    } else if (g->p.eq == PSS_EQ_SG) {
-        return sg_get_fields<Rl>(g, f, 1, a, b, where);
-    } else {
-        V2<Rl> *w[3];
-        for (int i = 0; i < 3; ++i) w[i] = B<Rl>(g, i) + ns_off(g, f);  // field f's slot of each vorticity buffer
-        const void *rec = static_cast<char *>(g->ns_field) + f * ns_field_bytes();
-        if (g->ns_half) {
-            V2<Rl> *h = B<Rl>(g, 3) + ns_off(g, f);
-            if ((rc = g->cuda(ns_gather<Rl>(rec, w, h, g->ny * g->nsx, 1, g->stream), "gather")) ||
-                (rc = g->cuda(unpack_half<Rl>(h, Bf<Rl>(g, 6, f), g->nx, g->ny, g->nsx, 1, g->stream), "unpack")))
-                return rc;
-        } else if ((rc = g->cuda(ns_gather<Rl>(rec, w, Bf<Rl>(g, 6, f), g->npts, 1, g->stream), "gather"))) {
-            return rc;
-        }
-        if ((rc = g->cuda(fft2_one<Rl>(g, Bf<Rl>(g, 6, f), +1), "inverse")) ||
-            (rc = store_real_one<Rl>(g, f, Bf<Rl>(g, 6, f), a, where, 3)))
-            return rc;
-    }
-    return g->sync();
+    if (g->p.eq == PSS_EQ_NLS) return nls_get<Rl>(g, f, 1, a, where);
+    if (g->p.eq == PSS_EQ_SG) return sg_get_fields<Rl>(g, f, 1, a, b, where);
+    return ns_get<Rl>(g, f, 1, a, where);
 }
 
 }  // namespace
@@ -1024,7 +958,7 @@ int pss_grid::set_state(const void *a, const void *b, int where)
     int rc;
 #define NLS(R) nls_set<R>(this, 0, batch, a, where)
 #define SG(R) sg_set_fields<R>(this, 0, batch, a, b, where)
-#define NS(R) ns_set<R>(this, a, where)
+#define NS(R) ns_set<R>(this, 0, batch, a, where)
     rc = p.eq == PSS_EQ_NLS ? PSS_BY_PRECISION(NLS) : p.eq == PSS_EQ_SG ? PSS_BY_PRECISION(SG) : PSS_BY_PRECISION(NS);
 #undef NLS
 #undef SG
@@ -1150,7 +1084,7 @@ int pss_grid::get_state(void *a, void *b, int where)
     if (rc) return rc;
 #define NLS(R) nls_get<R>(this, 0, batch, a, where)
 #define SG(R) sg_get_fields<R>(this, 0, batch, a, b, where)
-#define NS(R) ns_get<R>(this, a, where)
+#define NS(R) ns_get<R>(this, 0, batch, a, where)
     return p.eq == PSS_EQ_NLS ? PSS_BY_PRECISION(NLS) : p.eq == PSS_EQ_SG ? PSS_BY_PRECISION(SG) : PSS_BY_PRECISION(NS);
 #undef NLS
 #undef SG

@@ -123,6 +123,11 @@ template <class Rl>
 cudaError_t ns_prep_pass(V2<Rl> *const w[3], const void *fs, V2<Rl> *c1, V2<Rl> *c2, const Rl *kxo, const Rl *kyo,
                          const Rl *kx2, const Rl *ky2, int64_t nx, int64_t ny, int64_t batch,
                          const int *ctl, const TW<Rl> *twy, cudaStream_t s, int64_t sx = 0);
+// current vorticity of every field, column inverse transform times scale, into
+// out (rows of nx, full or half spectra)
+template <class Rl>
+cudaError_t ns_level_cols(const void *fs, V2<Rl> *const w[3], V2<Rl> *out, Rl scale, int64_t nx, int64_t ny,
+                          int64_t batch, const TW<Rl> *twy, cudaStream_t s);
 // Loop control (ctl: ints of the grid's flag block, k_ns.cuh): n steps of every
 // field; the decision after an update (`last`: the last one of a loop body).
 cudaError_t ns_begin(void *fs, int64_t batch, int *ctl, int n, cudaStream_t s);
@@ -131,9 +136,6 @@ cudaError_t ns_decide(void *fs, const double *partials, int64_t groups, int64_t 
                       cudaGraphConditionalHandle h, cudaStream_t s);
 
 // ---- elementwise helpers (k_util.cu) ----------------------------------------
-template <class Rl> cudaError_t real_to_complex(const Rl *src, V2<Rl> *dst, int64_t n, cudaStream_t s);
-template <class Rl>
-cudaError_t complex_to_real(const V2<Rl> *a, const V2<Rl> *b, Rl c, Rl *dst, int64_t n, cudaStream_t s);
 template <class Rl>
 cudaError_t ns_gather(const void *fs, V2<Rl> *const w[3], V2<Rl> *dst, int64_t per_field, int64_t batch,
                       cudaStream_t s);

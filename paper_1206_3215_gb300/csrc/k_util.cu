@@ -3,21 +3,6 @@
 
 namespace pss {
 
-// dst[i] = (src[i], 0)
-template <class Rl> __global__ void k_real_to_complex(const Rl *src, V2<Rl> *dst, int64_t n)
-{
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-        dst[i] = V2<Rl>{src[i], Rl(0)};
-}
-
-// dst[i] = Re(a[i]) - c * Re(b[i])   (b may be null)
-template <class Rl>
-__global__ void k_complex_to_real(const V2<Rl> *a, const V2<Rl> *b, Rl c, Rl *dst, int64_t n)
-{
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-        dst[i] = b ? a[i].x - c * b[i].x : a[i].x;
-}
-
 // copy every field's current vorticity (buffer fs[f].idx) into dst
 struct NsFieldView {
     int idx, active, nonconv, k;
@@ -53,17 +38,6 @@ __global__ void k_mask(V2<Rl> *a, const Rl *keepx, const Rl *keepy, int64_t nx, 
 
 static unsigned blocks_for(int64_t n) { return unsigned(n / 256 + 1 < 4096 ? n / 256 + 1 : 4096); }
 
-template <class Rl> cudaError_t real_to_complex(const Rl *src, V2<Rl> *dst, int64_t n, cudaStream_t s)
-{
-    k_real_to_complex<Rl><<<blocks_for(n), 256, 0, s>>>(src, dst, n);
-    return cudaGetLastError();
-}
-template <class Rl>
-cudaError_t complex_to_real(const V2<Rl> *a, const V2<Rl> *b, Rl c, Rl *dst, int64_t n, cudaStream_t s)
-{
-    k_complex_to_real<Rl><<<blocks_for(n), 256, 0, s>>>(a, b, c, dst, n);
-    return cudaGetLastError();
-}
 template <class Rl>
 cudaError_t ns_gather(const void *fs, V2<Rl> *const w[3], V2<Rl> *dst, int64_t per_field, int64_t batch,
                       cudaStream_t s)
@@ -90,8 +64,6 @@ cudaError_t apply_mask(V2<Rl> *a, const Rl *keepx, const Rl *keepy, int64_t nx, 
 #define PSS_INST(Rl)                                                                                      \
     template cudaError_t cplx_axpy<Rl>(const V2<Rl> *, const V2<Rl> *, Rl, V2<Rl> *, int64_t, cudaStream_t); \
     template cudaError_t apply_mask<Rl>(V2<Rl> *, const Rl *, const Rl *, int64_t, int64_t, int64_t, cudaStream_t); \
-    template cudaError_t real_to_complex<Rl>(const Rl *, V2<Rl> *, int64_t, cudaStream_t);                \
-    template cudaError_t complex_to_real<Rl>(const V2<Rl> *, const V2<Rl> *, Rl, Rl *, int64_t, cudaStream_t); \
     template cudaError_t ns_gather<Rl>(const void *, V2<Rl> *const[3], V2<Rl> *, int64_t, int64_t, cudaStream_t);
 PSS_INST(float)
 PSS_INST(double)
