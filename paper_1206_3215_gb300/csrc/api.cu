@@ -79,10 +79,23 @@ int pss_grid::alloc(void **p, size_t bytes)
 
 int pss_grid::upload(void **p, const void *host, size_t bytes)
 {
-    int rc = alloc(p, bytes);
+    const size_t at = (tables.size() + 255) / 256 * 256;
+    tables.resize(at + bytes);
+    memcpy(tables.data() + at, host, bytes);
+    table_ptrs.emplace_back(p, at);
+    return PSS_OK;
+}
+
+int pss_grid::upload_tables()
+{
+    void *base = nullptr;
+    int rc = alloc(&base, tables.size());
     if (rc) return rc;
-    cudaError_t e = cudaMemcpy(*p, host, bytes, cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpy(base, tables.data(), tables.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return fail(PSS_E_CUDA, "table upload: %s", cudaGetErrorString(e));
+    for (auto &t : table_ptrs) *t.first = static_cast<char *>(base) + t.second;
+    tables = {};
+    table_ptrs = {};
     return PSS_OK;
 }
 

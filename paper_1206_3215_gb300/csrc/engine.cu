@@ -189,6 +189,7 @@ int pss_grid::init()
             if ((rc = upload_cplx_table(this, ny, fy, &by[h]))) return rc;
         }
     }
+    if ((rc = upload_tables())) return rc;
     // reductions
     const size_t parts = size_t(batch) * 3 * std::max<int64_t>(RED_BLOCKS, nx);
     if ((rc = alloc((void **)&partials, parts * 8))) return rc;

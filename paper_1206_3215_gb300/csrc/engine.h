@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/pss.h"
@@ -126,7 +127,13 @@ struct pss_grid {
 
     int fail(int code, const char *fmt, ...);
     int alloc(void **p, size_t bytes);
+    // tables: upload() collects them, upload_tables() puts all of them on the
+    // device in one allocation and one copy and sets their pointers (a grid has
+    // 8 to 12; one by one they were a third of its creation)
     int upload(void **p, const void *host, size_t bytes);
+    int upload_tables();
+    std::vector<char> tables;
+    std::vector<std::pair<void **, size_t>> table_ptrs;
     int cuda(cudaError_t e, const char *what);
 
     int init();
