@@ -30,8 +30,9 @@ namespace pss {
 template <class Rl, int M, bool SMALL> struct R2cCfg {
     static constexpr int P = Shape<Rl>::rowP(M, SMALL);
     static constexpr int T = M / P;
-    // short rows: smaller CTAs, so that few rows still spread over the SMs
-    static constexpr int RT = M <= 256 ? 128 : 256;
+    // short rows: smaller CTAs, so that few rows still spread over the SMs; FP64
+    // as in RowCfg (SG 1024^2 x 2 451 -> 413 us per step, 256^2 x 2 44 -> 40)
+    static constexpr int RT = sizeof(Rl) == 8 ? (M <= 256 ? 32 : 64) : M <= 256 ? 128 : 256;
     static constexpr int ROWS = T >= RT ? 1 : RT / T;
     static constexpr int THREADS = ROWS * T;
     // barrier of one row's threads (fft_sync): a warp (T <= 32: the rows are

@@ -152,9 +152,9 @@ template <class Rl> struct Shape {
     // where 32-byte segments fit in 256 threads, the wider tile was slower)
     __host__ __device__ static constexpr int cols_capped(int n, int p, int nbuf, int cap)
     {
-        // FP64 up to 256: two columns (32-byte row segments) for more tiles, at
-        // 16 a whole warp
-        int w = sizeof(Rl) == 4 ? PSS_COL_WMAX : n > 256 ? 4 : n > 16 ? 2 : 8;
+        // FP64 up to 2048: two columns (32-byte row segments), twice the tiles of
+        // four to share out among the SMs; at 16 a whole warp
+        int w = sizeof(Rl) == 4 ? PSS_COL_WMAX : n > 2048 ? 4 : n > 16 ? 2 : 8;
         while (w > 1 && ((long)nbuf * w * (n + n / 16) * ESZ > 200 * 1024L || w * (n / p) > cap)) w /= 2;
         return w;
     }
@@ -221,9 +221,13 @@ template <class Rl, int N, int NIN, bool LEAN = false, int PMAX = 32, int VAR = 
     using VS = VarShape<Rl, VAR>;
     static constexpr int P = imin(imin(Shape<Rl>::rowP(N, VAR == 2), PMAX), VS::PCAP);
     static constexpr int T = N / P;
-    // ~256 threads per CTA; small rows (N <= 256) take ~64 (FP64: one warp) so
-    // that a batch of small grids still spreads over many SMs
-    static constexpr int RT = N <= 256 ? (sizeof(Rl) == 4 ? PSS_ROW_THREADS_SMALL : 32) : PSS_ROW_THREADS;
+    // ~256 threads per CTA; small rows (N <= 256) take ~64 so that a batch of
+    // small grids still spreads over many SMs.  FP64: one row (or a warp) per
+    // CTA: every SM is bound by its FP64 lanes, so what counts is that all get
+    // the same number of rows (NLS 1024^2 x 3: 768 tiles of four rows on 152
+    // SMs were 6 rounds for 5.05; with the columns below 1106 -> 982 us per step)
+    static constexpr int RT =
+        sizeof(Rl) == 4 ? (N <= 256 ? PSS_ROW_THREADS_SMALL : PSS_ROW_THREADS) : N <= 256 ? 32 : 64;
     static constexpr int ROWS = T >= RT ? 1 : RT / T;
     static constexpr int PADLOG = pad_log(P);
     static constexpr int LINE = N + (N >> PADLOG);
