@@ -27,8 +27,8 @@ struct pss_grid {
     int nbuf = 0;
 
     // sine-Gordon on half spectra (p.rfft): the stepping state lives in
-    // hbuf = {uhat, d, H}, [batch][ny][sx] with kx = 0 .. nx/2; the full
-    // buffers buf[0], buf[1] are rebuilt from it when a call reads the state
+    // hbuf = {uhat, d, H}, [batch][ny][sx] with kx = 0 .. nx/2, set and read
+    // there; the full buffers buf[0], buf[1] are rebuilt from it for checkpoints
     bool half = false;
     int64_t sx = 0;
     void *hbuf[3] = {};

@@ -111,7 +111,7 @@ __device__ __forceinline__ double one_minus_cos(double x)
 // spectra where w < nx (columns 0 and nx/2 once, those between them twice).
 // Bound by the FP64 lanes (two per SM): the division by dt is taken out of
 // the sum and 1 - cos is a polynomial where it may be; with real fields and
-// half spectra 2048^2 x 8 takes 0.9 ms (2.85 ms with complex fields, full
+// half spectra 2048^2 x 8 takes 1.4 ms (2.85 ms with complex fields, full
 // spectra, a division and a sine per point).
 template <class Rl>
 __global__ void __launch_bounds__(RED_THREADS)

@@ -15,8 +15,9 @@
 // 1e-8.
 //
 // 2048^2 x 8 on half spectra, against transforms of full complex arrays with
-// separate copies, conversions and FP64 elementwise kernels: set-up 4.2 -> 0.6 ms,
-// read-back of both levels 1.6 -> 0.5 ms, Hamiltonian 3.8 -> 1.8 ms.
+// separate copies, conversions and FP64 elementwise kernels (sums of kernel
+// times): set-up 3.4 -> 0.5 ms, read-back of both levels 1.2 -> 0.3 ms,
+// Hamiltonian 3.6 -> 1.9 ms.
 #include <algorithm>
 
 #include "k_sg_r2c.cuh"

@@ -624,7 +624,7 @@ template <class Rl, int N, class Op> struct TmaHalfStore {
 // op.later(0) and op.later(1), after its first transform: the pass asks for
 // their tiles to be brought into L2 when it asks for the tile itself, by one
 // tensor prefetch each (maps map_half and map_later; per-point prefetches of
-// every thread cost 64 instructions each: SG 2048^2 x 8 column pass 219 -> 210 us).
+// every thread cost 64 instructions each: SG 2048^2 x 8 column pass 224 -> 215 us).
 template <class Op, class = void> struct ColPrefetch : std::false_type {};
 template <class Op>
 struct ColPrefetch<Op, std::void_t<decltype(Op::COL_PREFETCH)>> : std::integral_constant<bool, Op::COL_PREFETCH> {};

@@ -33,7 +33,7 @@ __device__ __forceinline__ float sg_sin_poly(float r)
 constexpr float sg_sin_small = 0.785f;
 // whether every value of a thread is that small: its passes then run the sine
 // polynomial alone, 6 instead of 22 instructions per point (2048^2 x 8 half
-// spectra row pass 127 -> 117 us)
+// spectra row pass 135 -> 117 us)
 template <int P> __device__ __forceinline__ bool sg_all_small(const float2 (&v)[P], bool both)
 {
     float big = 0.0f;
