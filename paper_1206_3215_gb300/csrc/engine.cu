@@ -667,8 +667,8 @@ template <class Rl> int sg_conserved(pss_grid *g, double *out)
             return rc;
         }
     }
-    if ((rc = g->cuda(sg_sums<Rl>(X, Y, st.u, st.d, g->nx, g->ny, st.w, g->batch, g->kx2d, g->ky2d, g->p.dt,
-                                  g->partials, g->sums, g->stream), "sg sums")) ||
+    if ((rc = g->cuda(sg_sums<Rl>(X, Y, st.u, st.d, g->nx, g->ny, st.w, g->half, g->batch, g->kx2d, g->ky2d,
+                                  g->p.dt, g->partials, g->sums, g->stream), "sg sums")) ||
         (rc = finish_sums(g)))
         return rc;
     const double dA = g->dA(), inv_n = 1.0 / (double(g->nx) * double(g->ny));

@@ -158,12 +158,12 @@ cudaError_t nls_sums(const V2<Rl> *psi, const V2<Rl> *psi_hat, int64_t nx, int64
 void set_global_error(const char *msg);
 
 // SG: per field {sum (Y/dt)^2/2, sum 1 - cos(X - Y/2), sum |k|^2 |U - D/2|^2};
-// X, Y real fields, U, D spectra with rows of w columns: w = nx, or (half
-// spectra) w > nx/2, columns 0 .. nx/2 standing for both halves
+// X, Y real fields, U, D spectra with rows of w columns: all nx of them, or
+// (`half`) columns 0 .. nx/2 standing for both halves and padding beyond
 template <class Rl>
 cudaError_t sg_sums(const Rl *X, const Rl *Y, const V2<Rl> *U, const V2<Rl> *D, int64_t nx, int64_t ny, int64_t w,
-                    int64_t batch, const double *kx2, const double *ky2, double dt, double *partials, double *out,
-                    cudaStream_t s);
+                    bool half, int64_t batch, const double *kx2, const double *ky2, double dt, double *partials,
+                    double *out, cudaStream_t s);
 // NS: per field {Re w_hat(0,0), sum |w_hat|^2, sum_{k != 0} |w_hat|^2 / |k|^2}
 template <class Rl>
 cudaError_t ns_sums(const void *fs, V2<Rl> *const w[3], int64_t nx, int64_t ny, int64_t batch, const double *kx2,

@@ -107,8 +107,9 @@ __device__ __forceinline__ double one_minus_cos(double x)
 
 // SG at t_{n-1/2}: X = u^n, Y = u^n - u^{n-1} (real fields), U = uhat^n,
 // D = uhat^n - uhat^{n-1}.  Sums: (Y/dt)^2 / 2, 1 - cos(ubar) with
-// ubar = X - Y/2, and |k|^2 |U - D/2|^2 (the spectrum of ubar), over half
-// spectra where w < nx (columns 0 and nx/2 once, those between them twice).
+// ubar = X - Y/2, and |k|^2 |U - D/2|^2 (the spectrum of ubar), with `half` over
+// half spectra (columns 0 and nx/2 once, those between them twice; the row
+// length w does not tell the layout: half rows of nx = 16 are 16 long too).
 // Bound by the FP64 lanes (two per SM): the division by dt is taken out of
 // the sum and 1 - cos is a polynomial where it may be; with real fields and
 // half spectra 2048^2 x 8 takes 1.4 ms (2.85 ms with complex fields, full
@@ -116,8 +117,8 @@ __device__ __forceinline__ double one_minus_cos(double x)
 template <class Rl>
 __global__ void __launch_bounds__(RED_THREADS)
     k_sg_sums(const Rl *__restrict__ X, const Rl *__restrict__ Y, const V2<Rl> *__restrict__ U,
-              const V2<Rl> *__restrict__ D, int64_t nx, int64_t ny, int64_t w, const double *__restrict__ kx2,
-              const double *__restrict__ ky2, double half_dt2inv, double *partials)
+              const V2<Rl> *__restrict__ D, int64_t nx, int64_t ny, int64_t w, int half,
+              const double *__restrict__ kx2, const double *__restrict__ ky2, double half_dt2inv, double *partials)
 {
     __shared__ double sh[3 * RED_THREADS];
     const int64_t f = blockIdx.y, n = nx * ny, o = f * n, ns = w * ny, os = f * ns;
@@ -132,11 +133,11 @@ __global__ void __launch_bounds__(RED_THREADS)
 #pragma unroll 4
     for (unsigned i = blockIdx.x * RED_THREADS + threadIdx.x; i < unsigned(ns); i += RED_BLOCKS * RED_THREADS) {
         const unsigned y = i / uw, x = i - y * uw;
-        if (w < nx && x > mid) continue;  // padding of half spectra
+        if (half && x > mid) continue;  // padding of half spectra
         const V2<Rl> u = U[os + i], d = D[os + i];
         const double br = fma(-0.5, double(d.x), double(u.x)), bi = fma(-0.5, double(d.y), double(u.y));
         const double e = (kx2[x] + ky2[y]) * fma(br, br, bi * bi);
-        a[2] += w < nx && x != 0 && x != mid ? 2.0 * e : e;
+        a[2] += half && x != 0 && x != mid ? 2.0 * e : e;
     }
     a[0] *= half_dt2inv;
     block_sum<3>(a, sh);
@@ -180,11 +181,11 @@ __global__ void __launch_bounds__(RED_THREADS)
 
 template <class Rl>
 cudaError_t sg_sums(const Rl *X, const Rl *Y, const V2<Rl> *U, const V2<Rl> *D, int64_t nx, int64_t ny, int64_t w,
-                    int64_t batch, const double *kx2, const double *ky2, double dt, double *partials, double *out,
-                    cudaStream_t s)
+                    bool half, int64_t batch, const double *kx2, const double *ky2, double dt, double *partials,
+                    double *out, cudaStream_t s)
 {
-    k_sg_sums<Rl><<<dim3(RED_BLOCKS, unsigned(batch)), RED_THREADS, 0, s>>>(X, Y, U, D, nx, ny, w, kx2, ky2,
-                                                                           0.5 / (dt * dt), partials);
+    k_sg_sums<Rl><<<dim3(RED_BLOCKS, unsigned(batch)), RED_THREADS, 0, s>>>(X, Y, U, D, nx, ny, w, half ? 1 : 0, kx2,
+                                                                           ky2, 0.5 / (dt * dt), partials);
     k_fold<3><<<unsigned(batch), RED_THREADS, 0, s>>>(partials, out);
     return cudaGetLastError();
 }
@@ -200,11 +201,11 @@ cudaError_t ns_sums(const void *fs, V2<Rl> *const w[3], int64_t nx, int64_t ny, 
 }
 
 template cudaError_t sg_sums<float>(const float *, const float *, const float2 *, const float2 *, int64_t, int64_t,
-                                    int64_t, int64_t, const double *, const double *, double, double *, double *,
+                                    int64_t, bool, int64_t, const double *, const double *, double, double *, double *,
                                     cudaStream_t);
 template cudaError_t sg_sums<double>(const double *, const double *, const double2 *, const double2 *, int64_t,
-                                     int64_t, int64_t, int64_t, const double *, const double *, double, double *,
-                                     double *, cudaStream_t);
+                                     int64_t, int64_t, bool, int64_t, const double *, const double *, double, double *, double *,
+                                     cudaStream_t);
 template cudaError_t ns_sums<float>(const void *, float2 *const[3], int64_t, int64_t, int64_t, const double *,
                                     const double *, double *, double *, cudaStream_t);
 template cudaError_t ns_sums<double>(const void *, double2 *const[3], int64_t, int64_t, int64_t, const double *,
