@@ -21,9 +21,18 @@ __global__ void __launch_bounds__(NS_DECIDE_THREADS)
     __shared__ double red[NS_DECIDE_THREADS];
     grid_wait();
     grid_trigger(1);
-    const bool idle = ctl[NS_CTL_MORE] == 0;
+    // one thread reads the record and the loop's state for the block: it writes
+    // the record below, and the block that finishes last writes the state
+    __shared__ NsField rec;
+    __shared__ int over;
     const int64_t f = blockIdx.x;
-    NsField s = fs[f];
+    if (threadIdx.x == 0) {
+        rec = fs[f];
+        over = ctl[NS_CTL_MORE] == 0;
+    }
+    __syncthreads();
+    const bool idle = over != 0;
+    NsField s = rec;
     if (!idle && s.active) {  // the same for every thread of the block
         double sum = 0.0;
         for (int64_t g = threadIdx.x; g < groups; g += NS_DECIDE_THREADS) sum += partials[f * groups + g];
