@@ -446,9 +446,16 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
     template <int BLOCK> __device__ __forceinline__ void block_partial(double acc, double *out) const
     {
         __shared__ double red[32];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        if constexpr (BLOCK == 0) {
+            // the tile is one warp or less: only lanes that exist are named and read
+            const unsigned n = blockDim.x < 32 ? blockDim.x : 32;
+            const unsigned lanes = n < 32 ? (1u << n) - 1u : 0xffffffffu;
+            for (unsigned o = n / 2; o > 0; o >>= 1) acc += __shfl_down_sync(lanes, acc, o);
+        } else {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        }
         if constexpr (BLOCK > 1) {
             fft_sync<BLOCK>();
             if (lane == 0) red[warp] = acc;
@@ -459,7 +466,7 @@ template <class Rl, bool MID, bool HALF = false> struct NsCol {
                 *out = s;
             }
         } else if constexpr (BLOCK == 0) {
-            if (lane == 0) *out = acc;  // the tile is one warp (or less)
+            if (lane == 0) *out = acc;
         } else {
             __syncthreads();
             if (lane == 0) red[warp] = acc;
