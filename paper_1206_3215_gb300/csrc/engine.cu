@@ -1,4 +1,5 @@
 // Stepping drivers: which passes run, in which order, on which buffers.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdlib.h>
 #include <string.h>
@@ -30,20 +31,57 @@ template <class Rl> const TW<Rl> *Tw(const void *p) { return static_cast<const T
 cudaMemcpyKind kind_in(int where) { return where == PSS_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice; }
 cudaMemcpyKind kind_out(int where) { return where == PSS_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice; }
 
-// whether a kernel may read or write a caller's device array directly: memory
-// of the current device (or managed), aligned for the kernel's widest access; anything
-// else goes through a copy, which reports what it cannot do
-bool kernel_access(const void *p, size_t align)
+// The range [base, base + size) of the device allocation (or mapping) that holds
+// p, by the driver's cuMemGetAddressRange (looked up once through the runtime:
+// the library does not link the driver library); false where it has none.
+bool address_range(const void *p, uintptr_t *base, size_t *size)
 {
-    if (reinterpret_cast<uintptr_t>(p) % align) return false;
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    int dev = -1;
-    return cudaGetDevice(&dev) == cudaSuccess && at.device == dev &&
-           (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
+    using Range = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const Range range = []() -> Range {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &q);
+        if (e != cudaSuccess) cudaGetLastError();
+        return (e == cudaSuccess && q == cudaDriverEntryPointSuccess) ? reinterpret_cast<Range>(fn) : nullptr;
+    }();
+    CUdeviceptr b = 0;
+    if (!range || range(&b, size, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return false;
+    *base = uintptr_t(b);
+    return true;
+}
+
+// How the library reaches `bytes` bytes of a caller's device array.  DIRECT: a
+// kernel may read or write it: memory of the current device (or managed), inside
+// one allocation, aligned for the kernel's widest access.  SHORT: no memory
+// follows where the array would go on; the call is refused, as a copy of that
+// size would be (a kernel would fault).  COPY: anything else goes through a
+// copy, which reports what it cannot do.
+enum class Access { DIRECT, COPY, SHORT };
+Access kernel_access(const void *p, size_t align, size_t bytes)
+{
+    auto on_device = [](uintptr_t q) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, reinterpret_cast<const void *>(q)) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        int dev = -1;
+        return cudaGetDevice(&dev) == cudaSuccess && at.device == dev &&
+               (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
+    };
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    uintptr_t base = 0;
+    size_t size = 0;
+    if (!on_device(a) || !address_range(p, &base, &size)) return Access::COPY;
+    if (bytes <= base + size - a) return a % align ? Access::COPY : Access::DIRECT;
+    for (uintptr_t q = base + size; q - a < bytes; q = base + size)
+        if (!on_device(q) || !address_range(reinterpret_cast<const void *>(q), &base, &size)) return Access::SHORT;
+    return Access::COPY;
+}
+
+int short_array(pss_grid *g, const char *what, size_t bytes)
+{
+    return g->fail(PSS_E_CUDA, "%s: the device array is shorter than %zu bytes", what, bytes);
 }
 
 // Upload a per-axis table of n complex values given by f(m) -> (re, im) in FP64,
@@ -375,11 +413,13 @@ template <class Rl> int nls_set(pss_grid *g, int64_t f, int64_t nb, const void *
 {
     V2<Rl> *dst = B<Rl>(g, 0) + f * g->npts;
     const V2<Rl> *src = dst;
+    const size_t bytes = size_t(nb * g->npts) * g->esz;
+    const Access ac = where == PSS_DEVICE ? kernel_access(a, sizeof(V2<Rl>), bytes) : Access::COPY;
     int rc;
-    if (where == PSS_DEVICE && kernel_access(a, sizeof(V2<Rl>)))
+    if (ac == Access::SHORT) return short_array(g, "set_state", bytes);
+    if (ac == Access::DIRECT)
         src = C<Rl>(a);
-    else if ((rc = g->cuda(cudaMemcpyAsync(dst, a, size_t(nb * g->npts) * g->esz, kind_in(where), g->stream),
-                           "set_state copy")))
+    else if ((rc = g->cuda(cudaMemcpyAsync(dst, a, bytes, kind_in(where), g->stream), "set_state copy")))
         return rc;
     rc = g->cuda(fft_rows<Rl>(src, dst, g->nx, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twx), g->stream), "set_state row fft");
     if (rc) return rc;
@@ -424,12 +464,13 @@ template <class Rl> int nls_physical(pss_grid *g, int64_t f, int64_t nb, V2<Rl> 
 
 template <class Rl> int nls_get(pss_grid *g, int64_t f, int64_t nb, void *a, int where)
 {
-    const bool direct = where == PSS_DEVICE && kernel_access(a, sizeof(V2<Rl>));
-    V2<Rl> *dst = direct ? static_cast<V2<Rl> *>(a) : B<Rl>(g, 1) + f * g->npts;
+    const size_t bytes = size_t(nb * g->npts) * g->esz;
+    const Access ac = where == PSS_DEVICE ? kernel_access(a, sizeof(V2<Rl>), bytes) : Access::COPY;
+    if (ac == Access::SHORT) return short_array(g, "get_state", bytes);
+    V2<Rl> *dst = ac == Access::DIRECT ? static_cast<V2<Rl> *>(a) : B<Rl>(g, 1) + f * g->npts;
     int rc = nls_physical<Rl>(g, f, nb, dst);
-    if (!rc && !direct)
-        rc = g->cuda(cudaMemcpyAsync(a, dst, size_t(nb * g->npts) * g->esz, kind_out(where), g->stream),
-                     "get_state copy");
+    if (!rc && ac == Access::COPY)
+        rc = g->cuda(cudaMemcpyAsync(a, dst, bytes, kind_out(where), g->stream), "get_state copy");
     return rc ? rc : g->sync();
 }
 
@@ -512,12 +553,12 @@ template <class Rl> int sg_make_h(pss_grid *g, const SgState<Rl> &st)
 // where it is device memory aligned for that, else a copy in `tmp`.
 template <class Rl> int real_in(pss_grid *g, const void *src, int where, Rl *tmp, int64_t n, const Rl **out)
 {
-    if (where == PSS_DEVICE && kernel_access(src, 2 * sizeof(Rl))) {
-        *out = static_cast<const Rl *>(src);
-        return PSS_OK;
-    }
-    *out = tmp;
-    return g->cuda(cudaMemcpyAsync(tmp, src, size_t(n) * sizeof(Rl), kind_in(where), g->stream), "state copy");
+    const size_t bytes = size_t(n) * sizeof(Rl);
+    const Access ac = where == PSS_DEVICE ? kernel_access(src, 2 * sizeof(Rl), bytes) : Access::COPY;
+    if (ac == Access::SHORT) return short_array(g, "state", bytes);
+    *out = ac == Access::DIRECT ? static_cast<const Rl *>(src) : tmp;
+    if (ac == Access::DIRECT) return PSS_OK;
+    return g->cuda(cudaMemcpyAsync(tmp, src, bytes, kind_in(where), g->stream), "state copy");
 }
 
 // row transform of the real fields `a` into dst (rows of st.w)
@@ -638,14 +679,15 @@ template <class Rl> int sg_get_fields(pss_grid *g, int64_t f, int64_t nb, void *
 {
     const SgState<Rl> st = sg_state<Rl>(g, f, nb);
     void *const dst[2] = {a, b};
+    const size_t bytes = size_t(nb * g->npts) * sizeof(Rl);
     for (int k = 0; k < 2; ++k) {
         if (!dst[k]) continue;
-        const bool direct = where == PSS_DEVICE && kernel_access(dst[k], 2 * sizeof(Rl));
-        Rl *r = direct ? static_cast<Rl *>(dst[k]) : reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3));
+        const Access ac = where == PSS_DEVICE ? kernel_access(dst[k], 2 * sizeof(Rl), bytes) : Access::COPY;
+        if (ac == Access::SHORT) return short_array(g, "get_state", bytes);
+        Rl *r = ac == Access::DIRECT ? static_cast<Rl *>(dst[k]) : reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3));
         int rc = sg_real_of<Rl>(g, st, st.u, k ? st.d : nullptr, r);
-        if (!rc && !direct)
-            rc = g->cuda(cudaMemcpyAsync(dst[k], r, size_t(nb) * g->npts * sizeof(Rl), kind_out(where), g->stream),
-                         "state copy");
+        if (!rc && ac == Access::COPY)
+            rc = g->cuda(cudaMemcpyAsync(dst[k], r, bytes, kind_out(where), g->stream), "state copy");
         if (rc) return rc;
     }
     return g->sync();
@@ -879,9 +921,11 @@ template <class Rl> int ns_get(pss_grid *g, int64_t f, int64_t nb, void *a, int 
 {
     V2<Rl> *w[3];
     for (int i = 0; i < 3; ++i) w[i] = B<Rl>(g, i) + ns_off(g, f);
-    const bool direct = where == PSS_DEVICE && kernel_access(a, 2 * sizeof(Rl));
+    const size_t bytes = size_t(nb * g->npts) * sizeof(Rl);
+    const Access ac = where == PSS_DEVICE ? kernel_access(a, 2 * sizeof(Rl), bytes) : Access::COPY;
+    if (ac == Access::SHORT) return short_array(g, "get_state", bytes);
     // (J_hat^n in buf[3] is rebuilt at the start of every step)
-    Rl *dst = direct ? static_cast<Rl *>(a) : reinterpret_cast<Rl *>(g->buf[3]) + f * g->npts;
+    Rl *dst = ac == Access::DIRECT ? static_cast<Rl *>(a) : reinterpret_cast<Rl *>(g->buf[3]) + f * g->npts;
     V2<Rl> *t = Bf<Rl>(g, 6, f);
     const Rl s = Rl(1.0 / (double(g->nx) * double(g->ny)));
     int rc;
@@ -892,8 +936,8 @@ template <class Rl> int ns_get(pss_grid *g, int64_t f, int64_t nb, void *a, int 
                                                     g->stream)
                                  : rows_to_real<Rl>(t, dst, g->nx, g->ny, nb, Tw<Rl>(g->twx), g->stream),
                       "inverse rows")) ||
-        (!direct && (rc = g->cuda(cudaMemcpyAsync(a, dst, size_t(nb) * g->npts * sizeof(Rl), kind_out(where),
-                                                  g->stream), "state copy"))))
+        (ac == Access::COPY &&
+         (rc = g->cuda(cudaMemcpyAsync(a, dst, bytes, kind_out(where), g->stream), "state copy"))))
         return rc;
     return g->sync();
 }
