@@ -820,7 +820,8 @@ template <class Rl> int ns_body(pss_grid *g, int updates, bool in_graph)
     for (int u = 0; u < updates; ++u) {
         if (!in_graph && (rc = g->pass_begin(0))) return rc;
         cudaError_t e = ns_row_pass<Rl>(B<Rl>(g, 4), B<Rl>(g, 5), g->ns_field, g->nx, g->ny, g->batch, ctl,
-                                        Tw<Rl>(g->twx), g->stream, g->p.dealias != 0, g->ns_half);
+                                        Tw<Rl>(g->twx), g->stream, g->p.dealias != 0,
+                                        g->p.dealias != 0 && !g->ns_masked_modes, g->ns_half);
         if ((!in_graph && (rc = g->pass_end())) || (rc = g->cuda(e, "ns row pass"))) return rc;
         int groups = 0;
         if (!in_graph && (rc = g->pass_begin(1))) return rc;
@@ -996,6 +997,32 @@ template <class Rl> int field_get(pss_grid *g, int64_t f, void *a, void *b, int 
 
 #define PSS_BY_PRECISION(CALL) (p.precision == PSS_FP32 ? CALL(float) : CALL(double))
 
+// Whether a masked mode of the state may be non-zero (a dealiased grid that
+// restored another grid's checkpoint); the captured loop is rebuilt when that changes.
+void pss_grid::set_masked_modes(bool any)
+{
+    if (any == ns_masked_modes) return;
+    ns_masked_modes = any;
+    drop_graphs();
+}
+
+int pss_grid::find_masked_modes(bool *any)
+{
+    int *dev = reinterpret_cast<int *>(flags) + FLAG_SLOT_MASKED;
+    int *host = reinterpret_cast<int *>(host_flags) + FLAG_SLOT_MASKED;
+    int rc = cuda(cudaMemsetAsync(dev, 0, sizeof(int), stream), "masked modes");
+    if (rc) return rc;
+    const cudaError_t e = p.precision == PSS_FP32
+                              ? masked_columns<float>(B<float>(this, 0), Rt<float>(keepx), nx, ntot, dev, stream)
+                              : masked_columns<double>(B<double>(this, 0), Rt<double>(keepx), nx, ntot, dev, stream);
+    if ((rc = cuda(e, "masked modes")) ||
+        (rc = cuda(cudaMemcpyAsync(host, dev, sizeof(int), cudaMemcpyDeviceToHost, stream), "masked modes")) ||
+        (rc = cuda(cudaStreamSynchronize(stream), "masked modes")))
+        return rc;
+    *any = *host != 0;
+    return PSS_OK;
+}
+
 int pss_grid::set_state(const void *a, const void *b, int where)
 {
     steps = 0;
@@ -1012,6 +1039,7 @@ int pss_grid::set_state(const void *a, const void *b, int where)
         has_state = true;
         full_valid = !half;
         half_valid = half;
+        set_masked_modes(false);
     }
     return rc;
 }
@@ -1217,6 +1245,9 @@ int pss_grid::checkpoint(void *buf_, int where, bool save)
             for (int64_t i = 0; i < batch; ++i) h[i] = NsFieldHost{0, 0, 0, 0, i == 0 ? meta[1] : 0, 0, 0};
             rc = cuda(cudaMemcpyAsync(ns_field, h, size_t(batch) * ns_field_bytes(), cudaMemcpyHostToDevice, stream),
                       "fields");
+            bool masked = false;
+            if (!rc && p.dealias) rc = find_masked_modes(&masked);
+            if (!rc) set_masked_modes(masked);
             if (!rc && ns_half)
                 rc = p.precision == PSS_FP32 ? ns_to_half<float>(this, B<float>(this, 0), B<float>(this, 0), batch)
                                              : ns_to_half<double>(this, B<double>(this, 0), B<double>(this, 0), batch);

@@ -83,6 +83,9 @@ struct pss_grid {
     // captured CUDA graphs (NLS/SG: also while profiling; NS: off while
     // profiling; all off with PSS_GRAPHS=0)
     bool use_graphs = true;
+    bool ns_masked_modes = false;         // a mode the 2/3 rule masks may be non-zero: the row pass reads every column
+    void set_masked_modes(bool any);
+    int find_masked_modes(bool *any);     // of the full spectra in buf[0]; synchronises
     cudaGraph_t ns_graph = nullptr;       // NS: WHILE(steps left) { updates }
     cudaGraphExec_t ns_exec = nullptr;
     cudaGraphConditionalHandle ns_cond = 0;

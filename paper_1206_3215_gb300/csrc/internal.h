@@ -110,9 +110,10 @@ cudaError_t unpack_half(const V2<Rl> *half, V2<Rl> *full, int64_t nx, int64_t ny
 
 // ---- Navier-Stokes passes (k_ns.cu) -------------------------------------------
 size_t ns_field_bytes();  // bytes of the per-field fixed-point record
+// zero_in: the columns the 2/3 rule masks hold zeros in c1 and c2
 template <class Rl>
 cudaError_t ns_row_pass(V2<Rl> *c1, V2<Rl> *c2, const void *fs, int64_t nx, int64_t ny, int64_t batch,
-                        const int *ctl, const TW<Rl> *twx, cudaStream_t s, bool dealias, bool half = false);
+                        const int *ctl, const TW<Rl> *twx, cudaStream_t s, bool dealias, bool zero_in, bool half);
 template <class Rl>
 cudaError_t ns_col_pass(V2<Rl> *c1, V2<Rl> *c2, V2<Rl> *const w[3], V2<Rl> *jn, void *fs, double *partials,
                         const Rl *kxo, const Rl *kyo, const Rl *kx2, const Rl *ky2, const Rl *keepx,
@@ -136,6 +137,9 @@ cudaError_t ns_decide(void *fs, const double *partials, int64_t groups, int64_t 
                       cudaGraphConditionalHandle h, cudaStream_t s);
 
 // ---- elementwise helpers (k_util.cu) ----------------------------------------
+// *found |= 1 if a column with keepx = 0 of an array with rows of nx holds anything but zeros
+template <class Rl>
+cudaError_t masked_columns(const V2<Rl> *a, const Rl *keepx, int64_t nx, int64_t n, int *found, cudaStream_t s);
 template <class Rl>
 cudaError_t ns_gather(const void *fs, V2<Rl> *const w[3], V2<Rl> *dst, int64_t per_field, int64_t batch,
                       cudaStream_t s);
@@ -176,6 +180,7 @@ constexpr unsigned FLAG_NOT_CONVERGED = 2u;
 // int slot of the grid's 64-byte device flag block that pass kernels report
 // a lost tile copy in (slots 0 .. 3 and 6 carry the NS loop control, k_ns.cuh)
 constexpr int FLAG_SLOT_PASS_STATUS = 8;
+constexpr int FLAG_SLOT_MASKED = 7;  // scratch of masked_columns
 // NS split column pass: slot 4 its item counter (zeroed by k_ns_begin and
 // k_ns_decide), slot 5 the column-pass epoch (never reset; k_ns_decide
 // adds one), and from int FLAG_TILE_DONE on one word per column tile

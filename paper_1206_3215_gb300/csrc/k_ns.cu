@@ -114,8 +114,9 @@ __global__ void k_ns_begin(NsField *fs, int64_t batch, int *ctl, int n)
 // side by side: 246 us, 4096^2 940 (64 registers: 280, 1067).
 //
 // Dealiasing (2/3 rule): the columns with 3 |mx| >= nx hold zeros in C1 and C2
-// and are not read, and J is not written there (the column pass skips them,
-// the mask discards J); half spectra: J is written for columns 0 .. nx/2.
+// and are not read (zero_in; a restored state may have them filled), and J is
+// not written there (the column pass skips them, the mask discards J); half
+// spectra: J is written for columns 0 .. nx/2.
 constexpr int NS_ROW_MAX = 2048;
 template <int N> struct NsRowCfg {
     static constexpr int P = imin(Shape<float>::rowP(N), 16);
@@ -132,8 +133,8 @@ template <int N> struct NsRowCfg {
 
 template <int N>
 __global__ void __launch_bounds__(NsRowCfg<N>::THREADS, NsRowCfg<N>::MIN_CTAS)
-    k_ns_row(float2 *c1, const float2 *c2, const NsField *fs, int lgy, int dealias, int half, const int *ctl,
-             const float4 *__restrict__ tw, int64_t rows_total)
+    k_ns_row(float2 *c1, const float2 *c2, const NsField *fs, int lgy, int dealias, int zero_in, int half,
+             const int *ctl, const float4 *__restrict__ tw, int64_t rows_total)
 {
     using C = NsRowCfg<N>;
     using V = float2;
@@ -144,8 +145,9 @@ __global__ void __launch_bounds__(NsRowCfg<N>::THREADS, NsRowCfg<N>::MIN_CTAS)
     const int lr = threadIdx.x / T, t = threadIdx.x % T;
     const Sm sm{lines + lr * C::LINE}, park{lines + (C::ROWS + lr) * C::LINE};
     const int64_t tiles = (rows_total + C::ROWS - 1) / C::ROWS;
+    auto kept_col = [&](int x) { return 3 * (x < N / 2 ? x : N - x) < N; };
     // column x of C1, C2 is not known to be zero
-    auto live_col = [&](int x) { return !dealias || 3 * (x < N / 2 ? x : N - x) < N; };
+    auto live_col = [&](int x) { return !zero_in || kept_col(x); };
     auto issue = [&](int64_t tile, const V *in, const Sm &line) {
         const int64_t row = tile * C::ROWS + lr;
         if (tile < tiles && row < rows_total) {
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(NsRowCfg<N>::THREADS, NsRowCfg<N>::MIN_CTAS)
 #pragma unroll
             for (int m = 0; m < P; ++m) {
                 const int x = t + T * m;
-                if (live_col(x) && (!half || x <= N / 2)) p[T * m] = v[m];
+                if ((!dealias || kept_col(x)) && (!half || x <= N / 2)) p[T * m] = v[m];
             }
         }
     }
@@ -213,7 +215,7 @@ __global__ void __launch_bounds__(NsRowCfg<N>::THREADS, NsRowCfg<N>::MIN_CTAS)
 
 template <class Rl>
 cudaError_t ns_row_pass(V2<Rl> *c1, V2<Rl> *c2, const void *fs, int64_t nx, int64_t ny, int64_t batch,
-                        const int *ctl, const TW<Rl> *twx, cudaStream_t s, bool dealias, bool half)
+                        const int *ctl, const TW<Rl> *twx, cudaStream_t s, bool dealias, bool zero_in, bool half)
 {
     const NsField *f = static_cast<const NsField *>(fs);
     int lgy = 0;
@@ -231,10 +233,10 @@ cudaError_t ns_row_pass(V2<Rl> *c1, V2<Rl> *c2, const void *fs, int64_t nx, int6
         if ((e = resident_ctas(k, C::THREADS, C::SMEM, ctas, &grid)) != cudaSuccess) return e;
         if (tiles < grid) grid = int(tiles);
         return launch_chain(k, unsigned(grid), C::THREADS, C::SMEM, s, reinterpret_cast<float2 *>(c1),
-                            reinterpret_cast<const float2 *>(c2), f, lgy, dealias ? 1 : 0, half ? 1 : 0, ctl,
-                            reinterpret_cast<const float4 *>(twx), rows_total);
+                            reinterpret_cast<const float2 *>(c2), f, lgy, dealias ? 1 : 0, zero_in ? 1 : 0, half ? 1 : 0,
+                            ctl, reinterpret_cast<const float4 *>(twx), rows_total);
     };
-    const NsRow<Rl> op{c1, c2, f, lgy, dealias ? 1 : 0, half ? 1 : 0, ctl};
+    const NsRow<Rl> op{c1, c2, f, lgy, dealias ? 1 : 0, zero_in ? 1 : 0, half ? 1 : 0, ctl};
     switch (nx) {
 #define PSS_CASE(N)                                                                                       \
     case N:                                                                                               \
@@ -332,7 +334,7 @@ size_t ns_field_bytes() { return sizeof(NsField); }
     template cudaError_t ns_level_cols<Rl>(const void *, V2<Rl> *const[3], V2<Rl> *, Rl, int64_t, int64_t,   \
                                            int64_t, const TW<Rl> *, cudaStream_t);                           \
     template cudaError_t ns_row_pass<Rl>(V2<Rl> *, V2<Rl> *, const void *, int64_t, int64_t, int64_t,       \
-                                         const int *, const TW<Rl> *, cudaStream_t, bool, bool);             \
+                                         const int *, const TW<Rl> *, cudaStream_t, bool, bool, bool);       \
     template cudaError_t ns_col_pass<Rl>(V2<Rl> *, V2<Rl> *, V2<Rl> *const[3], V2<Rl> *, void *, double *,  \
                                          const Rl *, const Rl *, const Rl *, const Rl *, const Rl *,         \
                                          const Rl *, double, double, int64_t, int64_t, int64_t,             \

@@ -114,17 +114,15 @@ template <class Rl> struct NsRow {
     V2<Rl> *c1, *c2;  // in: C1, C2 rows; out: row transform of J into c1
     const NsField *fs;
     int lgy;      // log2 ny: row r belongs to field r >> lgy
-    int dealias;  // 2/3 rule: columns with 3 |mx| >= nx are not written (they stay
-                  // zero: the column pass skips them and the mask discards J there)
+    int dealias;  // 2/3 rule: columns with 3 |mx| >= nx are not written (the column
+                  // pass skips them and the mask discards J there)
+    int zero_in;  // and hold zeros in C1 and C2, so they are not read either
     int half;     // half spectra: only columns 0 .. nx/2 of J are read, so only they are written
     const int *ctl;
     __device__ __forceinline__ bool idle() const { return ctl[NS_CTL_ACTIVE] == 0; }
     __device__ const V2<Rl> *in(int k) const { return k == 0 ? c1 : c2; }
-    // the columns with 3 |mx| >= nx hold zeros in C1 and C2 (dealiasing)
-    template <int N> __device__ __forceinline__ bool live_col(int x) const
-    {
-        return !dealias || 3 * (x < N / 2 ? x : N - x) < N;
-    }
+    template <int N> static __device__ __forceinline__ bool kept_col(int x) { return 3 * (x < N / 2 ? x : N - x) < N; }
+    template <int N> __device__ __forceinline__ bool live_col(int x) const { return !zero_in || kept_col<N>(x); }
     template <int N, int P, int BLOCK, class Sm>
     __device__ __forceinline__ void row(V2<Rl> (&v)[2][P], int64_t r, bool ok, int t, const Sm (&sm)[2],
                                         const TW<Rl> *tw) const
@@ -143,7 +141,7 @@ template <class Rl> struct NsRow {
 #pragma unroll
         for (int m = 0; m < P; ++m, p += T) {
             const int x = t + T * m;
-            const bool kept = live_col<N>(x) && (!half || x <= N / 2);
+            const bool kept = (!dealias || kept_col<N>(x)) && (!half || x <= N / 2);
             if (live && kept) *p = v[0][m];
         }
     }

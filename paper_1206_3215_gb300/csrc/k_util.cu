@@ -36,6 +36,14 @@ __global__ void k_mask(V2<Rl> *a, const Rl *keepx, const Rl *keepy, int64_t nx, 
     }
 }
 
+template <class Rl> __global__ void k_masked_columns(const V2<Rl> *a, const Rl *keepx, int64_t nx, int64_t n, int *found)
+{
+    bool any = false;  // (NaN counts)
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+        if (keepx[i % nx] == Rl(0)) any = any || a[i].x != Rl(0) || a[i].y != Rl(0);
+    if (any) atomicOr(found, 1);
+}
+
 static unsigned blocks_for(int64_t n) { return unsigned(n / 256 + 1 < 4096 ? n / 256 + 1 : 4096); }
 
 template <class Rl>
@@ -61,8 +69,16 @@ cudaError_t apply_mask(V2<Rl> *a, const Rl *keepx, const Rl *keepy, int64_t nx, 
     return cudaGetLastError();
 }
 
+template <class Rl>
+cudaError_t masked_columns(const V2<Rl> *a, const Rl *keepx, int64_t nx, int64_t n, int *found, cudaStream_t s)
+{
+    k_masked_columns<Rl><<<blocks_for(n), 256, 0, s>>>(a, keepx, nx, n, found);
+    return cudaGetLastError();
+}
+
 #define PSS_INST(Rl)                                                                                      \
     template cudaError_t cplx_axpy<Rl>(const V2<Rl> *, const V2<Rl> *, Rl, V2<Rl> *, int64_t, cudaStream_t); \
+    template cudaError_t masked_columns<Rl>(const V2<Rl> *, const Rl *, int64_t, int64_t, int *, cudaStream_t); \
     template cudaError_t apply_mask<Rl>(V2<Rl> *, const Rl *, const Rl *, int64_t, int64_t, int64_t, cudaStream_t); \
     template cudaError_t ns_gather<Rl>(const void *, V2<Rl> *const[3], V2<Rl> *, int64_t, int64_t, cudaStream_t);
 PSS_INST(float)
