@@ -180,7 +180,6 @@ int pss_grid::init()
     if (p.eq == PSS_EQ_NS && p.rfft) {
         ns_half = true;
         nsx = nx / 2 + 8;  // a multiple of every column-tile width
-        if ((rc = upload_twiddles(this, nx / 2, &twm))) return rc;
     }
     if (p.eq == PSS_EQ_SG && p.rfft) {
         half = true;
@@ -545,16 +544,15 @@ template <class Rl> Rl sg_scale(pss_grid *g) { return Rl(1.0 / (double(g->nx) * 
 // H from uhat: the same scaling and transform as the step's column pass
 template <class Rl> int sg_make_h(pss_grid *g, const SgState<Rl> &st)
 {
-    return g->cuda(sg_level_cols<Rl>(st.u, nullptr, st.h, sg_scale<Rl>(g), st.w, g->ny, st.nb, Tw<Rl>(g->twy),
-                                     g->stream), "H");
+    return g->cuda(sg_level_cols<Rl>(st.u, st.h, sg_scale<Rl>(g), st.w, g->ny, st.nb, Tw<Rl>(g->twy), g->stream), "H");
 }
 
-// A caller's real array as the row kernels read it (pairs): the array itself
-// where it is device memory aligned for that, else a copy in `tmp`.
+// A caller's real array as a kernel reads it: the array itself where it can be,
+// else a copy in `tmp`.
 template <class Rl> int real_in(pss_grid *g, const void *src, int where, Rl *tmp, int64_t n, const Rl **out)
 {
     const size_t bytes = size_t(n) * sizeof(Rl);
-    const Access ac = where == PSS_DEVICE ? kernel_access(src, 2 * sizeof(Rl), bytes) : Access::COPY;
+    const Access ac = where == PSS_DEVICE ? kernel_access(src, sizeof(Rl), bytes) : Access::COPY;
     if (ac == Access::SHORT) return short_array(g, "state", bytes);
     *out = ac == Access::DIRECT ? static_cast<const Rl *>(src) : tmp;
     if (ac == Access::DIRECT) return PSS_OK;
@@ -564,8 +562,6 @@ template <class Rl> int real_in(pss_grid *g, const void *src, int where, Rl *tmp
 // row transform of the real fields `a` into dst (rows of st.w)
 template <class Rl> cudaError_t sg_split(pss_grid *g, const SgState<Rl> &st, const Rl *a, V2<Rl> *dst)
 {
-    if (g->half && sizeof(Rl) == 8)  // FP32: see k_sg_io.cu
-        return sg_half_split<Rl>(a, dst, g->nx, g->sx, g->ny, st.nb, Tw<Rl>(g->twm), Tw<Rl>(g->twx), g->stream);
     return rows_from_real<Rl>(a, dst, g->nx, g->half ? g->sx : 0, g->ny, st.nb, Tw<Rl>(g->twx), g->stream);
 }
 
@@ -577,15 +573,12 @@ template <class Rl> int sg_set_fields(pss_grid *g, int64_t f, int64_t nb, const 
     if ((rc = real_in<Rl>(g, u0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), nb * g->npts, &u)) ||
         (v0 && (rc = real_in<Rl>(g, v0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), nb * g->npts, &v))))
         return rc;
-    cudaError_t e;
-    if (g->half) {
-        e = sg_half_start<Rl>(u, v, st.d, g->p.dt, g->nx, g->sx, g->ny, nb, Tw<Rl>(g->twm), Tw<Rl>(g->twx), g->stream);
-    } else {
-        e = sg_start_field<Rl>(u, v, st.d, g->p.dt, nb * g->npts, g->stream);
-        if (e == cudaSuccess)
-            e = fft_rows<Rl>(st.d, st.d, g->nx, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twx), g->stream);
-    }
-    if ((rc = g->cuda(e, "start-up rows")) || (rc = g->cuda(sg_split<Rl>(g, st, u, st.u), "forward rows")) ||
+    // the start-up's physical part behind u's copy
+    const int64_t n = nb * g->npts;
+    Rl *start = reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)) + n;
+    if ((rc = g->cuda(sg_start_field<Rl>(u, v, start, g->p.dt, n, g->stream), "start-up field")) ||
+        (rc = g->cuda(sg_split<Rl>(g, st, start, st.d), "start-up rows")) ||
+        (rc = g->cuda(sg_split<Rl>(g, st, u, st.u), "forward rows")) ||
         (rc = g->cuda(fft_cols<Rl>(st.u, st.u, st.w, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
         (rc = g->cuda(sg_start_cols<Rl>(st.d, st.u, C<Rl>(g->sgcx), C<Rl>(g->sgcy), st.w, g->ny, nb, Tw<Rl>(g->twy),
                                         g->stream), "start-up columns")) ||
@@ -659,19 +652,16 @@ template <class Rl> int sg_step(pss_grid *g, int64_t n)
     return PSS_OK;
 }
 
-// real fields of the spectra a - b (b may be null) into dst: column pass into
-// scratch array 4, row pass into the real array
-template <class Rl>
-int sg_real_of(pss_grid *g, const SgState<Rl> &st, const V2<Rl> *a, const V2<Rl> *b, Rl *dst)
+// real fields of the spectra a - b (b may be null) into dst: row pass into
+// scratch array 4, column pass into the real array
+template <class Rl> int sg_real_of(pss_grid *g, const SgState<Rl> &st, V2<Rl> *a, const V2<Rl> *b, Rl *dst)
 {
-    V2<Rl> *t = sg_scratch<Rl>(g, st, 4);
-    int rc = g->cuda(sg_level_cols<Rl>(a, b, t, sg_scale<Rl>(g), st.w, g->ny, st.nb, Tw<Rl>(g->twy), g->stream),
-                     "inverse columns");
+    V2<Rl> *t = sg_scratch<Rl>(g, st, 4), *const src[3] = {a, a, a};
+    int rc = g->cuda(rows_inverse<Rl>(src, nullptr, 0, b, t, g->nx, g->half ? g->sx : 0, g->ny, st.nb, Tw<Rl>(g->twx),
+                                      g->stream), "inverse rows");
     if (rc) return rc;
-    return g->cuda(g->half ? sg_half_join<Rl>(t, dst, g->nx, g->sx, g->ny, st.nb, Tw<Rl>(g->twm), Tw<Rl>(g->twx),
-                                              g->stream)
-                           : rows_to_real<Rl>(t, dst, g->nx, g->ny, st.nb, Tw<Rl>(g->twx), g->stream),
-                   "inverse rows");
+    return g->cuda(cols_to_real<Rl>(t, dst, sg_scale<Rl>(g), g->nx, g->ny, st.nb, Tw<Rl>(g->twy), g->stream),
+                   "inverse columns");
 }
 
 // u^n -> a, u^{n-1} = F^-1 (uhat - d) -> b (may be null) of fields f .. f + nb - 1
@@ -682,7 +672,7 @@ template <class Rl> int sg_get_fields(pss_grid *g, int64_t f, int64_t nb, void *
     const size_t bytes = size_t(nb * g->npts) * sizeof(Rl);
     for (int k = 0; k < 2; ++k) {
         if (!dst[k]) continue;
-        const Access ac = where == PSS_DEVICE ? kernel_access(dst[k], 2 * sizeof(Rl), bytes) : Access::COPY;
+        const Access ac = where == PSS_DEVICE ? kernel_access(dst[k], sizeof(Rl), bytes) : Access::COPY;
         if (ac == Access::SHORT) return short_array(g, "get_state", bytes);
         Rl *r = ac == Access::DIRECT ? static_cast<Rl *>(dst[k]) : reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3));
         int rc = sg_real_of<Rl>(g, st, st.u, k ? st.d : nullptr, r);
@@ -698,17 +688,7 @@ template <class Rl> int sg_conserved(pss_grid *g, double *out)
     const SgState<Rl> st = sg_state<Rl>(g, 0, g->batch);
     Rl *X = reinterpret_cast<Rl *>(g->buf[3]), *Y = X + g->ntot;  // u^n, u^n - u^{n-1}
     int rc;
-    for (int k = 0; k < 2; ++k) {
-        const V2<Rl> *src = k ? st.d : st.u;
-        if (sizeof(Rl) == 8) {
-            if ((rc = sg_real_of<Rl>(g, st, src, nullptr, k ? Y : X))) return rc;
-        } else if ((rc = g->cuda(rows_inverse<Rl>(src, B<Rl>(g, 4), g->nx, g->half ? g->sx : 0, g->ny, g->batch,
-                                                  Tw<Rl>(g->twx), g->stream), "inverse rows")) ||
-                   (rc = g->cuda(cols_to_real<Rl>(B<Rl>(g, 4), k ? Y : X, sg_scale<Rl>(g), g->nx, g->ny, g->batch,
-                                                  Tw<Rl>(g->twy), g->stream), "inverse columns"))) {
-            return rc;
-        }
-    }
+    if ((rc = sg_real_of<Rl>(g, st, st.u, nullptr, X)) || (rc = sg_real_of<Rl>(g, st, st.d, nullptr, Y))) return rc;
     if ((rc = g->cuda(sg_sums<Rl>(X, Y, st.u, st.d, g->nx, g->ny, st.w, g->half, g->batch, g->kx2d, g->ky2d,
                                   g->p.dt, g->partials, g->sums, g->stream), "sg sums")) ||
         (rc = finish_sums(g)))
@@ -916,27 +896,25 @@ template <class Rl> int ns_current(pss_grid *g)
     return g->cuda(unpack_half<Rl>(B<Rl>(g, 3), B<Rl>(g, 6), g->nx, g->ny, g->nsx, g->batch, g->stream), "unpack");
 }
 
-// vorticity of fields f .. f + nb - 1 into a: column pass into buf[6], row pass
+// vorticity of fields f .. f + nb - 1 into a: row pass into buf[6], column pass
 // into the real array
 template <class Rl> int ns_get(pss_grid *g, int64_t f, int64_t nb, void *a, int where)
 {
     V2<Rl> *w[3];
     for (int i = 0; i < 3; ++i) w[i] = B<Rl>(g, i) + ns_off(g, f);
     const size_t bytes = size_t(nb * g->npts) * sizeof(Rl);
-    const Access ac = where == PSS_DEVICE ? kernel_access(a, 2 * sizeof(Rl), bytes) : Access::COPY;
+    const Access ac = where == PSS_DEVICE ? kernel_access(a, sizeof(Rl), bytes) : Access::COPY;
     if (ac == Access::SHORT) return short_array(g, "get_state", bytes);
     // (J_hat^n in buf[3] is rebuilt at the start of every step)
     Rl *dst = ac == Access::DIRECT ? static_cast<Rl *>(a) : reinterpret_cast<Rl *>(g->buf[3]) + f * g->npts;
     V2<Rl> *t = Bf<Rl>(g, 6, f);
     const Rl s = Rl(1.0 / (double(g->nx) * double(g->ny)));
     int rc;
-    if ((rc = g->cuda(ns_level_cols<Rl>(static_cast<char *>(g->ns_field) + f * ns_field_bytes(), w, t, s,
-                                        g->ns_half ? g->nsx : g->nx, g->ny, nb, Tw<Rl>(g->twy), g->stream),
-                      "inverse columns")) ||
-        (rc = g->cuda(g->ns_half ? sg_half_join<Rl>(t, dst, g->nx, g->nsx, g->ny, nb, Tw<Rl>(g->twm), Tw<Rl>(g->twx),
-                                                    g->stream)
-                                 : rows_to_real<Rl>(t, dst, g->nx, g->ny, nb, Tw<Rl>(g->twx), g->stream),
+    const int *rec = reinterpret_cast<const int *>(static_cast<char *>(g->ns_field) + f * ns_field_bytes());
+    if ((rc = g->cuda(rows_inverse<Rl>(w, rec, int64_t(ns_field_bytes() / sizeof(int)), nullptr, t, g->nx,
+                                       g->ns_half ? g->nsx : 0, g->ny, nb, Tw<Rl>(g->twx), g->stream),
                       "inverse rows")) ||
+        (rc = g->cuda(cols_to_real<Rl>(t, dst, s, g->nx, g->ny, nb, Tw<Rl>(g->twy), g->stream), "inverse columns")) ||
         (ac == Access::COPY &&
          (rc = g->cuda(cudaMemcpyAsync(a, dst, bytes, kind_out(where), g->stream), "state copy"))))
         return rc;

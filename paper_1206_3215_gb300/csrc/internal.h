@@ -61,42 +61,29 @@ cudaError_t sg_col_pass(V2<Rl> *h, V2<Rl> *u, V2<Rl> *d, int64_t nx, int64_t ny,
 template <class Rl>
 cudaError_t sg_row_pass_r2c(V2<Rl> *h, int64_t nx, int64_t sx, int64_t ny, int64_t batch, const TW<Rl> *twm,
                             const TW<Rl> *twn, cudaStream_t s);
-// Real rows and half spectra (k_sg_io.cu): row transform of a into h; of
-// dt v + (dt^2/2) sin u (v may be null) into h; inverse row transform of h into out.
+// dt v + (dt^2/2) sin u (v may be null) of n points (k_sg_io.cu).
 template <class Rl>
-cudaError_t sg_half_split(const Rl *a, V2<Rl> *h, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
-                          const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s);
-template <class Rl>
-cudaError_t sg_half_start(const Rl *u, const Rl *v, V2<Rl> *h, double dt, int64_t nx, int64_t sx, int64_t ny,
-                          int64_t batch, const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s);
-template <class Rl>
-cudaError_t sg_half_join(const V2<Rl> *h, Rl *out, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
-                         const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s);
-// dt v + (dt^2/2) sin u as a complex array of n points (full spectra).
-template <class Rl>
-cudaError_t sg_start_field(const Rl *u, const Rl *v, V2<Rl> *dst, double dt, int64_t n, cudaStream_t s);
+cudaError_t sg_start_field(const Rl *u, const Rl *v, Rl *dst, double dt, int64_t n, cudaStream_t s);
 // Complex transforms between real arrays and spectra, sx = 0: full spectra,
 // sx > 0: half spectra in rows of sx.  Row transform of real rows; inverse row
-// transform into full complex rows; real parts of an inverse row transform, or
-// of an inverse column transform times scale, into real arrays.
+// transform (of src - minus, minus may be null) into full complex rows; real
+// parts of an inverse column transform times scale into a real array.
+// sel (may be null: src[0]): field f is in src[sel[f * sel_stride]].
 template <class Rl>
 cudaError_t rows_from_real(const Rl *src, V2<Rl> *dst, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
                            const TW<Rl> *twx, cudaStream_t s);
 template <class Rl>
-cudaError_t rows_inverse(const V2<Rl> *src, V2<Rl> *dst, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
-                         const TW<Rl> *twx, cudaStream_t s);
-template <class Rl>
-cudaError_t rows_to_real(const V2<Rl> *src, Rl *dst, int64_t nx, int64_t ny, int64_t batch, const TW<Rl> *twx,
-                         cudaStream_t s);
+cudaError_t rows_inverse(V2<Rl> *const src[3], const int *sel, int64_t sel_stride, const V2<Rl> *minus, V2<Rl> *dst,
+                         int64_t nx, int64_t sx, int64_t ny, int64_t batch, const TW<Rl> *twx, cudaStream_t s);
 template <class Rl>
 cudaError_t cols_to_real(const V2<Rl> *src, Rl *dst, Rl scale, int64_t nx, int64_t ny, int64_t batch,
                          const TW<Rl> *twy, cudaStream_t s);
-// Columns of width nx, full or half: out = scale * inverse transform of a - b
-// (b may be null); data = transform of data + (dt^2/2) |k|^2 u, cx and cy
-// holding (dt^2/2) k^2 per axis as {hi, lo}.
+// Columns of width nx, full or half: out = scale * inverse transform of a;
+// data = transform of data + (dt^2/2) |k|^2 u, cx and cy holding
+// (dt^2/2) k^2 per axis as {hi, lo}.
 template <class Rl>
-cudaError_t sg_level_cols(const V2<Rl> *a, const V2<Rl> *b, V2<Rl> *out, Rl scale, int64_t nx, int64_t ny,
-                          int64_t batch, const TW<Rl> *twy, cudaStream_t s);
+cudaError_t sg_level_cols(const V2<Rl> *a, V2<Rl> *out, Rl scale, int64_t nx, int64_t ny, int64_t batch,
+                          const TW<Rl> *twy, cudaStream_t s);
 template <class Rl>
 cudaError_t sg_start_cols(V2<Rl> *data, const V2<Rl> *u, const V2<Rl> *cx, const V2<Rl> *cy, int64_t nx, int64_t ny,
                           int64_t batch, const TW<Rl> *twy, cudaStream_t s);
@@ -109,7 +96,7 @@ cudaError_t unpack_half(const V2<Rl> *half, V2<Rl> *full, int64_t nx, int64_t ny
                         cudaStream_t s);
 
 // ---- Navier-Stokes passes (k_ns.cu) -------------------------------------------
-size_t ns_field_bytes();  // bytes of the per-field fixed-point record
+size_t ns_field_bytes();  // bytes of the per-field fixed-point record; its first int is the field's current buffer
 // zero_in: the columns the 2/3 rule masks hold zeros in c1 and c2
 template <class Rl>
 cudaError_t ns_row_pass(V2<Rl> *c1, V2<Rl> *c2, const void *fs, int64_t nx, int64_t ny, int64_t batch,
@@ -124,11 +111,6 @@ template <class Rl>
 cudaError_t ns_prep_pass(V2<Rl> *const w[3], const void *fs, V2<Rl> *c1, V2<Rl> *c2, const Rl *kxo, const Rl *kyo,
                          const Rl *kx2, const Rl *ky2, int64_t nx, int64_t ny, int64_t batch,
                          const int *ctl, const TW<Rl> *twy, cudaStream_t s, int64_t sx = 0);
-// current vorticity of every field, column inverse transform times scale, into
-// out (rows of nx, full or half spectra)
-template <class Rl>
-cudaError_t ns_level_cols(const void *fs, V2<Rl> *const w[3], V2<Rl> *out, Rl scale, int64_t nx, int64_t ny,
-                          int64_t batch, const TW<Rl> *twy, cudaStream_t s);
 // Loop control (ctl: ints of the grid's flag block, k_ns.cuh): n steps of every
 // field; the decision after an update (`last`: the last one of a loop body).
 cudaError_t ns_begin(void *fs, int64_t batch, int *ctl, int n, cudaStream_t s);

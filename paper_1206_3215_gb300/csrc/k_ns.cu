@@ -290,49 +290,9 @@ cudaError_t ns_decide(void *fs, const double *partials, int64_t groups, int64_t 
                         use_graph ? 1 : 0, h);
 }
 
-namespace {
-// the current vorticity of every field (buffer fs[field].idx): column inverse
-// transform times scale into out
-template <class Rl> struct NsLevelCol {
-    static constexpr int NIN = 1;
-    static constexpr bool LEAN = true;
-    static constexpr int PMAX = 32;
-    static constexpr bool EARLY_NEXT = true;
-    const V2<Rl> *w0, *w1, *w2;
-    const NsField *fs;
-    V2<Rl> *out;
-    Rl scale;
-    int64_t nx;
-    __device__ const V2<Rl> *in(int, int64_t field) const
-    {
-        const int b = fs[field].idx;
-        return b == 0 ? w0 : b == 1 ? w1 : w2;
-    }
-    template <int N, int P, int BLOCK, class Sm, class H = NoHook>
-    __device__ __forceinline__ void col(V2<Rl> (&v)[1][P], int64_t field, int x, int t, const Sm (&sm)[1],
-                                        const TW<Rl> *tw, const H &hook = H{}) const
-    {
-        block_fft<N, P, +1, BLOCK>(v[0], sm[0], t, tw, hook);
-#pragma unroll
-        for (int m = 0; m < P; ++m) v[0][m] = cscale(v[0][m], scale);
-        store_line<P, N / P>(v[0], out + field * N * nx + x, nx, t, true);
-    }
-};
-}  // namespace
-
-template <class Rl>
-cudaError_t ns_level_cols(const void *fs, V2<Rl> *const w[3], V2<Rl> *out, Rl scale, int64_t nx, int64_t ny,
-                          int64_t batch, const TW<Rl> *twy, cudaStream_t s)
-{
-    return launch_col<Rl>(ny, nx, NsLevelCol<Rl>{w[0], w[1], w[2], static_cast<const NsField *>(fs), out, scale, nx},
-                          twy, batch, s);
-}
-
 size_t ns_field_bytes() { return sizeof(NsField); }
 
 #define PSS_INST(Rl)                                                                                         \
-    template cudaError_t ns_level_cols<Rl>(const void *, V2<Rl> *const[3], V2<Rl> *, Rl, int64_t, int64_t,   \
-                                           int64_t, const TW<Rl> *, cudaStream_t);                           \
     template cudaError_t ns_row_pass<Rl>(V2<Rl> *, V2<Rl> *, const void *, int64_t, int64_t, int64_t,       \
                                          const int *, const TW<Rl> *, cudaStream_t, bool, bool, bool);       \
     template cudaError_t ns_col_pass<Rl>(V2<Rl> *, V2<Rl> *, V2<Rl> *const[3], V2<Rl> *, void *, double *,  \

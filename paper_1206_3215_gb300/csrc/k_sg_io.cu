@@ -1,18 +1,22 @@
 // Sine-Gordon set-up and read-back: real fields <-> the stepping state
 // {uhat^n, d^n, H}, with full or half spectra.
 //
-// Reading u^n is one column pass (column inverse transform of uhat^n) and one
-// row pass that writes real rows; setting it is one row and one column pass
-// per array.  The start-up (backward Taylor step)
+// Reading u^n is one row pass (inverse, into full complex rows; half spectra are
+// extended as they are read) and one column pass that writes the real parts;
+// setting it is one row and one column pass per array.  The start-up (backward
+// Taylor step)
 //   d^0 = dt F v0 + (dt^2/2) (|k|^2 uhat^0 + F sin u0)
 //       = F [dt v0 + (dt^2/2) sin u0] + (dt^2/2) |k|^2 uhat^0
 // takes the physical-space sum through one transform; its factor
 // (dt^2/2) |k|^2 comes from per-axis tables made in FP64 (FP32: hi + lo).
 //
-// In FP32 uhat^0 and the real fields of the Hamiltonian go through full
-// complex rows (RowFromReal, RowInv): half-length transforms of packed pairs
-// round differently, which moves the Hamiltonian of a small field by up to
-// 1e-8.
+// Half spectra could be read with half the columns (columns first) and with
+// half-length rows of packed pairs, as the step's row pass has them.  Both cost
+// accuracy: taking the real part at the end drops half of the rounding error
+// that a full complex transform has collected.  Read-back alone at 512^2, FP32
+// / FP64: as here 1.10e-7 / 2.2e-16, columns first 1.27e-7 / 2.7e-16,
+// half-length rows 1.38e-7 / 2.9e-16; 2048^2 x 8 FP32 takes 0.05 ms more per
+// level than with half the bytes.
 //
 // 2048^2 x 8 on half spectra, against transforms of full complex arrays with
 // separate copies, conversions and FP64 elementwise kernels (sums of kernel
@@ -20,21 +24,21 @@
 // Hamiltonian 3.6 -> 1.9 ms.
 #include <algorithm>
 
-#include "k_sg_r2c.cuh"
+#include "launch.cuh"
+#include "sg_sin.cuh"
 
 namespace pss {
 
 namespace {
 
-// a - b (b may be null) of two spectra, column inverse transform times scale,
-// into out.  The arithmetic is that of the second half of the step's column
+// H of uhat: column inverse transform of a times scale, into out.  The arithmetic is that of the second half of the step's column
 // pass (SgCol), so H made here from uhat is the H the step left, bit for bit.
 template <class Rl> struct SgLevelCol {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
     static constexpr bool EARLY_NEXT = true;
-    const V2<Rl> *a, *b;
+    const V2<Rl> *a;
     V2<Rl> *out;
     Rl scale;
     int64_t nx;
@@ -46,9 +50,6 @@ template <class Rl> struct SgLevelCol {
         constexpr int T = N / P;
         V2<Rl>(&v)[P] = vv[0];
         const int64_t base = field * N * nx + x;
-        if (b)
-#pragma unroll
-            for (int m = 0; m < P; ++m) v[m] = csub(v[m], b[base + int64_t(t + T * m) * nx]);
 #pragma unroll
         for (int m = 0; m < P; ++m) v[m] = cscale(v[m], scale);
         if constexpr (sizeof(Rl) == 4) {
@@ -97,26 +98,6 @@ template <class Rl> struct SgStartCol {
     static __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 };
 
-// rows of a complex array, inverse row transform, real parts into real rows
-template <class Rl> struct RowToReal {
-    static constexpr int NIN = 1;
-    static constexpr bool LEAN = true;
-    static constexpr int PMAX = 32;
-    static constexpr bool EARLY_NEXT = true;
-    const V2<Rl> *src;
-    Rl *dst;
-    __device__ const V2<Rl> *in(int) const { return src; }
-    template <int N, int P, int BLOCK, class Sm, class H = NoHook>
-    __device__ __forceinline__ void row(V2<Rl> (&v)[1][P], int64_t r, bool ok, int t, const Sm (&sm)[1],
-                                        const TW<Rl> *tw, const H &hook = H{}) const
-    {
-        block_fft<N, P, +1, BLOCK>(v[0], sm[0], t, tw, hook);
-        if (!ok) return;
-#pragma unroll
-        for (int m = 0; m < P; ++m) dst[r * N + t + (N / P) * m] = v[0][m].x;
-    }
-};
-
 // real rows, complex forward row transform, columns 0 .. N/2 (half spectra:
 // rows of sx, zeros beyond) or all of them (sx = 0)
 template <class Rl> struct RowFromReal {
@@ -149,17 +130,26 @@ template <class Rl> struct RowFromReal {
     }
 };
 
-// inverse row transform of full spectra (sx = 0) or of half spectra extended
-// by their Hermitian symmetry, into full complex rows
+// inverse row transform of full spectra (sx = 0), or of half spectra (rows of sx)
+// extended by their Hermitian symmetry, into full complex rows; of the
+// difference with a second spectrum where `minus` is set.  With sel, field f is
+// in src[sel[f * sel_stride]].
 template <class Rl> struct RowInv {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
     static constexpr bool DIRECT_LOAD = true;
-    const V2<Rl> *src;
+    const V2<Rl> *src[3], *minus;
+    const int *sel;
+    int64_t sel_stride;
     V2<Rl> *dst;
     int64_t sx, ny;  // ny: a power of two
+    int lgy;
     __device__ const V2<Rl> *in(int) const { return nullptr; }
+    __device__ __forceinline__ V2<Rl> at(const V2<Rl> *a, int64_t i) const
+    {
+        return minus ? csub(a[i], minus[i]) : a[i];
+    }
     template <int N, int P>
     __device__ __forceinline__ void load(V2<Rl> (&v)[P], int64_t r, bool ok, int t) const
     {
@@ -170,14 +160,16 @@ template <class Rl> struct RowInv {
             return;
         }
         const int64_t y = r & (ny - 1);
-        const V2<Rl> *p = src + r * (sx ? sx : N), *q = src + (r - y + ((ny - y) & (ny - 1))) * sx;
+        const int b = sel ? sel[(r >> lgy) * sel_stride] : 0;
+        const V2<Rl> *a = b == 0 ? src[0] : b == 1 ? src[1] : src[2];
+        const int64_t p = r * (sx ? sx : N), q = (r - y + ((ny - y) & (ny - 1))) * sx;
 #pragma unroll
         for (int m = 0; m < P; ++m) {
             const int x = t + T * m;
             if (!sx || x <= N / 2) {
-                v[m] = p[x];
+                v[m] = at(a, p + x);
             } else {
-                const V2<Rl> c = q[N - x];
+                const V2<Rl> c = at(a, q + N - x);
                 v[m] = V2<Rl>{c.x, -c.y};
             }
         }
@@ -215,48 +207,28 @@ template <class Rl> struct ColToReal {
     }
 };
 
-// dt v + (dt^2/2) sin u (v may be null), as a complex array
-template <class Rl> __global__ void k_sg_start(const Rl *u, const Rl *v, V2<Rl> *dst, HalfRowArgs<Rl> g, int64_t n)
-{
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-        dst[i] = V2<Rl>{half_start(g, u[i], v ? v[i] : Rl(0)), Rl(0)};
-}
+// Constants of the start-up: dt and dt^2/2 (FP32: and the rests of their rounding)
+template <class Rl> struct StartArgs {
+    Rl dt, dt_lo, dt2_2, dt2_2_lo;
+};
 
-// the start-up's arguments: rows `a`, `b` into half spectra h
-template <class Rl> HalfRowArgs<Rl> start_args(V2<Rl> *h, const Rl *a, const Rl *b, int64_t sx, double dt)
+// dt v + (dt^2/2) sin u (v may be null); the rests of the constants enter inside
+// the fused multiply-adds, so that their rounding does not scale the whole field
+template <class Rl> __global__ void k_sg_start(const Rl *u, const Rl *v, Rl *dst, StartArgs<Rl> g, int64_t n)
 {
-    const double d2 = 0.5 * dt * dt;
-    return {h, reinterpret_cast<const V2<Rl> *>(a), reinterpret_cast<const V2<Rl> *>(b), nullptr, sx,
-            Rl(dt), Rl(dt - double(Rl(dt))), Rl(d2), Rl(d2 - double(Rl(d2)))};
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+        const Rl s = sg_sin(u[i]), w = v ? v[i] : Rl(0);
+        dst[i] = g.dt * w + (g.dt2_2 * s + (g.dt_lo * w + g.dt2_2_lo * s));
+    }
 }
 
 }  // namespace
 
 template <class Rl>
-cudaError_t sg_half_split(const Rl *a, V2<Rl> *h, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
-                          const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s)
+cudaError_t sg_level_cols(const V2<Rl> *a, V2<Rl> *out, Rl scale, int64_t nx, int64_t ny, int64_t batch,
+                          const TW<Rl> *twy, cudaStream_t s)
 {
-    return half_rows<Rl, HalfRow::SPLIT>(start_args<Rl>(h, a, nullptr, sx, 0.0), nx, ny, batch, twm, twn, s);
-}
-template <class Rl>
-cudaError_t sg_half_start(const Rl *u, const Rl *v, V2<Rl> *h, double dt, int64_t nx, int64_t sx, int64_t ny,
-                          int64_t batch, const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s)
-{
-    return half_rows<Rl, HalfRow::START>(start_args<Rl>(h, u, v, sx, dt), nx, ny, batch, twm, twn, s);
-}
-template <class Rl>
-cudaError_t sg_half_join(const V2<Rl> *h, Rl *out, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
-                         const TW<Rl> *twm, const TW<Rl> *twn, cudaStream_t s)
-{
-    HalfRowArgs<Rl> g = start_args<Rl>(const_cast<V2<Rl> *>(h), nullptr, nullptr, sx, 0.0);
-    g.out = reinterpret_cast<V2<Rl> *>(out);
-    return half_rows<Rl, HalfRow::JOIN>(g, nx, ny, batch, twm, twn, s);
-}
-template <class Rl>
-cudaError_t sg_level_cols(const V2<Rl> *a, const V2<Rl> *b, V2<Rl> *out, Rl scale, int64_t nx, int64_t ny,
-                          int64_t batch, const TW<Rl> *twy, cudaStream_t s)
-{
-    return launch_col<Rl>(ny, nx, SgLevelCol<Rl>{a, b, out, scale, nx}, twy, batch, s);
+    return launch_col<Rl>(ny, nx, SgLevelCol<Rl>{a, out, scale, nx}, twy, batch, s);
 }
 template <class Rl>
 cudaError_t sg_start_cols(V2<Rl> *data, const V2<Rl> *u, const V2<Rl> *cx, const V2<Rl> *cy, int64_t nx, int64_t ny,
@@ -265,22 +237,19 @@ cudaError_t sg_start_cols(V2<Rl> *data, const V2<Rl> *u, const V2<Rl> *cx, const
     return launch_col<Rl>(ny, nx, SgStartCol<Rl>{data, u, cx, cy, nx}, twy, batch, s);
 }
 template <class Rl>
-cudaError_t rows_to_real(const V2<Rl> *src, Rl *dst, int64_t nx, int64_t ny, int64_t batch, const TW<Rl> *twx,
-                         cudaStream_t s)
-{
-    return launch_row<Rl>(nx, ny, RowToReal<Rl>{src, dst}, twx, batch, s);
-}
-template <class Rl>
 cudaError_t rows_from_real(const Rl *src, V2<Rl> *dst, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
                            const TW<Rl> *twx, cudaStream_t s)
 {
     return launch_row<Rl>(nx, ny, RowFromReal<Rl>{src, dst, sx}, twx, batch, s);
 }
 template <class Rl>
-cudaError_t rows_inverse(const V2<Rl> *src, V2<Rl> *dst, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
-                         const TW<Rl> *twx, cudaStream_t s)
+cudaError_t rows_inverse(V2<Rl> *const src[3], const int *sel, int64_t sel_stride, const V2<Rl> *minus, V2<Rl> *dst,
+                         int64_t nx, int64_t sx, int64_t ny, int64_t batch, const TW<Rl> *twx, cudaStream_t s)
 {
-    return launch_row<Rl>(nx, ny, RowInv<Rl>{src, dst, sx, ny}, twx, batch, s);
+    int lgy = 0;
+    while ((int64_t(1) << lgy) < ny) ++lgy;
+    return launch_row<Rl>(nx, ny, RowInv<Rl>{{src[0], src[1], src[2]}, minus, sel, sel_stride, dst, sx, ny, lgy}, twx,
+                          batch, s);
 }
 template <class Rl>
 cudaError_t cols_to_real(const V2<Rl> *src, Rl *dst, Rl scale, int64_t nx, int64_t ny, int64_t batch,
@@ -289,33 +258,27 @@ cudaError_t cols_to_real(const V2<Rl> *src, Rl *dst, Rl scale, int64_t nx, int64
     return launch_col<Rl>(ny, nx, ColToReal<Rl>{src, dst, scale, nx}, twy, batch, s);
 }
 template <class Rl>
-cudaError_t sg_start_field(const Rl *u, const Rl *v, V2<Rl> *dst, double dt, int64_t n, cudaStream_t s)
+cudaError_t sg_start_field(const Rl *u, const Rl *v, Rl *dst, double dt, int64_t n, cudaStream_t s)
 {
+    const double d2 = 0.5 * dt * dt;
+    const StartArgs<Rl> g{Rl(dt), Rl(dt - double(Rl(dt))), Rl(d2), Rl(d2 - double(Rl(d2)))};
     const unsigned blocks = unsigned(std::min<int64_t>((n + 255) / 256, 4096));
-    k_sg_start<Rl><<<blocks, 256, 0, s>>>(u, v, dst, start_args<Rl>(nullptr, nullptr, nullptr, 0, dt), n);
+    k_sg_start<Rl><<<blocks, 256, 0, s>>>(u, v, dst, g, n);
     return cudaGetLastError();
 }
 
 #define PSS_INST(Rl)                                                                                             \
-    template cudaError_t sg_half_split<Rl>(const Rl *, V2<Rl> *, int64_t, int64_t, int64_t, int64_t,             \
-                                           const TW<Rl> *, const TW<Rl> *, cudaStream_t);                        \
-    template cudaError_t sg_half_start<Rl>(const Rl *, const Rl *, V2<Rl> *, double, int64_t, int64_t, int64_t,  \
-                                           int64_t, const TW<Rl> *, const TW<Rl> *, cudaStream_t);               \
-    template cudaError_t sg_half_join<Rl>(const V2<Rl> *, Rl *, int64_t, int64_t, int64_t, int64_t,              \
-                                          const TW<Rl> *, const TW<Rl> *, cudaStream_t);                         \
-    template cudaError_t sg_level_cols<Rl>(const V2<Rl> *, const V2<Rl> *, V2<Rl> *, Rl, int64_t, int64_t,       \
-                                           int64_t, const TW<Rl> *, cudaStream_t);                               \
+    template cudaError_t sg_level_cols<Rl>(const V2<Rl> *, V2<Rl> *, Rl, int64_t, int64_t, int64_t,              \
+                                           const TW<Rl> *, cudaStream_t);                                        \
     template cudaError_t sg_start_cols<Rl>(V2<Rl> *, const V2<Rl> *, const V2<Rl> *, const V2<Rl> *, int64_t,    \
                                            int64_t, int64_t, const TW<Rl> *, cudaStream_t);                      \
-    template cudaError_t rows_to_real<Rl>(const V2<Rl> *, Rl *, int64_t, int64_t, int64_t, const TW<Rl> *,       \
-                                          cudaStream_t);                                                         \
     template cudaError_t rows_from_real<Rl>(const Rl *, V2<Rl> *, int64_t, int64_t, int64_t, int64_t,            \
                                             const TW<Rl> *, cudaStream_t);                                       \
-    template cudaError_t rows_inverse<Rl>(const V2<Rl> *, V2<Rl> *, int64_t, int64_t, int64_t, int64_t,          \
-                                          const TW<Rl> *, cudaStream_t);                                         \
+    template cudaError_t rows_inverse<Rl>(V2<Rl> *const[3], const int *, int64_t, const V2<Rl> *, V2<Rl> *,      \
+                                          int64_t, int64_t, int64_t, int64_t, const TW<Rl> *, cudaStream_t);     \
     template cudaError_t cols_to_real<Rl>(const V2<Rl> *, Rl *, Rl, int64_t, int64_t, int64_t, const TW<Rl> *,   \
                                           cudaStream_t);                                                         \
-    template cudaError_t sg_start_field<Rl>(const Rl *, const Rl *, V2<Rl> *, double, int64_t, cudaStream_t);
+    template cudaError_t sg_start_field<Rl>(const Rl *, const Rl *, Rl *, double, int64_t, cudaStream_t);
 PSS_INST(float)
 PSS_INST(double)
 
