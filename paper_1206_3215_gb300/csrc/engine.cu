@@ -195,18 +195,16 @@ int pss_grid::init()
         if ((rc = p.precision == PSS_FP32 ? upload_real<float>(this, kh, &kx2h) : upload_real<double>(this, kh, &kx2h)))
             return rc;
     }
-    if (p.eq == PSS_EQ_SG) {
-        // (dt^2/2) k^2 per axis, {hi, lo} in the grid's precision (start-up)
+    if (p.eq == PSS_EQ_SG && p.precision == PSS_FP32) {
+        // (dt^2/2) k^2 per axis as {hi, lo} (start-up)
         auto halves = [&](const std::vector<double> &k2, void **dst) {
-            std::vector<double> t(2 * k2.size());
-            std::vector<float> tf(2 * k2.size());
+            std::vector<float> t(2 * k2.size());
             for (size_t m = 0; m < k2.size(); ++m) {
                 const double c = 0.5 * p.dt * p.dt * k2[m];
-                t[2 * m] = c;
-                tf[2 * m] = float(c);
-                tf[2 * m + 1] = float(c - double(float(c)));
+                t[2 * m] = float(c);
+                t[2 * m + 1] = float(c - double(float(c)));
             }
-            return p.precision == PSS_FP32 ? upload(dst, tf.data(), tf.size() * 4) : upload(dst, t.data(), t.size() * 8);
+            return upload(dst, t.data(), t.size() * 4);
         };
         if ((rc = halves(kx2v, &sgcx)) || (rc = halves(ky2v, &sgcy))) return rc;
     }
@@ -568,20 +566,24 @@ template <class Rl> cudaError_t sg_split(pss_grid *g, const SgState<Rl> &st, con
 template <class Rl> int sg_set_fields(pss_grid *g, int64_t f, int64_t nb, const void *u0, const void *v0, int where)
 {
     const SgState<Rl> st = sg_state<Rl>(g, f, nb);
-    const Rl *u = nullptr, *v = nullptr;
-    int rc;
-    if ((rc = real_in<Rl>(g, u0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), nb * g->npts, &u)) ||
-        (v0 && (rc = real_in<Rl>(g, v0, where, reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4)), nb * g->npts, &v))))
-        return rc;
-    // the start-up's physical part behind u's copy
     const int64_t n = nb * g->npts;
-    Rl *start = reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)) + n;
-    if ((rc = g->cuda(sg_start_field<Rl>(u, v, start, g->p.dt, n, g->stream), "start-up field")) ||
-        (rc = g->cuda(sg_split<Rl>(g, st, start, st.d), "start-up rows")) ||
-        (rc = g->cuda(sg_split<Rl>(g, st, u, st.u), "forward rows")) ||
-        (rc = g->cuda(fft_cols<Rl>(st.u, st.u, st.w, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream), "forward columns")) ||
-        (rc = g->cuda(sg_start_cols<Rl>(st.d, st.u, C<Rl>(g->sgcx), C<Rl>(g->sgcy), st.w, g->ny, nb, Tw<Rl>(g->twy),
-                                        g->stream), "start-up columns")) ||
+    // scratch: copies of u and v in array 3; sin u, then the transform of v, in array 4
+    Rl *copies = reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 3)), *sine = reinterpret_cast<Rl *>(sg_scratch<Rl>(g, st, 4));
+    V2<Rl> *vh = v0 ? sg_scratch<Rl>(g, st, 4) : nullptr;
+    const Rl *u = nullptr, *v = nullptr;
+    auto cols = [&](V2<Rl> *a) {
+        return fft_cols<Rl>(a, a, st.w, g->ny, nb, -1, Rl(1), Tw<Rl>(g->twy), g->stream);
+    };
+    int rc;
+    if ((rc = real_in<Rl>(g, u0, where, copies, n, &u)) || (v0 && (rc = real_in<Rl>(g, v0, where, copies + n, n, &v))))
+        return rc;
+    if ((rc = g->cuda(sg_sine<Rl>(u, sine, n, g->stream), "sin u")) ||
+        (rc = g->cuda(sg_split<Rl>(g, st, sine, st.d), "forward rows")) ||
+        (rc = g->cuda(sg_split<Rl>(g, st, u, st.u), "forward rows")) || (rc = g->cuda(cols(st.u), "forward columns")) ||
+        (vh && (rc = g->cuda(sg_split<Rl>(g, st, v, vh), "forward rows"))) ||
+        (vh && (rc = g->cuda(cols(vh), "forward columns"))) ||
+        (rc = g->cuda(sg_start_cols<Rl>(st.d, st.u, vh, g->p.dt, C<Rl>(g->sgcx), C<Rl>(g->sgcy), g->kx2d, g->ky2d, st.w,
+                                        g->ny, nb, Tw<Rl>(g->twy), g->stream), "start-up columns")) ||
         (rc = sg_make_h<Rl>(g, st)))
         return rc;
     return where == PSS_HOST ? g->cuda(cudaStreamSynchronize(g->stream), "set_state sync") : PSS_OK;

@@ -34,7 +34,7 @@ struct pss_grid {
     void *hbuf[3] = {};
     void *twm = nullptr;   // twiddles of length nx/2
     void *kx2h = nullptr;  // kx^2 of the half-spectrum columns (0 beyond nx/2)
-    void *sgcx = nullptr, *sgcy = nullptr;  // (dt^2/2) k^2 per axis, {hi, lo}
+    void *sgcx = nullptr, *sgcy = nullptr;  // FP32: (dt^2/2) k^2 per axis, {hi, lo}
     bool half_valid = false, full_valid = true;
     int half_sync(bool to_half);  // make the half (true) or full (false) copy current
     // Navier-Stokes on half spectra (p.rfft): the vorticity iterates and

@@ -61,9 +61,8 @@ cudaError_t sg_col_pass(V2<Rl> *h, V2<Rl> *u, V2<Rl> *d, int64_t nx, int64_t ny,
 template <class Rl>
 cudaError_t sg_row_pass_r2c(V2<Rl> *h, int64_t nx, int64_t sx, int64_t ny, int64_t batch, const TW<Rl> *twm,
                             const TW<Rl> *twn, cudaStream_t s);
-// dt v + (dt^2/2) sin u (v may be null) of n points (k_sg_io.cu).
-template <class Rl>
-cudaError_t sg_start_field(const Rl *u, const Rl *v, Rl *dst, double dt, int64_t n, cudaStream_t s);
+// sin u of n points, the rounded value (k_sg_io.cu).
+template <class Rl> cudaError_t sg_sine(const Rl *u, Rl *dst, int64_t n, cudaStream_t s);
 // Complex transforms between real arrays and spectra, sx = 0: full spectra,
 // sx > 0: half spectra in rows of sx.  Row transform of real rows; inverse row
 // transform (of src - minus, minus may be null) into full complex rows; real
@@ -79,14 +78,15 @@ template <class Rl>
 cudaError_t cols_to_real(const V2<Rl> *src, Rl *dst, Rl scale, int64_t nx, int64_t ny, int64_t batch,
                          const TW<Rl> *twy, cudaStream_t s);
 // Columns of width nx, full or half: out = scale * inverse transform of a;
-// data = transform of data + (dt^2/2) |k|^2 u, cx and cy holding
-// (dt^2/2) k^2 per axis as {hi, lo}.
+// data = dt v + (dt^2/2) (|k|^2 u + transform of data), v may be null, cx and cy
+// holding (dt^2/2) k^2 per axis as {hi, lo} (FP32), kx2 and ky2 k^2 (FP64).
 template <class Rl>
 cudaError_t sg_level_cols(const V2<Rl> *a, V2<Rl> *out, Rl scale, int64_t nx, int64_t ny, int64_t batch,
                           const TW<Rl> *twy, cudaStream_t s);
 template <class Rl>
-cudaError_t sg_start_cols(V2<Rl> *data, const V2<Rl> *u, const V2<Rl> *cx, const V2<Rl> *cy, int64_t nx, int64_t ny,
-                          int64_t batch, const TW<Rl> *twy, cudaStream_t s);
+cudaError_t sg_start_cols(V2<Rl> *data, const V2<Rl> *u, const V2<Rl> *v, double dt, const V2<Rl> *cx, const V2<Rl> *cy,
+                          const double *kx2, const double *ky2, int64_t nx, int64_t ny, int64_t batch,
+                          const TW<Rl> *twy, cudaStream_t s);
 // full [batch][ny][nx] spectrum of real fields <-> half spectrum [batch][ny][sx]
 template <class Rl>
 cudaError_t pack_half(const V2<Rl> *full, V2<Rl> *half, int64_t nx, int64_t ny, int64_t sx, int64_t batch,

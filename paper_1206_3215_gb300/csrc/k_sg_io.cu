@@ -4,11 +4,11 @@
 // Reading u^n is one row pass (inverse, into full complex rows; half spectra are
 // extended as they are read) and one column pass that writes the real parts;
 // setting it is one row and one column pass per array.  The start-up (backward
-// Taylor step)
-//   d^0 = dt F v0 + (dt^2/2) (|k|^2 uhat^0 + F sin u0)
-//       = F [dt v0 + (dt^2/2) sin u0] + (dt^2/2) |k|^2 uhat^0
-// takes the physical-space sum through one transform; its factor
-// (dt^2/2) |k|^2 comes from per-axis tables made in FP64 (FP32: hi + lo).
+// Taylor step) is
+//   d^0 = dt F v0 + (dt^2/2) (|k|^2 uhat^0 + F sin u0),
+// each of the three transforms rounded to the grid's precision, their sum
+// formed in double (FP32: in pairs of floats) and rounded once, and sin u0 the
+// rounded value of the sine in double (FP32: again through pairs where it can be).
 //
 // Half spectra could be read with half the columns (columns first) and with
 // half-length rows of packed pairs, as the step's row pass has them.  Both cost
@@ -25,7 +25,6 @@
 #include <algorithm>
 
 #include "launch.cuh"
-#include "sg_sin.cuh"
 
 namespace pss {
 
@@ -63,16 +62,43 @@ template <class Rl> struct SgLevelCol {
     }
 };
 
-// the start-up's second term: data = column transform of data + c u,
-// c = (dt^2/2) (kx^2 + ky^2) from the per-axis tables
+// A sum of products held as an unevaluated pair of floats: the error of each
+// product (fused multiply-add) and of each addition (Knuth's two-sum) collects
+// in lo, so that hi + lo rounds once, as a sum in double would.  Roundings are
+// written out: the compiler must not fuse across them.
+struct PairSum {
+    float hi, lo;
+    // + (c + cl) x
+    __device__ __forceinline__ void add(float c, float cl, float x)
+    {
+        const float p = __fmul_rn(c, x), e = __fmaf_rn(cl, x, __fmaf_rn(c, x, -p));
+        const float s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b))));
+        hi = s;
+    }
+    __device__ __forceinline__ float value() const { return __fadd_rn(hi, lo); }
+};
+
+// constants of the start-up and their rests below the grid's precision (FP64: 0)
+template <class Rl> struct StartArgs {
+    Rl dt, dt_lo, h, h_lo;  // dt and dt^2/2
+    double dt64, h64;
+};
+
+// the start-up's column pass: data = dt v + (dt^2/2) (|k|^2 u + column transform
+// of data), u and v (may be null) transformed already.  |k|^2 from the per-axis
+// tables in double, or (FP32) (dt^2/2) |k|^2 from {hi, lo} tables: the FP64
+// sums took 0.9 ms at 2048^2 x 8, this pass 0.1 ms more than a plain transform.
 template <class Rl> struct SgStartCol {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
     static constexpr int PMAX = 32;
     static constexpr bool EARLY_NEXT = true;
     V2<Rl> *data;
-    const V2<Rl> *u;
-    const V2<Rl> *cx, *cy;  // {hi, lo} of (dt^2/2) k^2 per axis
+    const V2<Rl> *u, *v;
+    const V2<Rl> *cx, *cy;    // FP32: {hi, lo} of (dt^2/2) k^2 per axis
+    const double *kx2, *ky2;  // FP64: k^2 per axis
+    StartArgs<Rl> g;
     int64_t nx;
     __device__ const V2<Rl> *in(int) const { return data; }
     template <int N, int P, int BLOCK, class Sm, class H = NoHook>
@@ -80,22 +106,35 @@ template <class Rl> struct SgStartCol {
                                         const TW<Rl> *tw, const H &hook = H{}) const
     {
         constexpr int T = N / P;
-        V2<Rl>(&v)[P] = vv[0];
+        V2<Rl>(&a)[P] = vv[0];
         const int64_t base = field * N * nx + x;
-        block_fft<N, P, -1, BLOCK>(v, sm[0], t, tw, hook);
-        const V2<Rl> kx = __ldg(cx + x);
+        block_fft<N, P, -1, BLOCK>(a, sm[0], t, tw, hook);
 #pragma unroll
         for (int m = 0; m < P; ++m) {
             const int y = t + T * m;
-            const V2<Rl> ky = __ldg(cy + y), un = u[base + int64_t(y) * nx];
-            // kx + ky as a sum and its rounding error (Knuth's two-sum) plus the low parts
-            const Rl c = kx.x + ky.x, bp = c - kx.x, lo = (kx.x - (c - bp)) + (ky.x - bp) + (kx.y + ky.y);
-            v[m] = V2<Rl>{fma_(c, un.x, fma_(lo, un.x, v[m].x)), fma_(c, un.y, fma_(lo, un.y, v[m].y))};
+            const int64_t o = base + int64_t(y) * nx;
+            const V2<Rl> un = u[o], vn = v ? v[o] : V2<Rl>{Rl(0), Rl(0)};
+            if constexpr (sizeof(Rl) == 4) {
+                // the tables' sum as a pair
+                const float2 kx = __ldg(cx + x), ky = __ldg(cy + y);
+                const float c = __fadd_rn(kx.x, ky.x), b = __fsub_rn(c, kx.x);
+                const float cl = __fadd_rn(__fadd_rn(__fsub_rn(kx.x, __fsub_rn(c, b)), __fsub_rn(ky.x, b)),
+                                           __fadd_rn(kx.y, ky.y));
+                auto sum = [&](float s, float uk, float vk) {
+                    PairSum r{0.0f, 0.0f};
+                    r.add(c, cl, uk);
+                    r.add(g.h, g.h_lo, s);
+                    r.add(g.dt, g.dt_lo, vk);
+                    return r.value();
+                };
+                a[m] = V2<Rl>{sum(a[m].x, un.x, vn.x), sum(a[m].y, un.y, vn.y)};
+            } else {
+                const double k2 = __ldg(kx2 + x) + __ldg(ky2 + y);
+                a[m] = V2<Rl>{g.dt64 * vn.x + g.h64 * (k2 * un.x + a[m].x), g.dt64 * vn.y + g.h64 * (k2 * un.y + a[m].y)};
+            }
         }
-        store_line<P, T>(v, data + base, nx, t, true);
+        store_line<P, T>(a, data + base, nx, t, true);
     }
-    static __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-    static __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 };
 
 // real rows, complex forward row transform, columns 0 .. N/2 (half spectra:
@@ -207,19 +246,31 @@ template <class Rl> struct ColToReal {
     }
 };
 
-// Constants of the start-up: dt and dt^2/2 (FP32: and the rests of their rounding)
-template <class Rl> struct StartArgs {
-    Rl dt, dt_lo, dt2_2, dt2_2_lo;
-};
-
-// dt v + (dt^2/2) sin u (v may be null); the rests of the constants enter inside
-// the fused multiply-adds, so that their rounding does not scale the whole field
-template <class Rl> __global__ void k_sg_start(const Rl *u, const Rl *v, Rl *dst, StartArgs<Rl> g, int64_t n)
+// sin x rounded to the grid's precision from a value good to 2^-45.  FP32 on
+// |x| <= 0.785: x - x^3/6 as pairs of floats (the second term's error is the
+// largest), the rest of its Taylor series (up to x^13; the next term is below
+// 2^-39) in float; beyond, the sine in double.
+__device__ __forceinline__ float sin_rounded(float x)
 {
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-        const Rl s = sg_sin(u[i]), w = v ? v[i] : Rl(0);
-        dst[i] = g.dt * w + (g.dt2_2 * s + (g.dt_lo * w + g.dt2_2_lo * s));
-    }
+    if (!(fabsf(x) <= 0.785f)) return float(sin(double(x)));
+    constexpr float S = float(-1.0 / 6), SL = float(-1.0 / 6 - double(S));
+    const float t = __fmul_rn(x, x), tl = __fmaf_rn(x, x, -t);
+    const float c = __fmul_rn(x, t), cl = __fmaf_rn(x, tl, __fmaf_rn(x, t, -c));  // x^3
+    const float v = __fmul_rn(c, S), vl = __fmaf_rn(cl, S, __fmaf_rn(c, SL, __fmaf_rn(c, S, -v)));
+    float w = __fmaf_rn(t, float(1.0 / 6227020800.0), float(-1.0 / 39916800.0));
+    w = __fmaf_rn(t, w, float(1.0 / 362880.0));
+    w = __fmaf_rn(t, w, float(-1.0 / 5040.0));
+    w = __fmaf_rn(t, w, float(1.0 / 120.0));
+    w = __fmul_rn(__fmul_rn(c, t), w);
+    const float d = __fadd_rn(x, v), e = __fsub_rn(v, __fsub_rn(d, x));  // |v| < |x|: exact
+    return __fadd_rn(d, __fadd_rn(e, __fadd_rn(vl, w)));
+}
+__device__ __forceinline__ double sin_rounded(double x) { return sin(x); }
+
+template <class Rl> __global__ void k_sg_sine(const Rl *u, Rl *dst, int64_t n)
+{
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+        dst[i] = sin_rounded(u[i]);
 }
 
 }  // namespace
@@ -231,10 +282,13 @@ cudaError_t sg_level_cols(const V2<Rl> *a, V2<Rl> *out, Rl scale, int64_t nx, in
     return launch_col<Rl>(ny, nx, SgLevelCol<Rl>{a, out, scale, nx}, twy, batch, s);
 }
 template <class Rl>
-cudaError_t sg_start_cols(V2<Rl> *data, const V2<Rl> *u, const V2<Rl> *cx, const V2<Rl> *cy, int64_t nx, int64_t ny,
-                          int64_t batch, const TW<Rl> *twy, cudaStream_t s)
+cudaError_t sg_start_cols(V2<Rl> *data, const V2<Rl> *u, const V2<Rl> *v, double dt, const V2<Rl> *cx, const V2<Rl> *cy,
+                          const double *kx2, const double *ky2, int64_t nx, int64_t ny, int64_t batch,
+                          const TW<Rl> *twy, cudaStream_t s)
 {
-    return launch_col<Rl>(ny, nx, SgStartCol<Rl>{data, u, cx, cy, nx}, twy, batch, s);
+    const double h = 0.5 * dt * dt;
+    const StartArgs<Rl> g{Rl(dt), Rl(dt - double(Rl(dt))), Rl(h), Rl(h - double(Rl(h))), dt, h};
+    return launch_col<Rl>(ny, nx, SgStartCol<Rl>{data, u, v, cx, cy, kx2, ky2, g, nx}, twy, batch, s);
 }
 template <class Rl>
 cudaError_t rows_from_real(const Rl *src, V2<Rl> *dst, int64_t nx, int64_t sx, int64_t ny, int64_t batch,
@@ -257,28 +311,26 @@ cudaError_t cols_to_real(const V2<Rl> *src, Rl *dst, Rl scale, int64_t nx, int64
 {
     return launch_col<Rl>(ny, nx, ColToReal<Rl>{src, dst, scale, nx}, twy, batch, s);
 }
-template <class Rl>
-cudaError_t sg_start_field(const Rl *u, const Rl *v, Rl *dst, double dt, int64_t n, cudaStream_t s)
+template <class Rl> cudaError_t sg_sine(const Rl *u, Rl *dst, int64_t n, cudaStream_t s)
 {
-    const double d2 = 0.5 * dt * dt;
-    const StartArgs<Rl> g{Rl(dt), Rl(dt - double(Rl(dt))), Rl(d2), Rl(d2 - double(Rl(d2)))};
     const unsigned blocks = unsigned(std::min<int64_t>((n + 255) / 256, 4096));
-    k_sg_start<Rl><<<blocks, 256, 0, s>>>(u, v, dst, g, n);
+    k_sg_sine<Rl><<<blocks, 256, 0, s>>>(u, dst, n);
     return cudaGetLastError();
 }
 
 #define PSS_INST(Rl)                                                                                             \
     template cudaError_t sg_level_cols<Rl>(const V2<Rl> *, V2<Rl> *, Rl, int64_t, int64_t, int64_t,              \
                                            const TW<Rl> *, cudaStream_t);                                        \
-    template cudaError_t sg_start_cols<Rl>(V2<Rl> *, const V2<Rl> *, const V2<Rl> *, const V2<Rl> *, int64_t,    \
-                                           int64_t, int64_t, const TW<Rl> *, cudaStream_t);                      \
+    template cudaError_t sg_start_cols<Rl>(V2<Rl> *, const V2<Rl> *, const V2<Rl> *, double, const V2<Rl> *,     \
+                                           const V2<Rl> *, const double *, const double *, int64_t, int64_t,     \
+                                           int64_t, const TW<Rl> *, cudaStream_t);                               \
     template cudaError_t rows_from_real<Rl>(const Rl *, V2<Rl> *, int64_t, int64_t, int64_t, int64_t,            \
                                             const TW<Rl> *, cudaStream_t);                                       \
     template cudaError_t rows_inverse<Rl>(V2<Rl> *const[3], const int *, int64_t, const V2<Rl> *, V2<Rl> *,      \
                                           int64_t, int64_t, int64_t, int64_t, const TW<Rl> *, cudaStream_t);     \
     template cudaError_t cols_to_real<Rl>(const V2<Rl> *, Rl *, Rl, int64_t, int64_t, int64_t, const TW<Rl> *,   \
                                           cudaStream_t);                                                         \
-    template cudaError_t sg_start_field<Rl>(const Rl *, const Rl *, Rl *, double, int64_t, cudaStream_t);
+    template cudaError_t sg_sine<Rl>(const Rl *, Rl *, int64_t, cudaStream_t);
 PSS_INST(float)
 PSS_INST(double)
 
