@@ -36,6 +36,7 @@ constexpr float sg_sin_small = 0.785f;
 // spectra row pass 135 -> 117 us)
 template <int P> __device__ __forceinline__ bool sg_all_small(const float2 (&v)[P], bool both)
 {
+    if constexpr (PSS_SG_LIBM_SIN) return false;  // that build's sine for every value
     float big = 0.0f;
 #pragma unroll
     for (int m = 0; m < P; ++m) big = fmaxf(big, both ? fmaxf(fabsf(v[m].x), fabsf(v[m].y)) : fabsf(v[m].x));
