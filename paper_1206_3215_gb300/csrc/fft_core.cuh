@@ -92,11 +92,19 @@ template <int DIR> __device__ __forceinline__ double2 twmul(double2 z, double2 w
     return DIR < 0 ? cmul(z, w) : cmulc(z, w);
 }
 
+// the same with the rest of w's rounding (ExactTw)
+template <int DIR> __device__ __forceinline__ double2 twmul(double2 z, double2 w, double2 wl)
+{
+    if (DIR > 0) w.y = -w.y, wl.y = -wl.y;
+    const double cr = fma(z.x, wl.x, -(z.y * wl.y)), ci = fma(z.x, wl.y, z.y * wl.x);
+    return {fma(z.x, w.x, fma(-z.y, w.y, cr)), fma(z.x, w.y, fma(z.y, w.x, ci))};
+}
+
 // s * x with s = hi + lo held exactly to one rounding
 __device__ __forceinline__ float mul_hl(float x, float h, float l) { return __fmaf_rn(x, h, x * l); }
 
-// z * exp(DIR * 2 pi i k / RAD), 0 <= k < RAD, RAD | 32
-template <int RAD, int DIR, int K, class V> __device__ __forceinline__ V rot(V z)
+// z * exp(DIR * 2 pi i k / RAD), 0 <= k < RAD, RAD | 32 (DOWN: see fft_stage)
+template <int RAD, int DIR, int K, bool DOWN = false, class V> __device__ __forceinline__ V rot(V z)
 {
     using R = decltype(z.x);
     constexpr int m = K * (32 / RAD);
@@ -123,7 +131,9 @@ template <int RAD, int DIR, int K, class V> __device__ __forceinline__ V rot(V z
             const float2 d{dr, di};
             return __ffma2_rn(d, float2{hh, hh}, __fmul2_rn(d, float2{hl, hl}));
         } else {
-            return {R(H) * dr, R(H) * di};
+            // the nearest double lies 6.8e-17 above H, the one below it 8.9e-17 below
+            constexpr R h = DOWN ? R(0.70710678118654746) : R(H);
+            return {h * dr, h * di};
         }
     } else {
         constexpr double c = cos32(m), s = DIR > 0 ? sin32(m) : -sin32(m);
@@ -145,7 +155,7 @@ template <int RAD, int DIR, int K, class V> __device__ __forceinline__ V rot(V z
 // of (a - c - DIR i (b - d)) w^{3k}.  Against plain radix-2 steps this needs
 // fewer non-trivial rotations (16 instead of 20 general ones and 10 instead
 // of 14 by odd multiples of pi/4 for 32 points), with the same additions.
-template <int RAD, int DIR, int S, int K, class V> __device__ __forceinline__ void sr_level(V *v)
+template <int RAD, int DIR, int S, int K, bool DOWN, class V> __device__ __forceinline__ void sr_level(V *v)
 {
     if constexpr (K < RAD / 4) {
         constexpr int Q = RAD / 4;
@@ -153,9 +163,9 @@ template <int RAD, int DIR, int S, int K, class V> __device__ __forceinline__ vo
         v[K * S] = cadd(a, c);
         v[(K + Q) * S] = cadd(b, d);
         const V t1 = csub(a, c), jt2 = mul_i<DIR>(csub(b, d));
-        v[(K + 2 * Q) * S] = rot<RAD, DIR, K>(cadd(t1, jt2));
-        v[(K + 3 * Q) * S] = rot<RAD, DIR, 3 * K>(csub(t1, jt2));
-        sr_level<RAD, DIR, S, K + 1>(v);
+        v[(K + 2 * Q) * S] = rot<RAD, DIR, K, DOWN>(cadd(t1, jt2));
+        v[(K + 3 * Q) * S] = rot<RAD, DIR, 3 * K, DOWN>(csub(t1, jt2));
+        sr_level<RAD, DIR, S, K + 1, DOWN>(v);
     }
 }
 
@@ -163,17 +173,17 @@ template <int RAD, int DIR, int S, int K, class V> __device__ __forceinline__ vo
 // decimation in frequency; the result is left in bit-reversed order (output
 // r at position bitrev(r)): the even outputs fill the first half, outputs
 // 4j + 1 the third quarter and 4j + 3 the last.
-template <int RAD, int DIR, int S, class V> __device__ __forceinline__ void dft_dif(V *v)
+template <int RAD, int DIR, int S, bool DOWN = false, class V> __device__ __forceinline__ void dft_dif(V *v)
 {
     if constexpr (RAD == 2) {
         const V a = v[0], b = v[S];
         v[0] = cadd(a, b);
         v[S] = csub(a, b);
     } else if constexpr (RAD >= 4) {
-        sr_level<RAD, DIR, S, 0>(v);
-        dft_dif<RAD / 2, DIR, S>(v);
-        dft_dif<RAD / 4, DIR, S>(v + (RAD / 2) * S);
-        dft_dif<RAD / 4, DIR, S>(v + (3 * RAD / 4) * S);
+        sr_level<RAD, DIR, S, 0, DOWN>(v);
+        dft_dif<RAD / 2, DIR, S, DOWN>(v);
+        dft_dif<RAD / 4, DIR, S, DOWN>(v + (RAD / 2) * S);
+        dft_dif<RAD / 4, DIR, S, DOWN>(v + (3 * RAD / 4) * S);
     }
 }
 
@@ -399,6 +409,16 @@ __device__ __forceinline__ void fact_stage(V *v, const W *__restrict__ tw, int t
     }
 }
 
+// FP64 transforms of more, shorter stages than the 16-point ones round more
+// often, and a twiddle's own rounding repeats in every step (it shrinks or grows
+// |z| by the same factor each time).  With two points per thread (lengths 32 and
+// 64 in small fields) and at length 16 the twiddles are therefore applied with
+// the rest of their rounding: 64^2 is 2.04e-16 off per transform (2.17e-16
+// without, 2.06e-16 in stages of 16 and 4) and 3.7e-15 after 200 NLS steps
+// (1.5e-14, 1.0e-14), for 13.9 instead of 12.2 us per step (57 in stages of 16
+// and 4).  Four points per thread are as accurate as 16 without.
+template <int N, int P> struct ExactTw : std::bool_constant<P == 2 || N == 16> {};
+
 // One Stockham stage s of a length-N transform (DIR = -1 forward, +1 inverse).
 // On entry register m holds element t + T m of the stage input; on exit (for
 // the last stage) register m holds output element t + T m.  Other stages leave
@@ -408,7 +428,7 @@ __device__ __forceinline__ void fft_stage(V (&v)[P], const Sm &sm, int t, const 
 {
     using PL = Plan<N, P>;
     constexpr int R = PL::radix(S), NS = PL::span(S), T = PL::T, Q = P / R;
-    constexpr bool LAST = (S == PL::STAGES - 1);
+    constexpr bool LAST = (S == PL::STAGES - 1), FP64 = std::is_same<W, double2>::value;
     if constexpr (LAST) hook();
     if constexpr (S > 0) {
         // twiddles W_{NS R}^{(j mod NS) r} = W_N^{(j mod NS) r N/(NS R)}
@@ -434,11 +454,17 @@ __device__ __forceinline__ void fft_stage(V (&v)[P], const Sm &sm, int t, const 
                     if (r + TWD < R) ring[(r - 1) % TWD] = lds_f4(a0 + unsigned((r + TWD - 1) * NS) * 16u);
                     v[q + r * Q] = twmul<DIR>(v[q + r * Q], w);
                 }
+            } else if constexpr (!FACT && FP64 && NS * R == 4) {
+                if (jm) v[q + Q] = mul_i<DIR>(v[q + Q]);  // W_4^jm, jm = 0 or 1
             } else if constexpr (!FACT) {
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    const W w = __ldg(tw + jm * r * (N / (NS * R)));
-                    v[q + r * Q] = twmul<DIR>(v[q + r * Q], w);
+                    const int e = jm * r * (N / (NS * R));
+                    const W w = __ldg(tw + e);
+                    if constexpr (FP64 && ExactTw<N, P>::value)
+                        v[q + r * Q] = twmul<DIR>(v[q + r * Q], w, __ldg(tw + N + e));
+                    else
+                        v[q + r * Q] = twmul<DIR>(v[q + r * Q], w);
                 }
             }
         }
@@ -447,8 +473,14 @@ __device__ __forceinline__ void fft_stage(V (&v)[P], const Sm &sm, int t, const 
         // constant rotation per butterfly
         if constexpr (FACT) fact_stage<P, DIR, Q, R, 1>(v, tw, t);
     }
+    // FP64 with eight points per thread: 1/sqrt(2) rounded up and down in turn,
+    // by stage and direction, so that its rounding does not add up over the
+    // stages of a transform and over a transform and its inverse (512^2: 2.69e-16
+    // off per transform instead of 2.88e-16, 2.0e-15 after 20 NLS steps; in
+    // stages of 16, 16 and 2 2.76e-16 and 2.7e-15)
+    constexpr bool DOWN = FP64 && P == 8 && ((S & 1) != 0) != (DIR > 0);
 #pragma unroll
-    for (int q = 0; q < Q; ++q) dft_dif<R, DIR, Q>(v + q);
+    for (int q = 0; q < Q; ++q) dft_dif<R, DIR, Q, DOWN>(v + q);
     constexpr int BITS = ilog2(R);
     if constexpr (LAST) {
         // undo the bit reversal: output r of butterfly q sits in v[q + bitrev(r) Q]

@@ -22,7 +22,8 @@ void unit_pair_f32(double c, double s, float *fc, float *fs);
 void hilo_f32(double re, double im, float *out4);
 
 // Twiddle table W_n^e = exp(-2 pi i e / n), e = 0..n-1: FP32 as hi + lo
-// quadruples (4 floats per entry), FP64 as (re, im) pairs.
+// quadruples (4 floats per entry), FP64 as n (re, im) pairs, followed by
+// the n pairs of rests that their rounding leaves.
 std::vector<float> twiddles_f32(int64_t n);
 std::vector<double> twiddles_f64(int64_t n);
 
