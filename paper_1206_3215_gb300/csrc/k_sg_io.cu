@@ -15,13 +15,17 @@
 // accuracy: taking the real part at the end drops half of the rounding error
 // that a full complex transform has collected.  Read-back alone at 512^2, FP32
 // / FP64: as here 1.10e-7 / 2.2e-16, columns first 1.27e-7 / 2.7e-16,
-// half-length rows 1.38e-7 / 2.9e-16; 2048^2 x 8 FP32 takes 0.05 ms more per
-// level than with half the bytes.
+// half-length rows 1.38e-7 / 2.9e-16.  At 2048^2 x 8 in FP32 a level takes 0.35
+// ms, with half-length rows 0.19.
 //
-// 2048^2 x 8 on half spectra, against transforms of full complex arrays with
-// separate copies, conversions and FP64 elementwise kernels (sums of kernel
-// times): set-up 3.4 -> 0.5 ms, read-back of both levels 1.2 -> 0.3 ms,
-// Hamiltonian 3.6 -> 1.9 ms.
+// 2048^2 x 8 on half spectra in FP32, against transforms of full complex arrays
+// with separate copies, conversions and FP64 elementwise kernels: set-up
+// 3.54 -> 0.60 ms (with a velocity 3.64 -> 0.81), read-back of both levels
+// 0.99 -> 0.70 ms, Hamiltonian 3.64 -> 2.07 ms.
+//
+// (The state is set on half spectra.  A field set and read back before its first
+// step carries the forward transform's error unhalved, 1.65e-7 at 512^2 in FP32
+// where full spectra give 1.49e-7; after a step both layouts always did.)
 #include <algorithm>
 
 #include "launch.cuh"
@@ -30,8 +34,9 @@ namespace pss {
 
 namespace {
 
-// H of uhat: column inverse transform of a times scale, into out.  The arithmetic is that of the second half of the step's column
-// pass (SgCol), so H made here from uhat is the H the step left, bit for bit.
+// H of uhat: column inverse transform of a times scale, into out.  The arithmetic
+// is that of the second half of the step's column pass (SgCol), so H made here
+// from uhat is the H the step left, bit for bit.
 template <class Rl> struct SgLevelCol {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
@@ -87,8 +92,8 @@ template <class Rl> struct StartArgs {
 
 // the start-up's column pass: data = dt v + (dt^2/2) (|k|^2 u + column transform
 // of data), u and v (may be null) transformed already.  |k|^2 from the per-axis
-// tables in double, or (FP32) (dt^2/2) |k|^2 from {hi, lo} tables: the FP64
-// sums took 0.9 ms at 2048^2 x 8, this pass 0.1 ms more than a plain transform.
+// tables in double, or (FP32) (dt^2/2) |k|^2 from {hi, lo} tables: the sums in
+// FP64 took 0.9 ms at 2048^2 x 8, the whole set-up takes 0.6.
 template <class Rl> struct SgStartCol {
     static constexpr int NIN = 1;
     static constexpr bool LEAN = true;
@@ -109,11 +114,21 @@ template <class Rl> struct SgStartCol {
         V2<Rl>(&a)[P] = vv[0];
         const int64_t base = field * N * nx + x;
         block_fft<N, P, -1, BLOCK>(a, sm[0], t, tw, hook);
+        // u and v four points ahead (the compiler does not move loads over stores
+        // or hold them all)
+        constexpr int CH = P < 4 ? P : 4;
+        V2<Rl> ua[CH], va[CH];
 #pragma unroll
         for (int m = 0; m < P; ++m) {
             const int y = t + T * m;
-            const int64_t o = base + int64_t(y) * nx;
-            const V2<Rl> un = u[o], vn = v ? v[o] : V2<Rl>{Rl(0), Rl(0)};
+            if (m % CH == 0)
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    const int64_t o = base + int64_t(t + T * (m + c)) * nx;
+                    ua[c] = u[o];
+                    va[c] = v ? v[o] : V2<Rl>{Rl(0), Rl(0)};
+                }
+            const V2<Rl> un = ua[m % CH], vn = va[m % CH];
             if constexpr (sizeof(Rl) == 4) {
                 // the tables' sum as a pair
                 const float2 kx = __ldg(cx + x), ky = __ldg(cy + y);
@@ -269,8 +284,16 @@ __device__ __forceinline__ double sin_rounded(double x) { return sin(x); }
 
 template <class Rl> __global__ void k_sg_sine(const Rl *u, Rl *dst, int64_t n)
 {
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-        dst[i] = sin_rounded(u[i]);
+    const int64_t step = int64_t(gridDim.x) * blockDim.x;
+    int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    for (; i + 3 * step < n; i += 4 * step) {
+        Rl x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = u[i + k * step];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dst[i + k * step] = sin_rounded(x[k]);
+    }
+    for (; i < n; i += step) dst[i] = sin_rounded(u[i]);
 }
 
 }  // namespace
