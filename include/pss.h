@@ -119,8 +119,9 @@ int pss_create_grid(pss_grid **out, const pss_params *p);
  *       u^{-1} = u^0 - dt u_t(0) + dt^2/2 (Lap u^0 - sin u^0)   (Section 4.2 start-up).
  *  NS:  a = omega(0), real [batch][ny][nx]; masked by the 2/3 rule if dealias.
  * Element type follows the precision (float or double).  where = PSS_HOST or
- * PSS_DEVICE; device buffers must be on the grid's device.  Synchronises the
- * grid's stream before returning when where = PSS_HOST. */
+ * PSS_DEVICE; device buffers must be on the grid's device and hold the whole
+ * state (PSS_E_CUDA where the allocation ends before it does).  Synchronises
+ * the grid's stream before returning when where = PSS_HOST. */
 int pss_set_state(pss_grid *g, const void *a, const void *b, int where);
 
 /* Advance every field of the batch by n >= 0 time steps, enqueued on the grid
@@ -194,7 +195,9 @@ int pss_stats(pss_grid *g, int64_t *steps, int64_t *ns_updates);
 
 /* Checkpoint of the exact internal state (bitwise resume).
  * pss_checkpoint_size gives the byte count; save/load copy to or from a
- * caller buffer at `where`.  Loading restores the step counter too. */
+ * caller buffer at `where`.  Loading restores the step counter too.  A
+ * dealiased NS grid keeps modes above the 2/3 cut that the checkpoint of a grid
+ * without dealiasing holds: they enter the Jacobian. */
 int pss_checkpoint_size(const pss_grid *g, size_t *bytes);
 int pss_checkpoint_save(pss_grid *g, void *buf, int where);
 int pss_checkpoint_load(pss_grid *g, const void *buf, int where);

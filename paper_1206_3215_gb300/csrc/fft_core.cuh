@@ -246,13 +246,14 @@ __device__ __forceinline__ void prefetch_l2(const void *p)
 // CTA waits, also one without work, so that a kernel never completes before
 // its predecessors; the trigger comes after the wait, so that only the next
 // kernel's CTAs sit waiting, not those of the whole chain.  Only grids of one
-// wave, with at most one CTA per SM of at most half an SM's shared memory,
-// give it: beside fuller grids the early CTAs pile up on the SMs that have
-// room first and the next kernel runs unevenly spread (a trigger in every
-// kernel: NLS 4096^2 x 2 447 -> 474 us per step, SG 512^2 x 8 27 -> 31;
-// without the limit on shared memory NLS 1024^2 19.0 -> 21.2).  Per step, plain
-// launches -> these: NLS 64^2 10.9 -> 8.2 us, 256^2 12.1 -> 9.0, 512^2 15.3 -> 12.7,
-// SG 512^2 x 2 26.6 -> 22.1; where no kernel gives the trigger, 0 - 3 %.
+// wave, with at most one CTA per SM and at most half an SM's shared memory
+// taken at launch (the static twiddle copy, up to 16 KB, comes on top), give it:
+// beside fuller grids the early CTAs pile up on the SMs that have room first
+// and the next kernel runs unevenly spread (a trigger in every kernel: NLS
+// 4096^2 x 2 447 -> 474 us per step, SG 512^2 x 8 27 -> 31; without the limit on
+// shared memory NLS 1024^2 19.0 -> 21.2).  Per step, plain launches -> these:
+// NLS 64^2 9.2 -> 7.9 us, 256^2 11.3 -> 9.0, 512^2 14.4 -> 12.8, 1024^2
+// 19.0 -> 17.4, SG 512^2 x 2 24.1 -> 21.9; where no kernel gives the trigger, 0 - 3 %.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 constexpr unsigned GRID_SMS = 152, GRID_EARLY_SMEM = 114 * 1024;
 __device__ __forceinline__ void grid_trigger(int64_t tiles)

@@ -124,12 +124,17 @@ template <class Rl> struct Shape {
     // stages; larger fields of short lines keep more points (fft
     // 64 x 4096 x 8, 4 / 2 points: 274 / 300 us).  The choice depends on the
     // grid alone, not on the batch, so that a batch rounds as its fields do
-    // alone.  Per step, from 16 points to these: NLS 64^2 57.5 -> 13.3 us,
-    // 256^2 72 -> 26, SG 256^2 x 2 on half spectra 152 -> 31, NS 256^2
-    // 243 -> 102; at 512 radix 8 three times instead of 16, 16, 2: one field
-    // 144 -> 99 us, four the same.  FP32 lines keep RP points: another
-    // factorisation rounds differently, which moves the conserved quantities
-    // of a small field by up to 1e-7.
+    // alone.  Per step, from 16 points (and larger tiles) to these: NLS 64^2
+    // 57.5 -> 13.9 us, 128^2 64.6 -> 19.8, 256^2 71.7 -> 38.5, 512^2 135 -> 84, x 8
+    // 644 -> 561; SG 256^2 x 8 on half spectra 157 -> 97; NS 256^2 243 -> 90.  What
+    // it costs: batches that fill the FP64 lanes pay for the extra stages where
+    // they gain nothing from the spread.  NLS 128^2 x 32 133 -> 138 us per step,
+    // transforms of 256^2 x 32 206 -> 213 us, of 128 x 8192 156 -> 158; 256^2 x 32
+    // NLS (533 -> 524) and 128^2 x 32 transforms (54.9 -> 54.2) are even.  Eight
+    // points instead of four bring those to 127 and 203, but one field of 128^2 to
+    // 33 us and NS 256^2 to 133.  FP32 lines keep RP points in the transforms
+    // (the short NS row pass has 16): another factorisation rounds differently,
+    // which moves the conserved quantities of a small field by up to 1e-7.
     static constexpr int SHORT = sizeof(Rl) == 4 ? 0 : 512;
     __host__ __device__ static constexpr int shortP(int n, bool small)
     {
